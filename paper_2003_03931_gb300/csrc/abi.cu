@@ -127,7 +127,7 @@ static size_t layout_lowmem(Sim& s, uint8_t* base) {
     // small persistent items
     const size_t h = s.nc / 2 + 1;
     s.green_coarse = reinterpret_cast<float4*>(take(16 * h * h * h));
-    s.green_fine = reinterpret_cast<float*>(take(4 * (size_t)kGreenS * kGreenS * kGreenS));
+    s.green_col = reinterpret_cast<float*>(take(4 * (size_t)kGreenS * kGreenS * kGreenS));
     s.green_packed = reinterpret_cast<float*>(take(4 * (size_t)kGreenS * kGreenS * (kGreenS + 1) / 2));
     s.Tdec = reinterpret_cast<float*>(take(4 * 256));
     s.Eedge = reinterpret_cast<float*>(take(4 * 256));
@@ -210,7 +210,7 @@ size_t layout(Sim& s, uint8_t* base) {
     s.Fl = reinterpret_cast<float*>(take(12 * (size_t)C));
     const size_t h = s.nc / 2 + 1;
     s.green_coarse = reinterpret_cast<float4*>(take(16 * h * h * h));
-    s.green_fine = reinterpret_cast<float*>(take(4 * (size_t)kGreenS * kGreenS * kGreenS));
+    s.green_col = reinterpret_cast<float*>(take(4 * (size_t)kGreenS * kGreenS * kGreenS));
     s.green_packed = reinterpret_cast<float*>(take(4 * (size_t)kGreenS * kGreenS * (kGreenS + 1) / 2));
     s.Tdec = reinterpret_cast<float*>(take(4 * 256));
     s.Eedge = reinterpret_cast<float*>(take(4 * 256));
@@ -488,7 +488,7 @@ static int init_finish(pmpm_sim* h, pmpm_sim** out) {
 
 
 GreenRefs sim_tables(const Sim& s) {
-    return GreenRefs{s.green_coarse, s.green_fine, s.green_packed};
+    return GreenRefs{s.green_coarse, s.green_col, s.green_packed};
 }
 
 size_t green_table_bytes(int nc, size_t part[3]) {

@@ -197,9 +197,12 @@ PMPM_HD void add_square_over_n128(long long S, int n, unsigned long long& lo,
 }
 
 // round-half-even(p 2^24) for a float32 p with |p| < 2^20, in integers (the
-// fixed-point momentum of the cell sums): p = m 2^(E - 150) exactly, so
-// p 2^24 = m 2^(E - 126) with m < 2^24; no FP64 (slow on this part).
+// fixed-point momentum of the cell sums).  The host form works it out in
+// integers: p = m 2^(E - 150) exactly, so p 2^24 = m 2^(E - 126), m < 2^24.
 PMPM_HD long long fix24_rn(float p) {
+#ifdef __CUDA_ARCH__
+    return __float2ll_rn(p * 16777216.f);   // the product is exact
+#else
     union { float f; uint32_t u; } bits;
     bits.f = p;
     const uint32_t E = (bits.u >> 23) & 255u, M = bits.u & 0x7fffffu;
@@ -216,6 +219,7 @@ PMPM_HD long long fix24_rn(float p) {
         r = (long long)(q + ((rem > half || (rem == half && (q & 1u))) ? 1u : 0u));
     }
     return (bits.u >> 31) ? -r : r;
+#endif
 }
 
 // ---------------------------------------------------------------- position format

@@ -14,7 +14,8 @@
 //  * Matching A(d): coarse-mesh force between fine-cell centres a fine
 //    separation d apart, averaged over the 64 centres of a coarse cell.
 //  * Short-range kernel K_s(d) = K_per(d) - A(d) for 0 < |d| < 6, and its
-//    32^3 DFT stored the same way in a 17^3 table.
+//    32^3 DFT stored the same way (for the FP16 tiles), and its 32^2 DFT over x
+//    and y for every dz (for the column pass).
 #include "pmpm_impl.cuh"
 
 namespace pmpm {
@@ -184,16 +185,18 @@ __global__ void k_fine_values(double L, const double* Tsmall, double* Ks) {
 }
 
 // S_s(a, b, c) = sum_d K_s^x(d) sin(2 pi a dx/32) cos(2 pi b dy/32) cos(2 pi c dz/32),
-// times 2^-21 (density units) and 2^-15 (unnormalised inverse 32^3 DFT)
-// one warp per entry, the lanes splitting the 1331 separations
-__global__ void k_fine_table(const double* Ks, float* table) {
+// times 2^-21 (density units) and 2^-15 (unnormalised inverse 32^3 DFT): the
+// b <= c half for own-axis rows a = 1..15 (rows 0 and 16 vanish: odd in its own
+// axis), row-major over (a - 1, b, c = b..16).
+// One warp per entry, the lanes splitting the 1331 separations.
+__global__ void k_fine_table(const double* Ks, float* packed) {
     const int i = (blockIdx.x * blockDim.x + threadIdx.x) >> 5, lane = threadIdx.x & 31;
-    if (i >= kGreenS * kGreenS * kGreenS) return;
-    const int a = i / (kGreenS * kGreenS), b = (i / kGreenS) % kGreenS, c = i % kGreenS;
-    if (a == 0 || a == 16) {
-        if (lane == 0) table[i] = 0.f;   // odd in its own axis: zero at k = 0 and at Nyquist
-        return;
-    }
+    const int tri = kGreenS * (kGreenS + 1) / 2;
+    if (i >= (kGreenS - 2) * tri) return;
+    const int a = 1 + i / tri;
+    int r = i % tri, b = 0;
+    while (r >= kGreenS - b) { r -= kGreenS - b; ++b; }
+    const int c = b + r;
     double acc = 0.0;
     for (int j = lane; j < 1331; j += 32) {
         const double k = Ks[j];
@@ -204,19 +207,36 @@ __global__ void k_fine_table(const double* Ks, float* table) {
     }
 #pragma unroll
     for (int o = 16; o > 0; o >>= 1) acc += __shfl_xor_sync(0xffffffffu, acc, o);
-    if (lane == 0) table[i] = (float)(acc * 0x1p-36);
+    if (lane == 0) packed[i] = (float)(acc * 0x1p-36);
 }
 
-// b <= c half of the 17^3 table for own-axis rows a = 1..15 (rows 0 and 16
-// vanish), row-major over (a - 1, b, c = b..16)
-__global__ void k_pack_fine(const float* table, float* packed) {
-    const int i = blockIdx.x * blockDim.x + threadIdx.x;
-    const int tri = kGreenS * (kGreenS + 1) / 2;
-    if (i >= (kGreenS - 2) * tri) return;
-    const int a = 1 + i / tri;
-    int r = i % tri, b = 0;
-    while (r >= kGreenS - b) { r -= kGreenS - b; ++b; }
-    packed[i] = table[(a * kGreenS + b) * kGreenS + (b + r)];
+// The kernel transformed along x and y only, for the column pass: entry
+// [t][a][b] at |kx| = a, |ky| = b,
+//   t = d      (d = 0..5): sum K_s^x(dx, dy, d) sin(2 pi a dx/32) cos(2 pi b dy/32)
+//   t = 6 + d  (d = 0..5): the same with x and y exchanged (the y component)
+//   t = 11 + d (d = 1..5): sum K_s^z(dx, dy, d) cos(2 pi a dx/32) cos(2 pi b dy/32)
+// times 2^-21 (density units) and 2^-10 (unnormalised inverse 32^2 DFT); K_s^z
+// (dx, dy, d) = K_s^x(d, dy, dx).  One warp per entry.
+__global__ void k_column_table(const double* Ks, float* table) {
+    const int i = (blockIdx.x * blockDim.x + threadIdx.x) >> 5, lane = threadIdx.x & 31;
+    if (i >= kGreenS * kGreenS * kGreenS) return;
+    const int t = i / (kGreenS * kGreenS);
+    int a = (i / kGreenS) % kGreenS, b = i % kGreenS;
+    if (t >= 6 && t < 12) { const int s = a; a = b; b = s; }
+    const int d = t < 12 ? t % 6 : t - 11;
+    double acc = 0.0;
+    for (int j = lane; j < 121; j += 32) {
+        const int dx = j % 11 - 5, dy = j / 11 - 5;
+        const double k = t < 12 ? Ks[(dx + 5) + 11 * ((dy + 5) + 11 * (d + 5))]
+                                : Ks[(d + 5) + 11 * ((dy + 5) + 11 * (dx + 5))];
+        const double fx = t < 12 ? sinpi((double)(2 * a * dx) / 32.0) : cospi((double)(2 * a * dx) / 32.0);
+        acc += k * fx * cospi((double)(2 * b * dy) / 32.0);
+    }
+#pragma unroll
+    for (int o = 16; o > 0; o >>= 1) acc += __shfl_xor_sync(0xffffffffu, acc, o);
+    // odd in its own axis: zero at k = 0 and at Nyquist
+    if (t < 12 && (a == 0 || a == kGreenS - 1)) acc = 0.0;
+    if (lane == 0) table[i] = (float)(acc * 0x1p-31);
 }
 
 // real-space part of the coarse kernel (x component) on the whole mesh,
@@ -289,9 +309,8 @@ int build_green_tables(Sim& s) {
     float* T1 = reinterpret_cast<float*>(mesh + (size_t)nc * nc * nc);
     k_coarse_small<<<(343 * 32 + 255) / 256, 256, 0, st>>>(L, Tsmall);
     k_fine_values<<<(1331 * 32 + 255) / 256, 256, 0, st>>>(L, Tsmall, Ks);
-    k_fine_table<<<(kGreenS * kGreenS * kGreenS * 32 + 255) / 256, 256, 0, st>>>(Ks, s.green_fine);
-    k_pack_fine<<<((kGreenS - 2) * kGreenS * (kGreenS + 1) / 2 + 255) / 256, 256, 0, st>>>(s.green_fine,
-                                                                                   s.green_packed);
+    k_fine_table<<<((kGreenS - 2) * kGreenS * (kGreenS + 1) / 2 * 32 + 255) / 256, 256, 0, st>>>(Ks, s.green_packed);
+    k_column_table<<<(kGreenS * kGreenS * kGreenS * 32 + 255) / 256, 256, 0, st>>>(Ks, s.green_col);
     const Ewald e = make_ewald(L, nc / 2 - 1);
     k_coarse_real<<<grid_for(s.ncells, 256), 256, 0, st>>>(nc, e, mesh);
     int rc = fft3d<double>(s, mesh, nc, -1);

@@ -49,8 +49,8 @@ struct Sim {
     float2* cB2 = nullptr;
     float* Fl = nullptr;                        // [3][nc^3]
     float4* green_coarse = nullptr;             // [(nc/2+1)^3] (S_x, S_y, S_z, 0), |kx| fastest
-    float* green_fine = nullptr;                // [17^3]
-    float* green_packed = nullptr;              // [17 x 153] b <= c half of green_fine
+    float* green_col = nullptr;                 // [17][17][17] column pass: taps x |kx| x |ky|
+    float* green_packed = nullptr;              // [15 x 153] 32^3 DFT (FP16 tiles)
     float* Tdec = nullptr;                      // [256]
     float* Eedge = nullptr;                     // [256]
     float2* tw_f = nullptr;                     // [fft_max] exp(-2 pi i k / fft_max)
@@ -153,7 +153,8 @@ inline size_t store_bytes(const Sim& s) { return (size_t)(3 * s.pb + 3) * s.n; }
 namespace pmpm {
 
 // Device pointers of the three force tables (Sec. II): the coarse-kernel
-// spectrum, the fine kernel K_s spectrum and its packed tile copy.
+// spectrum, the fine kernel K_s transformed along x and y (column pass) and its
+// packed 32^3 spectrum (FP16 tiles).
 struct GreenRefs {
     const float4* coarse;
     const float* fine;

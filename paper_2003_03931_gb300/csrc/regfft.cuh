@@ -69,12 +69,22 @@ PMPM_HD float2 twiddle_f(float2 d, int j, float& m) {
     return make_float2(t * d.x - d.y, t * d.y + d.x);
 }
 
-// (a, b) <- (a + w b, a - w b)
+// (a, b) <- (a + w b, a - w b).  On the device both outputs are packed
+// float2 operations (one instruction for the two components, each rounded
+// as the scalar one) except for the quarter-turn twiddles, whose swapped
+// components would have to be moved first.
 template <int S>
 PMPM_HD void butterfly(float2& a, float2& b, int j) {
     float m;
     const float2 u = twiddle_f<S>(b, j, m);
     const float2 x = a;
+#ifdef __CUDA_ARCH__
+    if ((j & 15) != 8) {
+        a = m == 1.f ? __fadd2_rn(x, u) : __ffma2_rn(make_float2(m, m), u, x);
+        b = __ffma2_rn(make_float2(-m, -m), u, x);
+        return;
+    }
+#endif
     a = make_float2(x.x + m * u.x, x.y + m * u.y);
     b = make_float2(x.x - m * u.x, x.y - m * u.y);
 }
@@ -120,16 +130,20 @@ PMPM_HD void rfft32x2(const float (&x)[32], float2 (&X)[17]) {
 #pragma unroll
     for (int m = 0; m < 16; ++m) z[bitrev<4>(m)] = make_float2(x[2 * m], x[2 * m + 1]);
     fft_dit<16, -1>(z);
+    X[0] = make_float2(2.f * (z[0].x + z[0].y), 0.f);
+    X[16] = make_float2(2.f * (z[0].x - z[0].y), 0.f);
+    X[8] = make_float2(2.f * z[8].x, -2.f * z[8].y);
 #pragma unroll
-    for (int k = 0; k <= 16; ++k) {
-        const float2 Zk = z[k & 15];
-        const float2 Zr = z[(16 - k) & 15];
-        // 2E = Zk + conj Zr, 2O = -i (Zk - conj Zr); 2X = 2E + w^k 2O
+    for (int k = 1; k < 8; ++k) {
+        const float2 Zk = z[k], Zr = z[16 - k];
+        // 2E = Zk + conj Zr, 2O = -i (Zk - conj Zr); 2X[k] = 2E + w^k 2O and, as
+        // E and O at 16 - k are the conjugates, 2X[16 - k] = conj(2E - w^k 2O)
         const float2 E = make_float2(Zk.x + Zr.x, Zk.y - Zr.y);
         const float2 O = make_float2(Zk.y + Zr.y, Zr.x - Zk.x);
         float m;
         const float2 u = twiddle_f<-1>(O, k, m);
         X[k] = make_float2(E.x + m * u.x, E.y + m * u.y);
+        X[16 - k] = make_float2(E.x - m * u.x, m * u.y - E.y);
     }
 }
 
@@ -137,14 +151,19 @@ PMPM_HD void rfft32x2(const float (&x)[32], float2 (&X)[17]) {
 // over the Hermitian-extended spectrum.  In: X[0..16]; out: x[0..31].
 PMPM_HD void irfft32(const float2 (&X)[17], float (&x)[32]) {
     float2 z[16];
+    // z[k] = E + i O with E = X[k] + conj X[16 - k], O = w^k (X[k] - conj X[16 - k]); E
+    // and O at 16 - k are the conjugates.  X[0] and X[16] are real.
+    z[bitrev<4>(0)] = make_float2(X[0].x + X[16].x, X[0].x - X[16].x);
+    z[bitrev<4>(8)] = make_float2(2.f * X[8].x, -2.f * X[8].y);
 #pragma unroll
-    for (int k = 0; k < 16; ++k) {
+    for (int k = 1; k < 8; ++k) {
         const float2 Xk = X[k];
         const float2 Xc = make_float2(X[16 - k].x, -X[16 - k].y);   // conj X[16-k]
         const float2 E = cadd(Xk, Xc);
         float m;
         const float2 u = twiddle_f<1>(csub(Xk, Xc), k, m);         // O = m u
-        z[bitrev<4>(k)] = make_float2(E.x - m * u.y, E.y + m * u.x); // E + i O
+        z[bitrev<4>(k)] = make_float2(E.x - m * u.y, E.y + m * u.x);
+        z[bitrev<4>(16 - k)] = make_float2(E.x + m * u.y, m * u.x - E.y);
     }
     fft_dit<16, 1>(z);
 #pragma unroll

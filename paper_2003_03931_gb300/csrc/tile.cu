@@ -8,20 +8,8 @@
 
 namespace pmpm {
 
-// Optional per-phase clock stamps of thread 0 (compiled only with
-// -DPMPM_PHASE_CLOCKS; read back through pmpm_debug_phases).
-#ifdef PMPM_PHASE_CLOCKS
-constexpr int kMarks = 24;
-__device__ unsigned long long g_phase[4096 * kMarks];
-#define PMPM_MARK(k)                                                                    \
-    do {                                                                                \
-        if (threadIdx.x == 0 && blockIdx.x < 4096) g_phase[blockIdx.x * kMarks + (k)] = clock64(); \
-    } while (0)
-#else
-#define PMPM_MARK(k) \
-    do {             \
-    } while (0)
-#endif
+void column_setup();
+void column_pass(cudaStream_t st, const TileParams& P, const float* table, bool lowmem, int pb);
 
 template <int D, bool LM, int PB, typename CT>
 __device__ __forceinline__ void tile_component(int tid, const TileGeom& g, const TileParams& P,
@@ -30,18 +18,14 @@ __device__ __forceinline__ void tile_component(int tid, const TileGeom& g, const
                                                unsigned long long& lo, unsigned long long& hi,
                                                float gscale) {
     __syncthreads();
-    PMPM_MARK(7 + 4 * D);
     if (D > 0) {   // the x force's inverse z ran with the forward z pass
         tile_inv_z<D>(tid, g, gS, C, W);
         __syncthreads();
     }
-    PMPM_MARK(8 + 4 * D);
     tile_inv_y(tid, g, W);
     __syncthreads();
-    PMPM_MARK(9 + 4 * D);
     tile_inv_x(tid, g, W);
     __syncthreads();
-    PMPM_MARK(10 + 4 * D);
     tile_interp<D, LM, PB>(tid, g, P, W, cells, lo, hi, gscale);
 }
 
@@ -92,18 +76,14 @@ __device__ __forceinline__ void tile_body(int tile, const TileParams& P,
     const int tid = threadIdx.x;
     const TileGeom g = tile_geom(tile, P.nc, P.nt);
     const TileCells cells = tile_cells(W, O);   // W is free until phase 5
-    PMPM_MARK(0);
     tile_prologue(tid, g, P, cells, R, gS);
     __syncthreads();
-    PMPM_MARK(1);
     tile_cells_scan(tid, g, cells);
     __syncthreads();
     tile_cells_map(tid, g, cells);
     __syncthreads();
-    PMPM_MARK(2);
     tile_deposit_flat<PB>(tid, g, P, R, cells);
     __syncthreads();
-    PMPM_MARK(3);
     // FP16 storage: the density less its mean over the halo box (the k = 0
     // mode, where the short-range kernel vanishes) is scaled by 2^-e so that
     // every spectrum value, at most 2 x 2^22 per particle of the box (the
@@ -120,10 +100,8 @@ __device__ __forceinline__ void tile_body(int tile, const TileParams& P,
     }
     tile_fwd_x<CT>(tid, R, scale, mean);
     __syncthreads();
-    PMPM_MARK(4);
     tile_fwd_y(tid, C);
     __syncthreads();
-    PMPM_MARK(5);
     tile_fwd_z_inv_z0(tid, g, gS, C, W);
     unsigned long long lo = 0, hi = 0;
     tile_component<0, LM, PB>(tid, g, P, gS, C, W, cells, lo, hi, gscale);
@@ -131,17 +109,14 @@ __device__ __forceinline__ void tile_body(int tile, const TileParams& P,
     tile_component<2, LM, PB>(tid, g, P, gS, C, W, cells, lo, hi, gscale);
     if (P.mode == 1 && P.counts_new != nullptr) tile_sigma_flush(tid, P, W, lo, hi);
     __syncthreads();
-    PMPM_MARK(19);
 }
 
-// One CTA per tile; one fits an SM at a time (the tile needs 232 KB of shared
-// memory).
-// PB: bytes per position bin; CT: storage of the tile spectrum; LM: the
-// low-memory step.
-template <int PB, typename CT, bool LM = false>
+// FP16 storage option: one CTA per tile; one fits an SM at a time (the tile
+// needs 232 KB of shared memory).  PB: bytes per position bin.
+template <int PB>
 __global__ void __launch_bounds__(kTileThreads, 1) k_tile(TileParams P) {
     extern __shared__ __align__(16) unsigned char tile_smem[];
-    tile_body<LM, PB, CT>((int)blockIdx.x, P, tile_smem);
+    tile_body<false, PB, __half2>((int)blockIdx.x, P, tile_smem);
 }
 
 // One tile's fine-mesh box right after the deposit, written out in x-fastest
@@ -169,14 +144,11 @@ __global__ void __launch_bounds__(kTileThreads, 1) k_tile_density(TileParams P, 
 }
 
 void tile_setup() {
-    cudaFuncSetAttribute(k_tile<1, float2>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)kTileSmemBytes);
-    cudaFuncSetAttribute(k_tile<2, float2>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)kTileSmemBytes);
-    cudaFuncSetAttribute(k_tile<1, __half2>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)kTileSmemBytes);
-    cudaFuncSetAttribute(k_tile<2, __half2>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)kTileSmemBytes);
-    cudaFuncSetAttribute(k_tile<1, float2, true>, cudaFuncAttributeMaxDynamicSharedMemorySize,
-                         (int)kTileSmemBytes);
+    cudaFuncSetAttribute(k_tile<1>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)kTileSmemBytes);
+    cudaFuncSetAttribute(k_tile<2>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)kTileSmemBytes);
     cudaFuncSetAttribute(k_tile_density<1>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)kTileSmemBytes);
     cudaFuncSetAttribute(k_tile_density<2>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)kTileSmemBytes);
+    column_setup();
 }
 
 // the parameters every tile kernel reads: the current store, the tables and F_l
@@ -209,21 +181,18 @@ int tile_pass(Sim& s, int mode, float* G) {
     TileParams P = base_params(s);
     P.mode = mode;
     P.G = G;
-    const int grid = s.nt * s.nt * s.nt;
     if (mode == 1) {
         P.counts_new = s.counts[1 - s.cur];
         P.S = s.S;
         P.d2 = s.d2;
     }
-    if (s.lowmem) {
-        // the low-memory step keeps the new momenta only (s.Pn); the new codes
-        // are derived again by its re-encode
-        P.Qn = nullptr;
-        k_tile<1, float2, true><<<grid, kTileThreads, kTileSmemBytes, s.stream>>>(P);
-    } else if (s.fp16 && s.pb == 2) k_tile<2, __half2><<<grid, kTileThreads, kTileSmemBytes, s.stream>>>(P);
-    else if (s.fp16) k_tile<1, __half2><<<grid, kTileThreads, kTileSmemBytes, s.stream>>>(P);
-    else if (s.pb == 2) k_tile<2, float2><<<grid, kTileThreads, kTileSmemBytes, s.stream>>>(P);
-    else k_tile<1, float2><<<grid, kTileThreads, kTileSmemBytes, s.stream>>>(P);
+    // the low-memory step keeps the new momenta only (s.Pn); the new codes are
+    // derived again by its re-encode
+    if (s.lowmem) P.Qn = nullptr;
+    const int grid = s.nt * s.nt * s.nt;
+    if (!s.fp16) column_pass(s.stream, P, s.green_col, s.lowmem, s.pb);
+    else if (s.pb == 2) k_tile<2><<<grid, kTileThreads, kTileSmemBytes, s.stream>>>(P);
+    else k_tile<1><<<grid, kTileThreads, kTileSmemBytes, s.stream>>>(P);
     s.launches++;
     return check_launch(s, "tile pass");
 }
@@ -238,9 +207,3 @@ int tile_density(Sim& s, int tile, uint32_t* d_out) {
 }
 
 }  // namespace pmpm
-
-#ifdef PMPM_PHASE_CLOCKS
-extern "C" int pmpm_debug_phases(unsigned long long* out, int n) {
-    return (int)cudaMemcpyFromSymbol(out, pmpm::g_phase, sizeof(unsigned long long) * n);
-}
-#endif

@@ -839,7 +839,7 @@ PMPM_HD void tile_fwd_z_inv_z0(int tid, const TileGeom& g, const float* gS, CT* 
 // The inverse y and x passes are the same for the three force components;
 // one out-of-line copy each keeps the kernel's code within the instruction
 // cache (measured: 1.2% faster than three inlined copies).
-__host__ __device__ __noinline__ void tile_inv_y(int tid, const TileGeom& g, float2* W) {
+inline __host__ __device__ __noinline__ void tile_inv_y(int tid, const TileGeom& g, float2* W) {
     const int nz = g.T[2] + 2, ny = g.T[1] + 2;
     if (tid >= 16 * nz) return;
     const int kx = tid & 15, zo = tid >> 4;
@@ -853,7 +853,7 @@ __host__ __device__ __noinline__ void tile_inv_y(int tid, const TileGeom& g, flo
 }
 
 // --- phase 5c: inverse real transform along x, pruned to T + 2 columns ----
-__host__ __device__ __noinline__ void tile_inv_x(int tid, const TileGeom& g, float2* W) {
+inline __host__ __device__ __noinline__ void tile_inv_x(int tid, const TileGeom& g, float2* W) {
     const int ny = g.T[1] + 2, nz = g.T[2] + 2, nx = g.T[0] + 2;   // all even
     for (int r = tid; r < ny * nz; r += kTileThreads) {
         const int yo = r % ny, zo = r / ny;

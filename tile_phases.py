@@ -1,10 +1,10 @@
-"""Per-phase clock breakdown of the tile pass: a measurement tool beside
-bench.py (the library itself is not built with it).
+"""Per-phase clock breakdown of the column pass (the short-range pass of a
+step): a measurement tool beside bench.py (the library itself is not built
+with it).
 
-Builds a second copy of the library with -DPMPM_PHASE_CLOCKS, in which
-thread 0 of every tile CTA stamps clock64() after each block barrier of the
-tile pass, runs a box, and prints the mean cycles per phase over the first
-4096 tiles of the chosen steps:
+Builds a second copy of the library with -DPMPM_PHASE_CLOCKS, in which every
+warp adds up clock64() between the marks of a layer, runs a box, and prints
+the mean cycles per layer and warp of the chosen steps:
 
     python tile_phases.py [--workload c3_512] [--steps 1 10 20]
 """
@@ -21,15 +21,10 @@ sys.path.insert(0, ROOT)
 PKG = os.path.join(ROOT, "paper_2003_03931_gb300")
 PROF_LIB = os.path.join(PKG, "_build_phases", "libpmpm_phases.so")
 
-# stamp k closes phase k - 1; names follow the kernel's phase order
-PHASES = ["prologue (loads, zero)", "halo scan + cell maps", "deposit + long-range gather",
-          "forward x (R2C)", "forward y", "forward z",
-          "Green x + inverse z", "inverse y (x force)", "inverse x (x force)", "interpolate x",
-          "Green y + inverse z", "inverse y (y force)", "inverse x (y force)", "interpolate y",
-          "Green z + inverse z", "inverse y (z force)", "inverse x (z force)",
-          "interpolate z + kick + drift"]
-MARKS = [0, 1, 2, 3, 4, 5, 7, 8, 9, 10, 11, 12, 13, 14, 15, 16, 17, 18, 19]
-N_MARKS = 24
+# the intervals that the marks of k_column close, in a layer's order
+PHASES = ["forward, tables | gather", "  wait", "z sum", "  wait", "inverse y", "inverse x", "  wait | clear",
+          "deposit", "own loads", "  wait"]
+N_MARKS, WARPS = 12, 8
 
 
 def main(argv=None):
@@ -49,20 +44,22 @@ def main(argv=None):
     sim = Simulation(SimConfig(**w))
     sim.ic_zeldovich(1, **synth.IC_SPECTRUM)
     sim.lib.pmpm_debug_phases.argtypes = [ctypes.c_void_p, ctypes.c_int]
+    buf = np.zeros(WARPS * N_MARKS, np.uint64)
     for step in sorted(args.steps):
         while sim.fetch_scalars()["step"] < step:
             sim.step(1)
+        sim.sync()
+        sim.lib.pmpm_debug_phases(buf.ctypes.data, buf.size)   # clears
         sim.step(1)
         sim.sync()
-        buf = np.zeros(4096 * N_MARKS, np.uint64)
         sim.lib.pmpm_debug_phases(buf.ctypes.data, buf.size)
-        b = buf.reshape(4096, N_MARKS).astype(np.int64)
-        b = b[b[:, 19] > 0]
-        d = np.diff(b[:, MARKS], axis=1)
-        tot = b[:, 19] - b[:, 0]
-        print(f"step {step}: {len(b)} tiles, cycles per tile mean {tot.mean():.0f} max {tot.max():.0f}")
+        b = buf.reshape(WARPS, N_MARKS).astype(np.float64)
+        layers = b[:, 10:11].max()
+        b = b[:, :len(PHASES)] / layers
+        print(f"step {step}: {int(layers)} layers walked, {b.sum(axis=1).mean():.0f} cycles a layer")
+        print("  %-30s" % "warp" + "".join(f"{i:7d}" for i in range(WARPS)))
         for i, name in enumerate(PHASES):
-            print(f"  {name:32s} {d[:, i].mean():9.0f}  ({100 * d[:, i].mean() / tot.mean():4.1f}%)")
+            print("  %-30s" % name + "".join(f"{v:7.0f}" for v in b[:, i]))
     sim.close()
 
 
