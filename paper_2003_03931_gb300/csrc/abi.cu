@@ -89,7 +89,7 @@ static void derive(Sim& s, const pmpm_config* c) {
     s.fft_max = s.nc;
     if (s.np > s.fft_max) s.fft_max = s.np;
     if (s.pk_max > s.fft_max) s.fft_max = s.pk_max;
-    s.nblocks_scan = (s.ncells + 4095) / 4096;
+    s.nblocks_scan = s.ncells / (256 * scan_items(s.ncells));
     s.lowmem = (c->flags & PMPM_FLAG_LOWMEM) != 0;
     s.fp16 = (c->flags & PMPM_FLAG_FINE_FP16) != 0;
     s.pb = c->pos_bytes == 2 ? 2 : 1;
@@ -140,7 +140,7 @@ static size_t layout_lowmem(Sim& s, uint8_t* base) {
     s.d_factors = reinterpret_cast<float*>(take(8 * (size_t)s.cfg.n_steps));
     s.d_step = reinterpret_cast<int*>(take(4));
     s.d_kd = reinterpret_cast<float*>(take(8));
-    s.d2 = reinterpret_cast<unsigned long long*>(take(64));
+    s.d2 = reinterpret_cast<unsigned long long*>(take(72));
     for (int b = 0; b < 2; ++b) s.sigma_d[b] = reinterpret_cast<float*>(take(4));
     off = align_up(off);
     const size_t p0 = off;
@@ -202,7 +202,7 @@ size_t layout(Sim& s, uint8_t* base) {
     }
     s.fill = reinterpret_cast<int32_t*>(take(4 * (size_t)C));
     s.S = reinterpret_cast<unsigned long long*>(take(24 * (size_t)C));
-    s.d2 = reinterpret_cast<unsigned long long*>(take(64));
+    s.d2 = reinterpret_cast<unsigned long long*>(take(72));
     s.rho_c = reinterpret_cast<long long*>(take(8 * (size_t)C));
     s.cA = reinterpret_cast<float2*>(take(8 * (size_t)C));
     s.cB1 = reinterpret_cast<float2*>(take(8 * (size_t)C));
@@ -303,18 +303,31 @@ static double sched_a(const Sim& s, int64_t n) {
     return s.cfg.a_init * pow(s.cfg.a_final / s.cfg.a_init, (double)n / (double)s.cfg.n_steps);
 }
 
-// The device step counter and the kick/drift factors of that step, which
-// the tile pass reads (one pair per step, so a captured step replays as is).
-__global__ void k_step_set(int* step, float* kd, const float* factors, int n_steps, int v) {
-    *step = v;
-    kd[0] = v < n_steps ? factors[2 * v] : 0.f;
-    kd[1] = v < n_steps ? factors[2 * v + 1] : 0.f;
-}
-__global__ void k_step_advance(int* step, float* kd, const float* factors, int n_steps) {
-    const int v = *step + 1;
-    *step = v;
-    kd[0] = v < n_steps ? factors[2 * v] : 0.f;
-    kd[1] = v < n_steps ? factors[2 * v + 1] : 0.f;
+// The device step counter: the index of the next step.
+__global__ void k_step_set(int* step, int v) { *step = v; }
+
+// Begins a step: takes the kick and drift factors of the counter's step (one
+// pair per step in device memory, so a captured step replays as is), moves the
+// counter on, and clears everything the step adds to, in one launch: the coarse
+// density, the new counts and momentum sums (all multiples of 16 bytes) and the
+// dispersion's digits.
+__global__ void __launch_bounds__(256) k_step_begin(int* step, float* kd, const float* factors, int n_steps,
+                                                    int64_t ncells, uint4* rho, uint4* counts, uint4* S,
+                                                    unsigned long long* d2) {
+    if (blockIdx.x == 0) {
+        if (threadIdx.x < 9) d2[threadIdx.x] = 0;
+        if (threadIdx.x == 32) {
+            const int v = *step;
+            *step = v + 1;
+            kd[0] = v < n_steps ? factors[2 * v] : 0.f;
+            kd[1] = v < n_steps ? factors[2 * v + 1] : 0.f;
+        }
+    }
+    const uint4 zero = make_uint4(0u, 0u, 0u, 0u);
+    const int64_t t = blockIdx.x * (int64_t)blockDim.x + threadIdx.x, stride = (int64_t)gridDim.x * blockDim.x;
+    for (int64_t i = t; i < ncells / 2; i += stride) rho[i] = zero;
+    for (int64_t i = t; i < ncells / 4; i += stride) counts[i] = zero;
+    for (int64_t i = t; i < 3 * ncells / 2; i += stride) S[i] = zero;
 }
 
 static double cfg_a(const pmpm_config& c, int64_t n) {
@@ -353,7 +366,7 @@ static void fill_factors(Sim& s) {
 }
 
 void set_device_step(Sim& s, int64_t step) {
-    k_step_set<<<1, 1, 0, s.stream>>>(s.d_step, s.d_kd, s.d_factors, s.cfg.n_steps, (int)step);
+    k_step_set<<<1, 1, 0, s.stream>>>(s.d_step, (int)step);
 }
 
 // Device work of one step; swaps the store buffers (s.cur).
@@ -361,18 +374,17 @@ static int enqueue_step(Sim& s) {
     int rc;
     prof_mark(s, -1);
     if (s.lowmem) lowmem_bind(s, 1 - s.cur);   // S and F_l in the next store's region
-    if ((rc = coarse_deposit(s))) return rc;
+    k_step_begin<<<grid_for(3 * s.ncells / 2, 256), 256, 0, s.stream>>>(
+        s.d_step, s.d_kd, s.d_factors, s.cfg.n_steps, s.ncells, reinterpret_cast<uint4*>(s.rho_c),
+        reinterpret_cast<uint4*>(s.counts[1 - s.cur]), reinterpret_cast<uint4*>(s.S), s.d2);
+    s.launches++;
+    if ((rc = coarse_deposit(s, true))) return rc;
     prof_mark(s, 0);
     if ((rc = coarse_force(s))) return rc;
     prof_mark(s, 1);
-    cudaMemsetAsync(s.counts[1 - s.cur], 0, sizeof(int32_t) * s.ncells, s.stream);
-    cudaMemsetAsync(s.S, 0, sizeof(unsigned long long) * 3 * s.ncells, s.stream);
-    cudaMemsetAsync(s.d2, 0, 64, s.stream);
     if ((rc = tile_pass(s, 1, nullptr))) return rc;
     prof_mark(s, 2);
     if ((rc = s.lowmem ? encode_from_parked(s) : encode_from_qp(s, true))) return rc;
-    k_step_advance<<<1, 1, 0, s.stream>>>(s.d_step, s.d_kd, s.d_factors, s.cfg.n_steps);
-    s.launches++;
     return check_launch(s, "step");
 }
 
@@ -462,6 +474,7 @@ static pmpm_sim* init_common(const pmpm_config* cfg, void* d_workspace, size_t b
     cudaGetDevice(&s.device);
     tile_setup();
     fft_setup();
+    coarse_setup();
     cudaMemsetAsync(s.err, 0, 4, s.stream);
     float T[256], E[256];
     codec_tables(T, E);

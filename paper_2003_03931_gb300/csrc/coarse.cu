@@ -10,7 +10,11 @@
 //  2. delta = rho - mean (float64 subtraction, float32 storage), 3-D FFT;
 //  3. Green multiply: B1 = rho~ (K~_x + i K~_y), B2 = rho~ K~_z (K~ = -i S);
 //  4. two inverse FFTs give F_x + i F_y and F_z.
+// Meshes up to 32^3 fit one SM's shared memory: 2-4 are one launch
+// (k_coarse_tiny, k_coarse_small).  Larger ones take five passes over memory, the
+// ends and the Green multiply fused into them.
 #include "pmpm_impl.cuh"
+#include "regfft.cuh"
 
 namespace pmpm {
 
@@ -107,57 +111,525 @@ __global__ void __launch_bounds__(256) k_coarse_deposit(int nc, const int32_t* _
     }
 }
 
-__global__ void k_coarse_delta(int64_t ncells, double mean, const long long* __restrict__ rho,
-                               float2* __restrict__ out) {
-    for (int64_t i = blockIdx.x * (int64_t)blockDim.x + threadIdx.x; i < ncells;
-         i += (int64_t)gridDim.x * blockDim.x)
-        out[i] = make_float2((float)((double)rho[i] - mean), 0.f);
-}
-
 __device__ __forceinline__ void kfold(int k, int nc, int& a, float& sg) {
     if (k == 0) { a = 0; sg = 0.f; }
     else if (k <= nc / 2) { a = k; sg = 1.f; }
     else { a = nc - k; sg = -1.f; }
 }
 
-__global__ void k_coarse_green(int nc, const float4* __restrict__ table,
-                               const float2* __restrict__ A, float2* __restrict__ B1,
-                               float2* __restrict__ B2) {
-    const int64_t ncells = (int64_t)nc * nc * nc;
-    const int64_t h = nc / 2 + 1;
-    for (int64_t i = blockIdx.x * (int64_t)blockDim.x + threadIdx.x; i < ncells;
-         i += (int64_t)gridDim.x * blockDim.x) {
-        const int kx = (int)(i % nc), ky = (int)((i / nc) % nc), kz = (int)(i / ((int64_t)nc * nc));
-        int ax, ay, az;
-        float sx, sy, sz;
-        kfold(kx, nc, ax, sx);
-        kfold(ky, nc, ay, sy);
-        kfold(kz, nc, az, sz);
-        // the three components' kernels at (|kx|, |ky|, |kz|), |kx| fastest
-        const float4 g = table[(az * h + ay) * h + ax];
-        const float Sx = sx * g.x, Sy = sy * g.y, Sz = sz * g.z;
-        const float2 a = A[i];
-        // B1 = a (S_y - i S_x),  B2 = a (-i S_z)
-        B1[i] = make_float2(a.x * Sy + a.y * Sx, a.y * Sy - a.x * Sx);
-        B2[i] = make_float2(a.y * Sz, -a.x * Sz);
+// fl32(rho - mean).  The mean, N 2^27 / nc^3 with powers of two, is an integer of
+// at least 8, so the difference is exact in 64 bits; two halves that float32
+// holds exactly and one multiply-add round it once.  (64-bit conversions and
+// FP64 run at 1/64 of the FP32 rate here: three per cell took 24 us of a 32^3
+// mesh on three SMs.)
+__device__ __forceinline__ float delta_of(long long rho, long long mean) {
+    const long long d = rho - mean;
+    const int hi = (int)(d >> 16);
+    if (d >= (1ll << 40) || d < -(1ll << 40)) return __ll2float_rn(d);
+    return __fmaf_rn((float)hi, 65536.f, (float)((int)d & 0xffff));
+}
+
+// ------------------------------------------------------------ up to 16^3 cells
+// The whole chain on a complex mesh in one CTA's shared memory: blockIdx.x = 0
+// transforms back to F_x + i F_y, 1 to F_z, and both do the forward transform
+// (as separate launches the chain is launch-bound: twelve take 68 us at 16^3 on
+// a GB300, this one 13).  A thread holds a pencil; the radix-2 autosort stages,
+// their twiddles, roundings and the order of the axes are those of fft.cu's
+// k_fft_pass, so the two give the same bits.
+__device__ __forceinline__ float2 cmul(float2 a, float2 b) {
+    return make_float2(__fmaf_rn(a.x, b.x, -__fmul_rn(a.y, b.y)), __fmaf_rn(a.y, b.x, __fmul_rn(a.x, b.y)));
+}
+
+template <int N, int S>
+__device__ __forceinline__ void autosort(float2 (&a)[N], const float2 (&tw)[N / 2]) {
+#pragma unroll
+    for (int Ns = 1; Ns < N; Ns *= 2) {
+        float2 d[N];
+#pragma unroll
+        for (int j = 0; j < N / 2; ++j) {
+            const int k = j & (Ns - 1), o = ((j - k) << 1) + k;
+            float2 w = tw[k * (N / 2 / Ns)];
+            if (S > 0) w.y = -w.y;
+            const float2 v0 = a[j], v1 = cmul(a[j + N / 2], w);
+            d[o] = make_float2(v0.x + v1.x, v0.y + v1.y);
+            d[o + Ns] = make_float2(v0.x - v1.x, v0.y - v1.y);
+        }
+#pragma unroll
+        for (int j = 0; j < N; ++j) a[j] = d[j];
     }
 }
 
-__global__ void k_coarse_extract(int64_t ncells, const float2* __restrict__ B1,
-                                 const float2* __restrict__ B2, float* __restrict__ Fl) {
-    for (int64_t i = blockIdx.x * (int64_t)blockDim.x + threadIdx.x; i < ncells;
-         i += (int64_t)gridDim.x * blockDim.x) {
-        const float2 b1 = B1[i];
-        Fl[i] = b1.x;
-        Fl[ncells + i] = b1.y;
-        Fl[2 * ncells + i] = B2[i].x;
+template <int N, int S>
+__device__ __forceinline__ void tiny_pencil(float2* c, int stride, const float2 (&tw)[N / 2]) {
+    float2 a[N];
+#pragma unroll
+    for (int k = 0; k < N; ++k) a[k] = c[k * stride];
+    autosort<N, S>(a, tw);
+#pragma unroll
+    for (int k = 0; k < N; ++k) c[k * stride] = a[k];
+}
+
+template <int N>
+__global__ void __launch_bounds__(N * N) k_coarse_tiny(long long mean, const long long* __restrict__ rho,
+                                                       const float4* __restrict__ table, float* __restrict__ Fl,
+                                                       const float2* __restrict__ twiddles, int twsh) {
+    constexpr int P = N + 1, h = N / 2 + 1, cells = N * N * N;
+    __shared__ float2 C[N * N * P];
+    const int tid = threadIdx.x, x = tid % N, y = tid / N;   // (y, z) for the x pencils, (x, z) and (x, y)
+    float2 tw[N / 2];
+#pragma unroll
+    for (int k = 0; k < N / 2; ++k) tw[k] = twiddles[k << twsh];
+#pragma unroll 4
+    for (int z = 0; z < N; ++z) C[(z * N + y) * P + x] = make_float2(delta_of(rho[z * N * N + tid], mean), 0.f);
+    __syncthreads();
+    tiny_pencil<N, -1>(C + tid * P, 1, tw);
+    __syncthreads();
+    tiny_pencil<N, -1>(C + y * N * P + x, P, tw);
+    __syncthreads();
+    float2 a[N];
+    float2* const col = C + y * P + x;   // the z pencil of (x, y)
+#pragma unroll
+    for (int z = 0; z < N; ++z) a[z] = col[z * (N * P)];
+    autosort<N, -1>(a, tw);
+    int ax, ay;
+    float sx, sy;
+    kfold(x, N, ax, sx);
+    kfold(y, N, ay, sy);
+#pragma unroll
+    for (int z = 0; z < N; ++z) {
+        int az;
+        float sz;
+        kfold(z, N, az, sz);
+        const float4 g = table[(az * h + ay) * h + ax];
+        const float Sx = sx * g.x, Sy = sy * g.y, Sz = sz * g.z;
+        // a (S_y - i S_x) or a (-i S_z)
+        col[z * (N * P)] = blockIdx.x == 0 ? make_float2(__fmaf_rn(a[z].x, Sy, __fmul_rn(a[z].y, Sx)),
+                                                         __fmaf_rn(a[z].y, Sy, -__fmul_rn(a[z].x, Sx)))
+                                           : make_float2(a[z].y * Sz, -a[z].x * Sz);
     }
+    __syncthreads();
+    tiny_pencil<N, 1>(C + tid * P, 1, tw);
+    __syncthreads();
+    tiny_pencil<N, 1>(C + y * N * P + x, P, tw);
+    __syncthreads();
+#pragma unroll
+    for (int z = 0; z < N; ++z) a[z] = col[z * (N * P)];
+    autosort<N, 1>(a, tw);
+#pragma unroll
+    for (int z = 0; z < N; ++z) {
+        if (blockIdx.x == 0) {
+            Fl[z * N * N + tid] = a[z].x;
+            Fl[cells + z * N * N + tid] = a[z].y;
+        } else {
+            Fl[2 * cells + z * N * N + tid] = a[z].x;
+        }
+    }
+}
+
+// ------------------------------------------------------------ 32^3 cells
+// The force of one component in one CTA: real transforms along x with the kx = 16
+// plane in the imaginary part of kx = 0 (139 KB of shared memory), rows 17
+// complex apart so that pencils along every axis fall in distinct banks; along
+// z forward, Green multiply and back from the registers.  Three CTAs transform
+// the density each, which is cheaper than twelve launches (69 us on a GB300,
+// against 29).
+template <int N>
+struct SmallMesh {
+    static constexpr int kH = N / 2, kP = kH + 1, kLog = 5;
+    static constexpr int kThreads = N * kH;
+    static constexpr size_t kBytes = sizeof(float2) * N * N * kP;
+};
+
+template <int N, int S>
+__device__ __forceinline__ void small_pencil(float2* c, int stride) {
+    float2 a[N];
+#pragma unroll
+    for (int k = 0; k < N; ++k) a[bitrev<SmallMesh<N>::kLog>(k)] = c[k * stride];
+    fft_dit<N, S>(a);
+#pragma unroll
+    for (int k = 0; k < N; ++k) c[k * stride] = a[k];
+}
+
+template <int N>
+__global__ void __launch_bounds__(SmallMesh<N>::kThreads) k_coarse_small(long long mean, const long long* __restrict__ rho,
+                                                                         const float4* __restrict__ table,
+                                                                         float* __restrict__ Fl) {
+    using M = SmallMesh<N>;
+    constexpr int H = M::kH, P = M::kP, T = M::kThreads, L = M::kLog;
+    extern __shared__ __align__(16) unsigned char small_smem[];
+    float2* C = reinterpret_cast<float2*>(small_smem);
+    float* R = reinterpret_cast<float*>(small_smem);
+    const int tid = threadIdx.x, comp = blockIdx.x;
+#pragma unroll 8
+    for (int i = tid; i < N * N * N; i += T) R[(i >> L) * (2 * P) + (i & (N - 1))] = delta_of(rho[i], mean);
+    __syncthreads();
+    for (int r = tid; r < N * N; r += T) {
+        float2* row = C + r * P;
+        float x[N];
+        float2 X[H + 1];
+#pragma unroll
+        for (int k = 0; k < H; ++k) {
+            x[2 * k] = row[k].x;
+            x[2 * k + 1] = row[k].y;
+        }
+        rfftx2<N>(x, X);
+        row[0] = make_float2(X[0].x, X[H].x);
+#pragma unroll
+        for (int k = 1; k < H; ++k) row[k] = X[k];
+    }
+    __syncthreads();
+    for (int t = tid; t < H * N; t += T)   // along y: kx, z
+        small_pencil<N, -1>(C + (t / H) * (N * P) + t % H, P);
+    __syncthreads();
+    for (int t = tid; t < H * N; t += T) {   // along z: kx = t / N, ky = t mod N
+        const int kx = t / N, ky = t % N;
+        float2* col = C + ky * P + kx;
+        float2 a[N];
+#pragma unroll
+        for (int k = 0; k < N; ++k) a[bitrev<L>(k)] = col[k * (N * P)];
+        fft_dit<N, -1>(a);
+        int ay;
+        float sy;
+        kfold(ky, N, ay, sy);
+        if (kx != 0) {
+#pragma unroll
+            for (int kz = 0; kz < N; ++kz) {
+                const int az = kz <= H ? kz : N - kz;
+                const float sz = kz == 0 ? 0.f : (kz <= H ? 1.f : -1.f);
+                const float4 g = table[(az * (H + 1) + ay) * (H + 1) + kx];
+                const float c = comp == 0 ? g.x : (comp == 1 ? sy * g.y : sz * g.z);
+                a[kz] = make_float2(c * a[kz].y, -(c * a[kz].x));   // -i c a
+            }
+        } else {
+            // Z = A + i B holds kx = 0 and kx = N/2; with the partner Z' at (-ky, -kz),
+            // -i (s0 A + i sH B) = -i [(s0 + sH)/2 Z + (s0 - sH)/2 conj Z'] (the x
+            // component's s0 and sH vanish).  One warp holds the column.
+#pragma unroll
+            for (int kz = 0; kz < N; ++kz) col[kz * (N * P)] = a[kz];
+            __syncwarp();
+            const float2* mate = C + ((N - ky) & (N - 1)) * P;
+            float2 b[N];
+#pragma unroll
+            for (int kz = 0; kz < N; ++kz) b[kz] = mate[((N - kz) & (N - 1)) * (N * P)];
+            __syncwarp();
+#pragma unroll
+            for (int kz = 0; kz < N; ++kz) {
+                const int az = kz <= H ? kz : N - kz;
+                const float sz = kz == 0 ? 0.f : (kz <= H ? 1.f : -1.f);
+                const float4 g0 = table[(az * (H + 1) + ay) * (H + 1)], gH = table[(az * (H + 1) + ay) * (H + 1) + H];
+                const float s0 = comp == 0 ? 0.f : (comp == 1 ? sy * g0.y : sz * g0.z);
+                const float sH = comp == 0 ? 0.f : (comp == 1 ? sy * gH.y : sz * gH.z);
+                const float cA = 0.5f * (s0 + sH), cB = 0.5f * (s0 - sH);
+                const float vx = cA * a[kz].x + cB * b[kz].x, vy = cA * a[kz].y - cB * b[kz].y;
+                a[kz] = make_float2(vy, -vx);
+            }
+        }
+        float2 w[N];
+#pragma unroll
+        for (int k = 0; k < N; ++k) w[bitrev<L>(k)] = a[k];
+        fft_dit<N, 1>(w);
+#pragma unroll
+        for (int k = 0; k < N; ++k) col[k * (N * P)] = w[k];
+    }
+    __syncthreads();
+    for (int t = tid; t < H * N; t += T) small_pencil<N, 1>(C + (t / H) * (N * P) + t % H, P);
+    __syncthreads();
+    for (int r = tid; r < N * N; r += T) {
+        float2* row = C + r * P;
+        float x[N];
+        float2 X[H + 1];
+        X[0] = make_float2(row[0].x, 0.f);
+        X[H] = make_float2(row[0].y, 0.f);
+#pragma unroll
+        for (int k = 1; k < H; ++k) X[k] = row[k];
+        irfft<N>(X, x);
+#pragma unroll
+        for (int k = 0; k < H; ++k) row[k] = make_float2(0.5f * x[2 * k], 0.5f * x[2 * k + 1]);   // rfftx2 doubles
+    }
+    __syncthreads();
+    for (int i = tid; i < N * N * N; i += T) Fl[(int64_t)comp * N * N * N + i] = R[(i >> L) * (2 * P) + (i & (N - 1))];
+}
+
+// ------------------------------------------------------------ 64^3 cells and more
+// Passes of n = N1 N2 points per pencil in two register steps with one
+// transpose through shared memory (fft.cu).  With j = N2 n1 + n2 and
+// k = k1 + N1 k2 the forward pass ends with all k2 of one k1 in a thread's
+// registers, which is where the inverse one begins: the z pass transforms,
+// multiplies and transforms back without another exchange.  116 bytes a cell
+// over five launches against 212 over twelve: 64^3 cells 73 -> 38 us, 128^3
+// 126 -> 72, 256^3 (HBM-bound) 710 -> 399.
+constexpr int kCoarseThreads = 256;
+constexpr int clog2(int v) { return v <= 1 ? 0 : 1 + clog2(v / 2); }
+
+template <int N1, int N2>
+struct Pass {
+    static constexpr int n = N1 * N2, L1 = clog2(N1), L2 = clog2(N2), LN = L1 + L2;
+    static constexpr int P = 4096 / n < 8 ? 8 : 4096 / n, LP = clog2(P);   // pencils of a block
+    static constexpr int RS = N2 + 1, PS = N1 * RS + 1;                    // see k_fft_pass_r
+    static constexpr size_t kBytes = sizeof(float2) * P * PS;
+};
+
+__device__ __forceinline__ float2 cmulw(float2 a, float2 w) {
+    return make_float2(a.x * w.x - a.y * w.y, a.x * w.y + a.y * w.x);
+}
+
+// N1-point step over n1 of item (p, n2), times W_n^(n2 k1), into the buffer
+template <int N1, int N2>
+__device__ __forceinline__ void pass_first(float2 (&a)[N1], float2* Y, int p, int n2, const float2* tw, int twsh) {
+    using Q = Pass<N1, N2>;
+    fft_dit<N1, -1>(a);
+#pragma unroll
+    for (int k1 = 0; k1 < N1; ++k1) Y[p * Q::PS + k1 * Q::RS + n2] = cmulw(a[k1], tw[(n2 * k1) << twsh]);
+}
+// and the N2-point step of item (p, k1) from it
+template <int N1, int N2>
+__device__ __forceinline__ void pass_second(float2 (&a)[N2], const float2* Y, int p, int k1) {
+    using Q = Pass<N1, N2>;
+#pragma unroll
+    for (int n2 = 0; n2 < N2; ++n2) a[bitrev<Q::L2>(n2)] = Y[p * Q::PS + k1 * Q::RS + n2];
+    fft_dit<N2, -1>(a);
+}
+// inverse: the N2-point step of item (p, k1) into the buffer
+template <int N1, int N2>
+__device__ __forceinline__ void back_first(float2 (&a)[N2], float2* Y, int p, int k1, const float2* tw, int twsh) {
+    using Q = Pass<N1, N2>;
+    fft_dit<N2, 1>(a);
+#pragma unroll
+    for (int n2 = 0; n2 < N2; ++n2) {
+        const float2 w = tw[(n2 * k1) << twsh];
+        Y[p * Q::PS + k1 * Q::RS + n2] = cmulw(a[n2], make_float2(w.x, -w.y));
+    }
+}
+// and the N1-point step of item (p, n2): a[n1]
+template <int N1, int N2>
+__device__ __forceinline__ void back_second(float2 (&a)[N1], const float2* Y, int p, int n2) {
+    using Q = Pass<N1, N2>;
+#pragma unroll
+    for (int k1 = 0; k1 < N1; ++k1) a[bitrev<Q::L1>(k1)] = Y[p * Q::PS + k1 * Q::RS + n2];
+    fft_dit<N1, 1>(a);
+}
+
+// x: integer density rows -> delta -> spectrum
+template <int N1, int N2>
+__global__ void __launch_bounds__(kCoarseThreads) k_coarse_fwd_x(long long mean, const long long* __restrict__ rho,
+                                                                 float2* __restrict__ out,
+                                                                 const float2* __restrict__ tw, int twsh) {
+    using Q = Pass<N1, N2>;
+    extern __shared__ __align__(16) unsigned char pass_smem[];
+    float2* Y = reinterpret_cast<float2*>(pass_smem);
+    const int64_t q0 = (int64_t)blockIdx.x * Q::P;
+    for (int it = threadIdx.x; it < Q::P * N2; it += kCoarseThreads) {
+        const int p = it >> Q::L2, n2 = it & (N2 - 1);
+        const long long* src = rho + ((q0 + p) << Q::LN) + n2;
+        float2 a[N1];
+#pragma unroll
+        for (int n1 = 0; n1 < N1; ++n1)
+            a[bitrev<Q::L1>(n1)] = make_float2(delta_of(src[N2 * n1], mean), 0.f);
+        pass_first<N1, N2>(a, Y, p, n2, tw, twsh);
+    }
+    __syncthreads();
+    for (int it = threadIdx.x; it < Q::P * N1; it += kCoarseThreads) {
+        const int p = it >> Q::L1, k1 = it & (N1 - 1);
+        float2 a[N2];
+        pass_second<N1, N2>(a, Y, p, k1);
+        float2* dst = out + ((q0 + p) << Q::LN) + k1;
+#pragma unroll
+        for (int k2 = 0; k2 < N2; ++k2) dst[N1 * k2] = a[k2];
+    }
+}
+
+// y: in place, forward (S = -1) or back; blockIdx.y picks the array
+template <int N1, int N2, int S>
+__global__ void __launch_bounds__(kCoarseThreads) k_coarse_y(float2* d0, float2* d1, const float2* __restrict__ tw,
+                                                             int twsh) {
+    using Q = Pass<N1, N2>;
+    extern __shared__ __align__(16) unsigned char pass_smem[];
+    float2* Y = reinterpret_cast<float2*>(pass_smem);
+    const int64_t q0 = (int64_t)blockIdx.x * Q::P;   // pencils (x, z), x fastest
+    float2* data = (blockIdx.y ? d1 : d0) + ((q0 >> Q::LN) << (2 * Q::LN)) + (q0 & (Q::n - 1));
+    if (S < 0) {
+        for (int it = threadIdx.x; it < Q::P * N2; it += kCoarseThreads) {
+            const int p = it & (Q::P - 1), n2 = it >> Q::LP;
+            float2 a[N1];
+#pragma unroll
+            for (int n1 = 0; n1 < N1; ++n1) a[bitrev<Q::L1>(n1)] = data[p + ((N2 * n1 + n2) << Q::LN)];
+            pass_first<N1, N2>(a, Y, p, n2, tw, twsh);
+        }
+        __syncthreads();
+        for (int it = threadIdx.x; it < Q::P * N1; it += kCoarseThreads) {
+            const int p = it & (Q::P - 1), k1 = it >> Q::LP;
+            float2 a[N2];
+            pass_second<N1, N2>(a, Y, p, k1);
+#pragma unroll
+            for (int k2 = 0; k2 < N2; ++k2) data[p + ((k1 + N1 * k2) << Q::LN)] = a[k2];
+        }
+    } else {
+        for (int it = threadIdx.x; it < Q::P * N1; it += kCoarseThreads) {
+            const int p = it & (Q::P - 1), k1 = it >> Q::LP;
+            float2 a[N2];
+#pragma unroll
+            for (int k2 = 0; k2 < N2; ++k2) a[bitrev<Q::L2>(k2)] = data[p + ((k1 + N1 * k2) << Q::LN)];
+            back_first<N1, N2>(a, Y, p, k1, tw, twsh);
+        }
+        __syncthreads();
+        for (int it = threadIdx.x; it < Q::P * N2; it += kCoarseThreads) {
+            const int p = it & (Q::P - 1), n2 = it >> Q::LP;
+            float2 a[N1];
+            back_second<N1, N2>(a, Y, p, n2);
+#pragma unroll
+            for (int n1 = 0; n1 < N1; ++n1) data[p + ((N2 * n1 + n2) << Q::LN)] = a[n1];
+        }
+    }
+}
+
+// z: forward, Green multiply and back for B1 and B2
+template <int N1, int N2>
+__global__ void __launch_bounds__(kCoarseThreads) k_coarse_z(const float4* __restrict__ table,
+                                                             const float2* __restrict__ A, float2* __restrict__ B1,
+                                                             float2* __restrict__ B2, const float2* __restrict__ tw,
+                                                             int twsh) {
+    using Q = Pass<N1, N2>;
+    constexpr int64_t plane = (int64_t)Q::n * Q::n;
+    constexpr int h = Q::n / 2 + 1;
+    extern __shared__ __align__(16) unsigned char pass_smem[];
+    float2* Y = reinterpret_cast<float2*>(pass_smem);
+    float2* Z = Y + Q::P * Q::PS;
+    const int64_t q0 = (int64_t)blockIdx.x * Q::P;   // pencils (kx, ky), kx fastest
+    for (int it = threadIdx.x; it < Q::P * N2; it += kCoarseThreads) {
+        const int p = it & (Q::P - 1), n2 = it >> Q::LP;
+        float2 a[N1];
+#pragma unroll
+        for (int n1 = 0; n1 < N1; ++n1) a[bitrev<Q::L1>(n1)] = A[q0 + p + (N2 * n1 + n2) * plane];
+        pass_first<N1, N2>(a, Y, p, n2, tw, twsh);
+    }
+    __syncthreads();
+    const int ky = (int)(q0 >> Q::LN);   // a block's pencils share ky (P divides n)
+    int ay;
+    float sy;
+    kfold(ky, Q::n, ay, sy);
+#pragma unroll 1
+    for (int b = 0; b < 2; ++b) {
+        for (int it = threadIdx.x; it < Q::P * N1; it += kCoarseThreads) {
+            const int p = it & (Q::P - 1), k1 = it >> Q::LP;
+            int ax;
+            float sx;
+            kfold((int)(q0 & (Q::n - 1)) + p, Q::n, ax, sx);
+            float2 a[N2];
+            pass_second<N1, N2>(a, Y, p, k1);
+            float2 w[N2];
+#pragma unroll
+            for (int k2 = 0; k2 < N2; ++k2) {
+                int az;
+                float sz;
+                kfold(k1 + N1 * k2, Q::n, az, sz);
+                const float4 g = table[((int64_t)az * h + ay) * h + ax];
+                const float2 v = a[k2];
+                float2 r;
+                if (b == 0) {   // B1 = v (S_y - i S_x)
+                    const float Sx = sx * g.x, Sy = sy * g.y;
+                    r = make_float2(v.x * Sy + v.y * Sx, v.y * Sy - v.x * Sx);
+                } else {        // B2 = -i S_z v
+                    const float Sz = sz * g.z;
+                    r = make_float2(v.y * Sz, -v.x * Sz);
+                }
+                w[bitrev<Q::L2>(k2)] = r;
+            }
+            back_first<N1, N2>(w, Z, p, k1, tw, twsh);
+        }
+        __syncthreads();
+        float2* B = b == 0 ? B1 : B2;
+        for (int it = threadIdx.x; it < Q::P * N2; it += kCoarseThreads) {
+            const int p = it & (Q::P - 1), n2 = it >> Q::LP;
+            float2 a[N1];
+            back_second<N1, N2>(a, Z, p, n2);
+#pragma unroll
+            for (int n1 = 0; n1 < N1; ++n1) B[q0 + p + (N2 * n1 + n2) * plane] = a[n1];
+        }
+        if (b == 0) __syncthreads();
+    }
+}
+
+// x: back to F_x + i F_y (blockIdx.y = 0) and F_z
+template <int N1, int N2>
+__global__ void __launch_bounds__(kCoarseThreads) k_coarse_inv_x(const float2* __restrict__ B1,
+                                                                 const float2* __restrict__ B2,
+                                                                 float* __restrict__ Fl,
+                                                                 const float2* __restrict__ tw, int twsh) {
+    using Q = Pass<N1, N2>;
+    constexpr int64_t cells = (int64_t)Q::n * Q::n * Q::n;
+    extern __shared__ __align__(16) unsigned char pass_smem[];
+    float2* Y = reinterpret_cast<float2*>(pass_smem);
+    const int64_t q0 = (int64_t)blockIdx.x * Q::P;
+    const float2* B = blockIdx.y ? B2 : B1;
+    for (int it = threadIdx.x; it < Q::P * N1; it += kCoarseThreads) {
+        const int p = it >> Q::L1, k1 = it & (N1 - 1);
+        const float2* src = B + ((q0 + p) << Q::LN) + k1;
+        float2 a[N2];
+#pragma unroll
+        for (int k2 = 0; k2 < N2; ++k2) a[bitrev<Q::L2>(k2)] = src[N1 * k2];
+        back_first<N1, N2>(a, Y, p, k1, tw, twsh);
+    }
+    __syncthreads();
+    for (int it = threadIdx.x; it < Q::P * N2; it += kCoarseThreads) {
+        const int p = it >> Q::L2, n2 = it & (N2 - 1);
+        float2 a[N1];
+        back_second<N1, N2>(a, Y, p, n2);
+        float* dst = Fl + ((q0 + p) << Q::LN) + n2;
+        if (blockIdx.y) {
+#pragma unroll
+            for (int n1 = 0; n1 < N1; ++n1) dst[2 * cells + N2 * n1] = a[n1].x;
+        } else {
+#pragma unroll
+            for (int n1 = 0; n1 < N1; ++n1) {
+                dst[N2 * n1] = a[n1].x;
+                dst[cells + N2 * n1] = a[n1].y;
+            }
+        }
+    }
+}
+
+template <int N1, int N2>
+void pass_setup() {
+    using Q = Pass<N1, N2>;
+    const int one = (int)Q::kBytes, two = 2 * one;
+    cudaFuncSetAttribute(k_coarse_fwd_x<N1, N2>, cudaFuncAttributeMaxDynamicSharedMemorySize, one);
+    cudaFuncSetAttribute(k_coarse_y<N1, N2, -1>, cudaFuncAttributeMaxDynamicSharedMemorySize, one);
+    cudaFuncSetAttribute(k_coarse_y<N1, N2, 1>, cudaFuncAttributeMaxDynamicSharedMemorySize, one);
+    cudaFuncSetAttribute(k_coarse_z<N1, N2>, cudaFuncAttributeMaxDynamicSharedMemorySize, two);
+    cudaFuncSetAttribute(k_coarse_inv_x<N1, N2>, cudaFuncAttributeMaxDynamicSharedMemorySize, one);
+}
+
+template <int N>
+void launch_tiny(Sim& s, long long mean) {
+    int twsh = 0;
+    while ((N << twsh) < s.fft_max) ++twsh;
+    k_coarse_tiny<N><<<2, N * N, 0, s.stream>>>(mean, s.rho_c, s.green_coarse, s.Fl, s.tw_f, twsh);
+    s.launches++;
+}
+void launch_small(Sim& s, long long mean) {
+    using M = SmallMesh<32>;
+    k_coarse_small<32><<<3, M::kThreads, M::kBytes, s.stream>>>(mean, s.rho_c, s.green_coarse, s.Fl);
+    s.launches++;
+}
+template <int N1, int N2>
+void launch_passes(Sim& s, long long mean) {
+    using Q = Pass<N1, N2>;
+    const unsigned groups = (unsigned)((int64_t)Q::n * Q::n / Q::P);
+    int twsh = 0;
+    while ((Q::n << twsh) < s.fft_max) ++twsh;   // W_n^e = tw[e << twsh]
+    const size_t sm = Q::kBytes;
+    k_coarse_fwd_x<N1, N2><<<groups, kCoarseThreads, sm, s.stream>>>(mean, s.rho_c, s.cA, s.tw_f, twsh);
+    k_coarse_y<N1, N2, -1><<<groups, kCoarseThreads, sm, s.stream>>>(s.cA, s.cA, s.tw_f, twsh);
+    k_coarse_z<N1, N2><<<groups, kCoarseThreads, 2 * sm, s.stream>>>(s.green_coarse, s.cA, s.cB1, s.cB2, s.tw_f, twsh);
+    k_coarse_y<N1, N2, 1><<<dim3(groups, 2), kCoarseThreads, sm, s.stream>>>(s.cB1, s.cB2, s.tw_f, twsh);
+    k_coarse_inv_x<N1, N2><<<dim3(groups, 2), kCoarseThreads, sm, s.stream>>>(s.cB1, s.cB2, s.Fl, s.tw_f, twsh);
+    s.launches += 5;
 }
 
 }  // namespace
 
-int coarse_deposit(Sim& s) {
-    cudaMemsetAsync(s.rho_c, 0, sizeof(long long) * s.ncells, s.stream);
+int coarse_deposit(Sim& s, bool cleared) {
+    if (!cleared) cudaMemsetAsync(s.rho_c, 0, sizeof(long long) * s.ncells, s.stream);
     const int nb = (s.nc / kBX) * (s.nc / kBY) * (s.nc / kBZ);
     auto k = s.pb == 2 ? k_coarse_deposit<2> : k_coarse_deposit<1>;
     k<<<nb, 256, 0, s.stream>>>(s.nc, s.counts[s.cur], s.offsets[s.cur], m_stream(s, s.cur, 0),
@@ -167,20 +639,29 @@ int coarse_deposit(Sim& s) {
     return check_launch(s, "coarse deposit");
 }
 
+void coarse_setup() {
+    cudaFuncSetAttribute(k_coarse_small<32>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)SmallMesh<32>::kBytes);
+    pass_setup<8, 8>();
+    pass_setup<8, 16>();
+    pass_setup<16, 16>();
+    pass_setup<16, 32>();
+    pass_setup<32, 32>();
+}
+
 int coarse_force(Sim& s) {
-    const int64_t nc3 = s.ncells;
-    const double mean = (double)s.n * 134217728.0 / (double)nc3;   // N 2^27 / nc^3
-    k_coarse_delta<<<grid_for(nc3, 256), 256, 0, s.stream>>>(nc3, mean, s.rho_c, s.cA);
-    s.launches++;
-    int rc = fft3d<float>(s, s.cA, s.nc, -1);
-    if (rc) return rc;
-    k_coarse_green<<<grid_for(nc3, 256), 256, 0, s.stream>>>(s.nc, s.green_coarse, s.cA, s.cB1,
-                                                            s.cB2);
-    s.launches++;
-    if ((rc = fft3d<float>(s, s.cB1, s.nc, 1))) return rc;
-    if ((rc = fft3d<float>(s, s.cB2, s.nc, 1))) return rc;
-    k_coarse_extract<<<grid_for(nc3, 256), 256, 0, s.stream>>>(nc3, s.cB1, s.cB2, s.Fl);
-    s.launches++;
+    // N 2^27 / nc^3, all powers of two (N up to 2^36)
+    const long long mean = s.n >= s.ncells ? (s.n / s.ncells) << 27 : (1ll << 27) / (s.ncells / s.n);
+    switch (s.nc) {
+        case 8: launch_tiny<8>(s, mean); break;
+        case 16: launch_tiny<16>(s, mean); break;
+        case 32: launch_small(s, mean); break;
+        case 64: launch_passes<8, 8>(s, mean); break;
+        case 128: launch_passes<8, 16>(s, mean); break;
+        case 256: launch_passes<16, 16>(s, mean); break;
+        case 512: launch_passes<16, 32>(s, mean); break;
+        case 1024: launch_passes<32, 32>(s, mean); break;
+        default: return set_error(s, PMPM_EINVAL, "coarse mesh of %d cells a side", s.nc);
+    }
     return check_launch(s, "coarse force");
 }
 

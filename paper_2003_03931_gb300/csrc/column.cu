@@ -334,7 +334,7 @@ __device__ __forceinline__ void col_fwd_x(uint32_t* row) {
         x[2 * n + 1] = u32_to_f32(r.y);
     }
     float2 X[17];
-    rfft32x2(x, X);
+    rfftx2<32, true>(x, X);
     float2* C = reinterpret_cast<float2*>(row);
     C[0] = make_float2(X[0].x, X[16].x);
 #pragma unroll
@@ -344,7 +344,7 @@ __device__ __forceinline__ void col_fwd_y(float2* col) {
     float2 a[32];
 #pragma unroll
     for (int k = 0; k < 32; ++k) a[bitrev<5>(k)] = col[qidx(0, k)];
-    fft_dit<32, -1>(a);
+    fft_dit<32, -1, true>(a);
 #pragma unroll
     for (int k = 0; k < 32; ++k) col[qidx(0, k)] = a[k];
 }
@@ -473,7 +473,7 @@ __device__ __forceinline__ void col_inv_y(int ny, float2* col) {
     float2 a[32];
 #pragma unroll
     for (int k = 0; k < 32; ++k) a[bitrev<5>(k)] = col[qidx(0, k)];
-    fft_dit<32, 1>(a);
+    fft_dit<32, 1, true>(a);
 #pragma unroll
     for (int yo = 0; yo < kTileOut; ++yo)
         if (yo < kColOutMin || ny > kColOutMin) col[qidx(0, yo)] = a[yo + kBuffer - 1];

@@ -42,7 +42,8 @@ struct Sim {
     // step buffers
     int32_t* fill = nullptr;                    // [nc^3]
     unsigned long long* S = nullptr;            // [3][nc^3] fixed-point momentum sums
-    unsigned long long* d2 = nullptr;           // [8] T = sum P^2, U = sum floor(S^2/n), 32-bit digits
+    unsigned long long* d2 = nullptr;           // [8] T = sum P^2, U = sum floor(S^2/n), 32-bit digits;
+                                                // [1] blocks done with U
     long long* rho_c = nullptr;                 // [nc^3]
     float2* cA = nullptr;                       // [nc^3] coarse spectra
     float2* cB1 = nullptr;
@@ -60,8 +61,8 @@ struct Sim {
     int64_t nblocks_scan = 0;
     double* ic_partial = nullptr;               // [3*1024 + 1] IC rms partial sums
     float* d_factors = nullptr;                 // [2 n_steps] kick, drift (codes) per step
-    int* d_step = nullptr;                      // device copy of the step counter
-    float* d_kd = nullptr;                      // [2] kick and drift factors of that step
+    int* d_step = nullptr;                      // index of the next step (k_step_begin)
+    float* d_kd = nullptr;                      // [2] kick and drift factors of the step under way
     double* pk_bins = nullptr;                  // [3][pk_max/2 + 1] power-spectrum sums
 
     // transient scratch (step, init, ICs and power spectrum share it)
@@ -117,11 +118,14 @@ template <typename R>
 int fft3d(Sim& s, void* data, int n, int sign);
 int fft_pass_count(int n);
 int coarse_force(Sim& s);             // deposit + FFT + Green -> s.Fl
-int coarse_deposit(Sim& s);           // -> s.rho_c
+int coarse_deposit(Sim& s, bool cleared = false);   // -> s.rho_c
 int tile_pass(Sim& s, int mode, float* G);
 int tile_density(Sim& s, int tile, uint32_t* d_out);   // one tile's fine box after the deposit
 void tile_setup();
 void fft_setup();
+void coarse_setup();
+// cells a thread of the scan takes (sort.cu)
+inline int scan_items(int64_t ncells) { return ncells <= (1 << 18) ? 1 : (ncells <= (1 << 24) ? 4 : 8); }
 int scan_counts(Sim& s, const int32_t* counts, int64_t* offsets);
 int encode_from_qp(Sim& s, bool counts_ready);
 int scan_and_means(Sim& s, int nxt);

@@ -69,17 +69,17 @@ PMPM_HD float2 twiddle_f(float2 d, int j, float& m) {
     return make_float2(t * d.x - d.y, t * d.y + d.x);
 }
 
-// (a, b) <- (a + w b, a - w b).  On the device both outputs are packed
-// float2 operations (one instruction for the two components, each rounded
-// as the scalar one) except for the quarter-turn twiddles, whose swapped
-// components would have to be moved first.
-template <int S>
+// (a, b) <- (a + w b, a - w b).  PACK: on the device both outputs are packed
+// float2 operations (one instruction for the two components, each rounded as
+// the scalar one) except for the quarter-turn twiddles, whose swapped components
+// would have to be moved first.
+template <int S, bool PACK>
 PMPM_HD void butterfly(float2& a, float2& b, int j) {
     float m;
     const float2 u = twiddle_f<S>(b, j, m);
     const float2 x = a;
 #ifdef __CUDA_ARCH__
-    if ((j & 15) != 8) {
+    if (PACK && (j & 15) != 8) {
         a = m == 1.f ? __fadd2_rn(x, u) : __ffma2_rn(make_float2(m, m), u, x);
         b = __ffma2_rn(make_float2(-m, -m), u, x);
         return;
@@ -91,19 +91,19 @@ PMPM_HD void butterfly(float2& a, float2& b, int j) {
 
 // One radix-2 decimation-in-time stage (span 2 HALF) of an N-point transform,
 // then the next larger span.
-template <int N, int HALF, int S>
+template <int N, int HALF, int S, bool PACK>
 struct DitStage {
     static PMPM_HD void run(float2 (&a)[N]) {
 #pragma unroll
         for (int g = 0; g < N; g += 2 * HALF) {
 #pragma unroll
-            for (int k = 0; k < HALF; ++k) butterfly<S>(a[g + k], a[g + k + HALF], k * (32 / (2 * HALF)));
+            for (int k = 0; k < HALF; ++k) butterfly<S, PACK>(a[g + k], a[g + k + HALF], k * (32 / (2 * HALF)));
         }
-        DitStage<N, 2 * HALF, S>::run(a);
+        DitStage<N, 2 * HALF, S, true>::run(a);
     }
 };
-template <int N, int S>
-struct DitStage<N, N, S> {
+template <int N, int S, bool PACK>
+struct DitStage<N, N, S, PACK> {
     static PMPM_HD void run(float2 (&)[N]) {}
 };
 
@@ -118,59 +118,68 @@ PMPM_HD int bitrev(int k) {
 // In-place unnormalised N-point DFT (N = 16 or 32) by radix-2 decimation in
 // time: on entry a[bitrev(n)] holds x[n]; on return a[k] holds
 // X[k] = sum_n x[n] exp(S 2 pi i n k / N).
-template <int N, int S>
+// FIRST: the first stage packed too.  Where the inputs are products, scalar
+// additions take them in with the multiply (one rounding less).
+template <int N, int S, bool FIRST = false>
 PMPM_HD void fft_dit(float2 (&a)[N]) {
-    DitStage<N, 1, S>::run(a);
+    DitStage<N, 1, S, FIRST>::run(a);
 }
 
-// Real 32-point forward DFT through a 16-point complex one, scaled by 2.
-// In: x[0..31] real.  Out: X[0..16] = 2 DFT(x)[0..16] (X[0], X[16] real).
-PMPM_HD void rfft32x2(const float (&x)[32], float2 (&X)[17]) {
-    float2 z[16];
+// Real N-point forward DFT (N = 8, 16 or 32) through an N/2-point complex one,
+// scaled by 2.  In: x[0..N-1] real.  Out: X[0..N/2] = 2 DFT(x)[0..N/2] (X[0],
+// X[N/2] real).
+template <int N, bool FIRST = false>
+PMPM_HD void rfftx2(const float (&x)[N], float2 (&X)[N / 2 + 1]) {
+    constexpr int H = N / 2, L = N == 32 ? 4 : (N == 16 ? 3 : 2);
+    float2 z[H];
 #pragma unroll
-    for (int m = 0; m < 16; ++m) z[bitrev<4>(m)] = make_float2(x[2 * m], x[2 * m + 1]);
-    fft_dit<16, -1>(z);
+    for (int m = 0; m < H; ++m) z[bitrev<L>(m)] = make_float2(x[2 * m], x[2 * m + 1]);
+    fft_dit<H, -1, FIRST>(z);
     X[0] = make_float2(2.f * (z[0].x + z[0].y), 0.f);
-    X[16] = make_float2(2.f * (z[0].x - z[0].y), 0.f);
-    X[8] = make_float2(2.f * z[8].x, -2.f * z[8].y);
+    X[H] = make_float2(2.f * (z[0].x - z[0].y), 0.f);
+    X[H / 2] = make_float2(2.f * z[H / 2].x, -2.f * z[H / 2].y);
 #pragma unroll
-    for (int k = 1; k < 8; ++k) {
-        const float2 Zk = z[k], Zr = z[16 - k];
+    for (int k = 1; k < H / 2; ++k) {
+        const float2 Zk = z[k], Zr = z[H - k];
         // 2E = Zk + conj Zr, 2O = -i (Zk - conj Zr); 2X[k] = 2E + w^k 2O and, as
-        // E and O at 16 - k are the conjugates, 2X[16 - k] = conj(2E - w^k 2O)
+        // E and O at H - k are the conjugates, 2X[H - k] = conj(2E - w^k 2O)
         const float2 E = make_float2(Zk.x + Zr.x, Zk.y - Zr.y);
         const float2 O = make_float2(Zk.y + Zr.y, Zr.x - Zk.x);
         float m;
-        const float2 u = twiddle_f<-1>(O, k, m);
+        const float2 u = twiddle_f<-1>(O, k * (32 / N), m);
         X[k] = make_float2(E.x + m * u.x, E.y + m * u.y);
-        X[16 - k] = make_float2(E.x - m * u.x, m * u.y - E.y);
+        X[H - k] = make_float2(E.x - m * u.x, m * u.y - E.y);
     }
 }
+PMPM_HD void rfft32x2(const float (&x)[32], float2 (&X)[17]) { rfftx2<32>(x, X); }
 
-// Inverse of the true DFT without the 1/32: x[n] = sum_k X[k] exp(+2 pi i n k/32)
-// over the Hermitian-extended spectrum.  In: X[0..16]; out: x[0..31].
-PMPM_HD void irfft32(const float2 (&X)[17], float (&x)[32]) {
-    float2 z[16];
-    // z[k] = E + i O with E = X[k] + conj X[16 - k], O = w^k (X[k] - conj X[16 - k]); E
-    // and O at 16 - k are the conjugates.  X[0] and X[16] are real.
-    z[bitrev<4>(0)] = make_float2(X[0].x + X[16].x, X[0].x - X[16].x);
-    z[bitrev<4>(8)] = make_float2(2.f * X[8].x, -2.f * X[8].y);
+// Inverse of the true DFT without the 1/N: x[n] = sum_k X[k] exp(+2 pi i n k/N)
+// over the Hermitian-extended spectrum.  In: X[0..N/2]; out: x[0..N-1].
+template <int N>
+PMPM_HD void irfft(const float2 (&X)[N / 2 + 1], float (&x)[N]) {
+    constexpr int H = N / 2, L = N == 32 ? 4 : (N == 16 ? 3 : 2);
+    float2 z[H];
+    // z[k] = E + i O with E = X[k] + conj X[H - k], O = w^k (X[k] - conj X[H - k]); E
+    // and O at H - k are the conjugates.  X[0] and X[H] are real.
+    z[bitrev<L>(0)] = make_float2(X[0].x + X[H].x, X[0].x - X[H].x);
+    z[bitrev<L>(H / 2)] = make_float2(2.f * X[H / 2].x, -2.f * X[H / 2].y);
 #pragma unroll
-    for (int k = 1; k < 8; ++k) {
+    for (int k = 1; k < H / 2; ++k) {
         const float2 Xk = X[k];
-        const float2 Xc = make_float2(X[16 - k].x, -X[16 - k].y);   // conj X[16-k]
+        const float2 Xc = make_float2(X[H - k].x, -X[H - k].y);   // conj X[H-k]
         const float2 E = cadd(Xk, Xc);
         float m;
-        const float2 u = twiddle_f<1>(csub(Xk, Xc), k, m);         // O = m u
-        z[bitrev<4>(k)] = make_float2(E.x - m * u.y, E.y + m * u.x);
-        z[bitrev<4>(16 - k)] = make_float2(E.x + m * u.y, m * u.x - E.y);
+        const float2 u = twiddle_f<1>(csub(Xk, Xc), k * (32 / N), m);   // O = m u
+        z[bitrev<L>(k)] = make_float2(E.x - m * u.y, E.y + m * u.x);
+        z[bitrev<L>(H - k)] = make_float2(E.x + m * u.y, m * u.x - E.y);
     }
-    fft_dit<16, 1>(z);
+    fft_dit<H, 1, true>(z);
 #pragma unroll
-    for (int m = 0; m < 16; ++m) {
+    for (int m = 0; m < H; ++m) {
         x[2 * m] = z[m].x;
         x[2 * m + 1] = z[m].y;
     }
 }
+PMPM_HD void irfft32(const float2 (&X)[17], float (&x)[32]) { irfft<32>(X, x); }
 
 }  // namespace pmpm

@@ -10,8 +10,7 @@
 //           rounded to 2^-24) and T = sum P^2 (128 bits): exact integers,
 //           independent of order (fused into the tile pass in a step)
 //   scan    offsets = exclusive scan of counts (int64); v_c = fl32(fl32(S)
-//           2^-24 / n)
-//   sigma   U = sum over cells of floor(S^2 / n) (128 bits); sigma =
+//           2^-24 / n); U = sum over cells of floor(S^2 / n) (128 bits); sigma =
 //           fl32(sqrt((T - U) 2^-48 / 3N)), the dispersion about the exact
 //           cell means
 //   scatter slot = offsets[c] + rank (atomic per cell); m = Q mod 256 and the
@@ -24,9 +23,9 @@ namespace pmpm {
 
 namespace {
 
+// Cells of a block: 256 threads of 1 cell (up to 64^3 cells: many SMs matter
+// more than long blocks), 4 (256^3) or 8.
 constexpr int kScanThreads = 256;
-constexpr int kScanItems = 16;
-constexpr int kScanTile = kScanThreads * kScanItems;   // 4096 cells per block
 
 __device__ __forceinline__ long long block_exclusive_scan(long long v, long long* sh, long long& total) {
     const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
@@ -55,21 +54,17 @@ __device__ __forceinline__ long long block_exclusive_scan(long long v, long long
 }
 
 __global__ void __launch_bounds__(kScanThreads) k_scan_reduce(int64_t ncells, const int32_t* __restrict__ counts,
-                                                              long long* __restrict__ blocksums) {
+                                                              long long* __restrict__ blocksums, int items) {
     __shared__ long long sh[32];
-    const int64_t b0 = (int64_t)blockIdx.x * kScanTile;
+    const int64_t b0 = (int64_t)blockIdx.x * kScanThreads * items;
     long long acc = 0;
-    for (int k = 0; k < kScanItems; ++k) {
-        const int64_t i = b0 + (int64_t)k * kScanThreads + threadIdx.x;
-        if (i < ncells) acc += counts[i];
-    }
+    for (int k = 0; k < items; ++k) acc += counts[b0 + (int64_t)k * kScanThreads + threadIdx.x];
     long long total;
     block_exclusive_scan(acc, sh, total);
     if (threadIdx.x == 0) blocksums[blockIdx.x] = total;
 }
 
-__global__ void __launch_bounds__(1024) k_scan_top(int64_t nb, long long* blocksums, int64_t n,
-                                                   int64_t* offsets_end, uint32_t* err) {
+__global__ void __launch_bounds__(1024) k_scan_top(int64_t nb, long long* blocksums) {
     __shared__ long long sh[32];
     long long carry = 0;
     for (int64_t base = 0; base < nb; base += blockDim.x) {
@@ -80,77 +75,162 @@ __global__ void __launch_bounds__(1024) k_scan_top(int64_t nb, long long* blocks
         if (i < nb) blocksums[i] = carry + ex;
         carry += total;
     }
+}
+
+// (lo, hi) of every thread of the block added to the 128-bit total held as
+// digits in dst[0..3]: a warp then a block reduction, then add128_digits
+__device__ __forceinline__ void block_add128(unsigned long long lo, unsigned long long hi,
+                                             unsigned long long* dst) {
+#pragma unroll
+    for (int o = 16; o > 0; o >>= 1) {
+        const unsigned long long l2 = __shfl_down_sync(0xffffffffu, lo, o);
+        const unsigned long long h2 = __shfl_down_sync(0xffffffffu, hi, o);
+        lo += l2;
+        hi += h2 + (lo < l2 ? 1ull : 0ull);
+    }
+    __shared__ unsigned long long shl[32], shh[32];
+    const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
+    if (lane == 0) { shl[warp] = lo; shh[warp] = hi; }
+    __syncthreads();
     if (threadIdx.x == 0) {
-        *offsets_end = carry;
-        if (carry != n) atomicOr(err, kErrCount);
+        lo = 0; hi = 0;
+        for (int w = 0; w < (int)(blockDim.x >> 5); ++w) {
+            lo += shl[w];
+            hi += shh[w] + (lo < shl[w] ? 1ull : 0ull);
+        }
+        add128_digits(dst, lo, hi);
     }
 }
 
-// One tile of kScanTile cells per block.  Global loads and stores are
-// striped (consecutive threads, consecutive cells); the scan runs over each
-// thread's kScanItems consecutive cells, and shared memory, padded by one
-// word in 16 against bank conflicts, transposes between the two orders.
+// sigma = fl32(sqrt((T - U) 2^-48 / 3N)), 2^-24 when T - U = 0 (T and U
+// from the digits d2[0..3] and d2[4..7]; Eq. 3's dispersion about the exact
+// cell means)
+__device__ float sigma_of(const unsigned long long* d2, int64_t n) {
+    unsigned long long d[8], tl, th, ul, uh;
+    for (int i = 0; i < 8; ++i) d[i] = __ldcg(d2 + i);
+    combine128(d, tl, th);
+    combine128(d + 4, ul, uh);
+    const unsigned long long lo = tl - ul;
+    const unsigned long long hi = th - uh - (tl < ul ? 1ull : 0ull);
+    if (lo == 0 && hi == 0) return kSigmaFloor;
+    const double v = __dadd_rn(__dmul_rn(__ull2double_rn(hi), 18446744073709551616.0), __ull2double_rn(lo));
+    const double s2 = __ddiv_rn(__dmul_rn(v, 0x1p-48), (double)(3 * n));
+    return __double2float_rn(__dsqrt_rn(s2));
+}
+
+// Where a block takes the particles before it from: it adds up the counts
+// itself (up to 32^3 cells), or up to kScanFew blocks' sums, or finds the prefix
+// that k_scan_top made of them.
+constexpr int kScanFew = 1024;
+constexpr int64_t kScanDirect = 32768;
+
+// One tile of kScanThreads ITEMS cells per block (the cells, at least 512 and a
+// power of two, are a multiple of it).  Global loads and stores are striped
+// (consecutive threads, consecutive cells); the scan runs over each thread's
+// ITEMS consecutive cells, and shared memory, padded by one word in 16 against
+// bank conflicts, transposes between the two orders.
+// MEANS: also the cell means v_c, zeroed slot counters, and, from the same
+// reads of counts and momentum sums S, the cell part of Eq. 3's dispersion,
+// U = sum over cells and axes of floor(S^2 / n), into the digits d2[4..7]; the
+// last block done (d2[8] counts them; none waits) writes sigma.  Scan, means and
+// dispersion of a step, with separate passes over counts and S before: 16^3
+// cells 43 -> 10 us (one launch), 64^3 46 -> 21, 256^3 625 -> 363 (of 48 B a
+// cell: 119 us at the copy bandwidth; the divisions bound it).
+template <bool MEANS, int ITEMS>
 __global__ void __launch_bounds__(kScanThreads) k_scan_apply(int64_t ncells, const int32_t* __restrict__ counts,
                                                              const long long* __restrict__ blocksums,
-                                                             int64_t* __restrict__ offsets,
+                                                             int64_t* __restrict__ offsets, int64_t n,
+                                                             uint32_t* err,
                                                              const unsigned long long* __restrict__ S,
-                                                             float* __restrict__ vc,
-                                                             int32_t* __restrict__ fill) {
+                                                             float* __restrict__ vc, int32_t* __restrict__ fill,
+                                                             unsigned long long* d2, float* __restrict__ sigma) {
+    constexpr int kTile = kScanThreads * ITEMS;
     __shared__ long long sh[32];
-    __shared__ long long buf[kScanTile + kScanTile / 16];
+    __shared__ long long buf[kTile + kTile / 16];
     int* cbuf = reinterpret_cast<int*>(buf);
-    const int64_t b0 = (int64_t)blockIdx.x * kScanTile;
+    const int64_t b0 = (int64_t)blockIdx.x * kTile;
     const int t = threadIdx.x;
-    int cst[kScanItems];
+    int cst[ITEMS];
 #pragma unroll
-    for (int k = 0; k < kScanItems; ++k) {
+    for (int k = 0; k < ITEMS; ++k) {
         const int p = k * kScanThreads + t;
-        const int64_t i = b0 + p;
-        cst[k] = i < ncells ? counts[i] : 0;
+        cst[k] = counts[b0 + p];
         cbuf[p + (p >> 4)] = cst[k];
     }
-    // slot counters and cell means, in the striped order
+    // cell means, dispersion and slot counters, in the striped order
+    unsigned long long lo = 0, hi = 0;
+    if (MEANS) {
 #pragma unroll
-    for (int k = 0; k < kScanItems; ++k) {
-        const int64_t i = b0 + k * kScanThreads + t;
-        if (i >= ncells) break;
-        if (fill) fill[i] = 0;
-        if (S) {
+        for (int k = 0; k < ITEMS; ++k) {
+            const int64_t i = b0 + k * kScanThreads + t;
+            fill[i] = 0;
+            long long s[3];
+#pragma unroll
+            for (int d = 0; d < 3; ++d) s[d] = (long long)S[d * ncells + i];
 #pragma unroll
             for (int d = 0; d < 3; ++d) {
                 float v = 0.f;
                 if (cst[k] > 0) {
-                    const float sum = __fmul_rn(__ll2float_rn((long long)S[d * ncells + i]), 0x1p-24f);
-                    v = __fdiv_rn(sum, (float)cst[k]);
+                    v = __fdiv_rn(__fmul_rn(__ll2float_rn(s[d]), 0x1p-24f), (float)cst[k]);
+                    add_square_over_n128(s[d], cst[k], lo, hi);
                 }
                 vc[d * ncells + i] = v;
             }
         }
     }
+    // the particles of the blocks before this one
+    long long base = 0;
+    if (ncells <= kScanDirect) {
+        long long part = 0;
+        for (int i = 4 * t; i < (int)b0; i += 4 * kScanThreads) {
+            const int4 c = *reinterpret_cast<const int4*>(counts + i);
+            part += (long long)c.x + c.y + c.z + c.w;
+        }
+        block_exclusive_scan(part, sh, base);
+    } else if (gridDim.x > kScanFew) {
+        base = blocksums[blockIdx.x];
+    } else {
+        long long part = 0;
+        for (int b = t; b < (int)blockIdx.x; b += kScanThreads) part += blocksums[b];
+        block_exclusive_scan(part, sh, base);
+    }
     __syncthreads();
-    int c[kScanItems];
+    int c[ITEMS];
     long long acc = 0;
 #pragma unroll
-    for (int k = 0; k < kScanItems; ++k) {
-        const int p = t * kScanItems + k;
+    for (int k = 0; k < ITEMS; ++k) {
+        const int p = t * ITEMS + k;
         c[k] = cbuf[p + (p >> 4)];
         acc += c[k];
     }
     long long total;
     // (its barriers also order the reads of cbuf before the writes to buf)
-    long long run = blocksums[blockIdx.x] + block_exclusive_scan(acc, sh, total);
+    long long run = base + block_exclusive_scan(acc, sh, total);
 #pragma unroll
-    for (int k = 0; k < kScanItems; ++k) {
-        const int p = t * kScanItems + k;
+    for (int k = 0; k < ITEMS; ++k) {
+        const int p = t * ITEMS + k;
         buf[p + (p >> 4)] = run;
         run += c[k];
     }
+    if (blockIdx.x == gridDim.x - 1 && t == 0) {
+        offsets[ncells] = base + total;
+        if (base + total != n) atomicOr(err, kErrCount);
+    }
     __syncthreads();
 #pragma unroll
-    for (int k = 0; k < kScanItems; ++k) {
+    for (int k = 0; k < ITEMS; ++k) {
         const int p = k * kScanThreads + t;
-        const int64_t i = b0 + p;
-        if (i < ncells) offsets[i] = buf[p + (p >> 4)];
+        offsets[b0 + p] = buf[p + (p >> 4)];
+    }
+    if (MEANS) {
+        block_add128(lo, hi, d2 + 4);
+        if (t == 0) {
+            __threadfence();
+            if (atomicAdd(d2 + 8, 1ull) == gridDim.x - 1) {
+                __threadfence();
+                *sigma = sigma_of(d2, n);
+            }
+        }
     }
 }
 
@@ -201,31 +281,6 @@ __device__ __forceinline__ int key3(const int32_t (&q)[3], int nc) {
     return (q[0] >> sh) + nc * ((q[1] >> sh) + nc * (q[2] >> sh));
 }
 
-// (lo, hi) of every thread of the block added to the 128-bit total held as
-// digits in dst[0..3]: a warp then a block reduction, then add128_digits
-__device__ __forceinline__ void block_add128(unsigned long long lo, unsigned long long hi,
-                                             unsigned long long* dst) {
-#pragma unroll
-    for (int o = 16; o > 0; o >>= 1) {
-        const unsigned long long l2 = __shfl_down_sync(0xffffffffu, lo, o);
-        const unsigned long long h2 = __shfl_down_sync(0xffffffffu, hi, o);
-        lo += l2;
-        hi += h2 + (lo < l2 ? 1ull : 0ull);
-    }
-    __shared__ unsigned long long shl[32], shh[32];
-    const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
-    if (lane == 0) { shl[warp] = lo; shh[warp] = hi; }
-    __syncthreads();
-    if (threadIdx.x == 0) {
-        lo = 0; hi = 0;
-        for (int w = 0; w < (int)(blockDim.x >> 5); ++w) {
-            lo += shl[w];
-            hi += shh[w] + (lo < shl[w] ? 1ull : 0ull);
-        }
-        add128_digits(dst, lo, hi);
-    }
-}
-
 // New-cell counts, fixed-point momentum sums S and the second moment
 // T = sum P^2 of Eq. 3's dispersion (digits d2[0..3]).  Each thread takes kHistIlp
 // particles at a time and issues all their loads before the atomics; the
@@ -267,52 +322,6 @@ __global__ void __launch_bounds__(256) k_hist(Src src, int64_t n, int nc, int32_
         }
     }
     block_add128(tlo, thi, d2);
-}
-
-// U = sum over cells and axes of floor(S^2 / n) into the digits d2[4..7]
-// (the cell-mean part of Eq. 3's dispersion; the new counts and sums S)
-__global__ void __launch_bounds__(256) k_cell_moment(int64_t ncells, const int32_t* __restrict__ counts,
-                                                     const unsigned long long* __restrict__ S,
-                                                     unsigned long long* d2) {
-    unsigned long long lo = 0, hi = 0;
-    for (int64_t c = blockIdx.x * (int64_t)blockDim.x + threadIdx.x; c < ncells;
-         c += (int64_t)gridDim.x * blockDim.x) {
-        const int cnt = counts[c];
-        if (cnt <= 0) continue;
-#pragma unroll
-        for (int d = 0; d < 3; ++d) add_square_over_n128((long long)S[d * ncells + c], cnt, lo, hi);
-    }
-    block_add128(lo, hi, d2 + 4);
-}
-
-// sigma = fl32(sqrt((T - U) 2^-48 / 3N)), 2^-24 when T - U = 0 (T and U
-// from the digits d2[0..3] and d2[4..7]; Eq. 3's dispersion about the exact
-// cell means)
-__global__ void k_sigma_final(const unsigned long long* d2, int64_t n, float* sigma) {
-    unsigned long long tl, th, ul, uh;
-    combine128(d2, tl, th);
-    combine128(d2 + 4, ul, uh);
-    const unsigned long long lo = tl - ul;
-    const unsigned long long hi = th - uh - (tl < ul ? 1ull : 0ull);
-    float s;
-    if (lo == 0 && hi == 0) {
-        s = kSigmaFloor;
-    } else {
-        const double v = __dadd_rn(__dmul_rn(__ull2double_rn(hi), 18446744073709551616.0),
-                                   __ull2double_rn(lo));
-        const double s2 = __ddiv_rn(__dmul_rn(v, 0x1p-48), (double)(3 * n));
-        s = __double2float_rn(__dsqrt_rn(s2));
-    }
-    *sigma = s;
-}
-
-// The dispersion after the counts, sums S and T of the new cells: U per
-// cell, then sigma of buffer nxt.
-static void finish_sigma(Sim& s, int nxt) {
-    k_cell_moment<<<grid_for(s.ncells, 256, 152 * 8), 256, 0, s.stream>>>(s.ncells, s.counts[nxt], s.S,
-                                                                           s.d2);
-    k_sigma_final<<<1, 1, 0, s.stream>>>(s.d2, s.n, s.sigma_d[nxt]);
-    s.launches += 2;
 }
 
 // Slots and Eq. 2-3 codes of two particles per lane: slot = offsets[cell] +
@@ -521,15 +530,27 @@ __global__ void k_decode(int64_t n, int nc, const int64_t* __restrict__ offsets,
 
 }  // namespace
 
-int scan_counts(Sim& s, const int32_t* counts, int64_t* offsets) {
-    const int64_t nb = (s.ncells + kScanTile - 1) / kScanTile;
-    k_scan_reduce<<<(unsigned)nb, kScanThreads, 0, s.stream>>>(s.ncells, counts, s.blocksums);
-    k_scan_top<<<1, 1024, 0, s.stream>>>(nb, s.blocksums, s.n, offsets + s.ncells, s.err);
-    k_scan_apply<<<(unsigned)nb, kScanThreads, 0, s.stream>>>(s.ncells, counts, s.blocksums, offsets,
-                                                             nullptr, nullptr, nullptr);
-    s.launches += 3;
+// Offsets of `counts`; MEANS: with the rest of k_scan_apply for buffer nxt.
+template <bool MEANS>
+static int scan(Sim& s, const int32_t* counts, int64_t* offsets, int nxt) {
+    const int items = scan_items(s.ncells);
+    const unsigned nb = (unsigned)(s.ncells / (kScanThreads * items));
+    if (s.ncells > kScanDirect) {
+        k_scan_reduce<<<nb, kScanThreads, 0, s.stream>>>(s.ncells, counts, s.blocksums, items);
+        s.launches++;
+        if (nb > kScanFew) {
+            k_scan_top<<<1, 1024, 0, s.stream>>>(nb, s.blocksums);
+            s.launches++;
+        }
+    }
+    auto k = items == 1 ? k_scan_apply<MEANS, 1> : (items == 4 ? k_scan_apply<MEANS, 4> : k_scan_apply<MEANS, 8>);
+    k<<<nb, kScanThreads, 0, s.stream>>>(s.ncells, counts, s.blocksums, offsets, s.n, s.err, s.S, s.vc[nxt], s.fill,
+                                         s.d2, s.sigma_d[nxt]);
+    s.launches++;
     return check_launch(s, "scan");
 }
+
+int scan_counts(Sim& s, const int32_t* counts, int64_t* offsets) { return scan<false>(s, counts, offsets, 0); }
 
 // Check of loaded counts on the device, before any kernel indexes the store
 // through them: every count >= 0 and their sum N.  acc[0] gathers the sum,
@@ -578,18 +599,9 @@ void check_loaded_counts(Sim& s) {
     s.launches += 2;
 }
 
-// Offsets of the new counts, zeroed slot counters, and the new cell means
-// v_c = fl32(fl32(S 2^-24) / count) of buffer nxt.
-int scan_and_means(Sim& s, int nxt) {
-    const int64_t nb = (s.ncells + kScanTile - 1) / kScanTile;
-    cudaStream_t st = s.stream;
-    k_scan_reduce<<<(unsigned)nb, kScanThreads, 0, st>>>(s.ncells, s.counts[nxt], s.blocksums);
-    k_scan_top<<<1, 1024, 0, st>>>(nb, s.blocksums, s.n, s.offsets[nxt] + s.ncells, s.err);
-    k_scan_apply<<<(unsigned)nb, kScanThreads, 0, st>>>(s.ncells, s.counts[nxt], s.blocksums,
-                                                        s.offsets[nxt], s.S, s.vc[nxt], s.fill);
-    s.launches += 3;
-    return check_launch(s, "scan");
-}
+// Offsets of the new counts, zeroed slot counters, the new cell means
+// v_c = fl32(fl32(S 2^-24) / count) of buffer nxt and its sigma (Eq. 3).
+int scan_and_means(Sim& s, int nxt) { return scan<true>(s, s.counts[nxt], s.offsets[nxt], nxt); }
 
 // Encode s.Qn / s.Pn into the other store buffer and make it current.  With
 // counts_ready the new counts and momentum sums were accumulated already
@@ -600,7 +612,7 @@ int encode_from_qp(Sim& s, bool counts_ready) {
     if (!counts_ready) {
         cudaMemsetAsync(s.counts[nxt], 0, sizeof(int32_t) * s.ncells, st);
         cudaMemsetAsync(s.S, 0, sizeof(unsigned long long) * 3 * s.ncells, st);
-        cudaMemsetAsync(s.d2, 0, 64, st);
+        cudaMemsetAsync(s.d2, 0, 72, st);
         auto kh = s.pb == 2 ? k_hist<2, QPArrays> : k_hist<1, QPArrays>;
         kh<<<grid_for(s.n, 256, 152 * 8), 256, 0, st>>>(QPArrays{s.Qn, s.Pn, s.n}, s.n, s.nc,
                                                          s.counts[nxt], s.S, s.d2, s.err);
@@ -609,8 +621,6 @@ int encode_from_qp(Sim& s, bool counts_ready) {
     int rc = scan_and_means(s, nxt);
     if (rc) return rc;
     prof_mark(s, 3);
-    finish_sigma(s, nxt);
-    prof_mark(s, 4);
     auto kc = s.pb == 2 ? k_scatter<2, QPArrays> : k_scatter<1, QPArrays>;
     kc<<<grid_for(s.n, 256), 256, 0, st>>>(QPArrays{s.Qn, s.Pn, s.n}, s.n, s.nc, s.vc[nxt],
                                            s.offsets[nxt], s.fill, s.sigma_d[nxt], s.Eedge,
@@ -636,13 +646,12 @@ int encode_from_psi(Sim& s, const double* scale) {
     lowmem_bind(s, nxt);   // S in store 0's region until the scatter writes it
     cudaMemsetAsync(s.counts[nxt], 0, sizeof(int32_t) * s.ncells, st);
     cudaMemsetAsync(s.S, 0, sizeof(unsigned long long) * 3 * s.ncells, st);
-    cudaMemsetAsync(s.d2, 0, 64, st);
+    cudaMemsetAsync(s.d2, 0, 72, st);
     k_hist<1><<<grid_for(s.n, 256, 152 * 8), 256, 0, st>>>(src, s.n, s.nc, s.counts[nxt], s.S, s.d2,
                                                            s.err);
     s.launches++;
     int rc = scan_and_means(s, nxt);
     if (rc) return rc;
-    finish_sigma(s, nxt);
     k_scatter<1><<<grid_for(s.n, 256), 256, 0, st>>>(src, s.n, s.nc, s.vc[nxt], s.offsets[nxt], s.fill,
                                                   s.sigma_d[nxt], s.Eedge, s.streams[nxt], s.err);
     s.launches += 1;
@@ -662,8 +671,6 @@ int encode_from_parked(Sim& s) {
     int rc = scan_and_means(s, nxt);
     if (rc) return rc;
     prof_mark(s, 3);
-    finish_sigma(s, nxt);
-    prof_mark(s, 4);
     const int grid = grid_for((int64_t)s.nc * s.nc, kParkThreads / 32, 152 * 4);
     k_scatter_parked<<<grid, kParkThreads, 0, s.stream>>>(
         s.n, s.nc, s.offsets[s.cur], s.streams[s.cur], s.Pn, s.d_kd, s.vc[nxt], s.offsets[nxt],

@@ -111,12 +111,13 @@ __device__ __forceinline__ void tile_body(int tile, const TileParams& P,
     __syncthreads();
 }
 
-// FP16 storage option: one CTA per tile; one fits an SM at a time (the tile
-// needs 232 KB of shared memory).  PB: bytes per position bin.
-template <int PB>
+// One CTA per tile; one fits an SM at a time (the tile needs 232 KB of shared
+// memory).  PB: bytes per position bin; CT: storage of the tile spectrum; LM: the
+// low-memory step.
+template <int PB, typename CT, bool LM = false>
 __global__ void __launch_bounds__(kTileThreads, 1) k_tile(TileParams P) {
     extern __shared__ __align__(16) unsigned char tile_smem[];
-    tile_body<false, PB, __half2>((int)blockIdx.x, P, tile_smem);
+    tile_body<LM, PB, CT>((int)blockIdx.x, P, tile_smem);
 }
 
 // One tile's fine-mesh box right after the deposit, written out in x-fastest
@@ -144,8 +145,12 @@ __global__ void __launch_bounds__(kTileThreads, 1) k_tile_density(TileParams P, 
 }
 
 void tile_setup() {
-    cudaFuncSetAttribute(k_tile<1>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)kTileSmemBytes);
-    cudaFuncSetAttribute(k_tile<2>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)kTileSmemBytes);
+    const auto smem = cudaFuncAttributeMaxDynamicSharedMemorySize;
+    cudaFuncSetAttribute(k_tile<1, float2>, smem, (int)kTileSmemBytes);
+    cudaFuncSetAttribute(k_tile<2, float2>, smem, (int)kTileSmemBytes);
+    cudaFuncSetAttribute(k_tile<1, __half2>, smem, (int)kTileSmemBytes);
+    cudaFuncSetAttribute(k_tile<2, __half2>, smem, (int)kTileSmemBytes);
+    cudaFuncSetAttribute(k_tile<1, float2, true>, smem, (int)kTileSmemBytes);
     cudaFuncSetAttribute(k_tile_density<1>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)kTileSmemBytes);
     cudaFuncSetAttribute(k_tile_density<2>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)kTileSmemBytes);
     column_setup();
@@ -189,10 +194,18 @@ int tile_pass(Sim& s, int mode, float* G) {
     // the low-memory step keeps the new momenta only (s.Pn); the new codes are
     // derived again by its re-encode
     if (s.lowmem) P.Qn = nullptr;
+    // Boxes of up to kTileCells cells a side are one wave of tiles, where the depth
+    // of walking columns does not pay: 16^3 cells are 64 CTAs and 39 us on a GB300
+    // against 42 to 50 (by how the particles cluster).  32^3 cells: 343 tiles, 125 us
+    // against 88; 64^3 cells: 607 against 413.
+    constexpr int kTileCells = 16;
     const int grid = s.nt * s.nt * s.nt;
-    if (!s.fp16) column_pass(s.stream, P, s.green_col, s.lowmem, s.pb);
-    else if (s.pb == 2) k_tile<2><<<grid, kTileThreads, kTileSmemBytes, s.stream>>>(P);
-    else k_tile<1><<<grid, kTileThreads, kTileSmemBytes, s.stream>>>(P);
+    if (!s.fp16 && s.nc > kTileCells) column_pass(s.stream, P, s.green_col, s.lowmem, s.pb);
+    else if (s.lowmem) k_tile<1, float2, true><<<grid, kTileThreads, kTileSmemBytes, s.stream>>>(P);
+    else if (s.fp16 && s.pb == 2) k_tile<2, __half2><<<grid, kTileThreads, kTileSmemBytes, s.stream>>>(P);
+    else if (s.fp16) k_tile<1, __half2><<<grid, kTileThreads, kTileSmemBytes, s.stream>>>(P);
+    else if (s.pb == 2) k_tile<2, float2><<<grid, kTileThreads, kTileSmemBytes, s.stream>>>(P);
+    else k_tile<1, float2><<<grid, kTileThreads, kTileSmemBytes, s.stream>>>(P);
     s.launches++;
     return check_launch(s, "tile pass");
 }

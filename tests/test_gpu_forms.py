@@ -1,0 +1,106 @@
+"""The coarse chain, the scan and the column pass (short-range force by walking
+columns of tiles along z) at the sizes where their forms change; for the column
+pass also the shapes where its parts change: ragged tiles of 4 and 5 cells, both
+position formats, segments of a few layers and of many, and layers with
+more particles than its tables, its first round of threads and its unchecked
+deposit take.  Bar: the force of test_gpu_force.py, 1e-4 against the oracle."""
+
+import numpy as np
+import pytest
+
+from oracle import force
+from paper_2003_03931_gb300 import synth
+from tests.gpu_util import make_sim, need_gpu, oracle_state, vector_rel_err
+
+pytestmark = pytest.mark.gpu
+
+TOL = 1e-4
+
+
+def _check(sim):
+    g = sim.fetch_force()
+    ref = force.ForceOperator(sim.cfg.nc, sim.cfg.pos_bytes).particle_force(oracle_state(sim).codes()).T
+    err = vector_rel_err(g, ref)
+    assert err <= TOL, err
+
+
+@pytest.mark.parametrize("np_,nc,tile_max,pos_bytes", [(16, 32, 5, 2), (32, 32, 5, 1), (64, 32, 4, 2), (32, 64, 5, 1)])
+def test_column_force_shapes(np_, nc, tile_max, pos_bytes):
+    need_gpu()
+    rng = np.random.default_rng(np_ + nc + tile_max)
+    sim = make_sim(np=np_, nc=nc, a_init=0.02, a_final=1.0, n_steps=4, tile_max=tile_max, pos_bytes=pos_bytes)
+    Q = synth.clustered_codes(rng, sim.cfg.n, nc, bins=256 if pos_bytes == 1 else 65536)
+    sim.load_qp(Q, synth.momenta(rng, sim.cfg.n), 0.3)
+    _check(sim)
+    sim.close()
+
+
+@pytest.mark.parametrize("in_cell", [250, 300, 5000])
+def test_column_crowded_layer(in_cell):
+    # all other particles uniform; `in_cell` share one coarse cell, one side of
+    # the limit of 255 from which every node is checked, and past the 1024
+    # particles whose cell comes from a table and the 256 of a first round
+    need_gpu()
+    nc = 32
+    rng = np.random.default_rng(in_cell)
+    sim = make_sim(np=32, nc=nc, a_init=0.02, a_final=1.0, n_steps=4)
+    Q = synth.uniform_codes(rng, sim.cfg.n, nc)
+    Q[:, :in_cell] = rng.integers(0, 256, size=(3, in_cell)) + 256 * np.array([[0], [7], [31]])
+    sim.load_qp(Q.astype(np.int32), synth.momenta(rng, sim.cfg.n), 0.3)
+    _check(sim)
+    sim.close()
+
+
+@pytest.mark.parametrize("nc", [8, 16, 32, 64])
+def test_coarse_force_chain(nc):
+    # the coarse chain's forms: one launch up to 16^3 and at 32^3 cells, five passes
+    # from 64^3; far from everything the force is the coarse mesh's alone
+    need_gpu()
+    rng = np.random.default_rng(nc)
+    sim = make_sim(np=8, nc=nc, a_init=0.02, a_final=1.0, n_steps=4)
+    sim.load_qp(synth.uniform_codes(rng, sim.cfg.n, nc), synth.momenta(rng, sim.cfg.n), 0.3)
+    _check(sim)
+    sim.close()
+
+
+@pytest.mark.parametrize("nc", [8, 32, 64, 128])
+def test_scan_of_every_form(nc):
+    # counts, offsets (through the decoded store), v_c and sigma of the one-, two-
+    # and three-launch scans, sparse and with one crowded cell
+    need_gpu()
+    rng = np.random.default_rng(nc)
+    sim = make_sim(np=32, nc=nc, a_init=0.02, a_final=1.0, n_steps=4)
+    Q = synth.clustered_codes(rng, sim.cfg.n, nc)
+    P = synth.momenta(rng, sim.cfg.n)
+    sim.load_qp(Q, P, 0.3)
+    st = oracle_state(sim)
+    cell = (Q[0] >> 8) + nc * ((Q[1] >> 8) + nc * (Q[2] >> 8).astype(np.int64))
+    np.testing.assert_array_equal(st.counts, np.bincount(cell, minlength=nc ** 3))
+    S = np.stack([np.round(P[d].astype(np.float64) * 2 ** 24).astype(np.int64) for d in range(3)])
+    sums = [np.zeros(nc ** 3, np.int64) for _ in range(3)]
+    for d in range(3):
+        np.add.at(sums[d], cell, S[d])
+    live = np.flatnonzero(st.counts)
+    U = 0
+    for d in range(3):
+        vc = (sums[d][live].astype(np.float32) * np.float32(2.0 ** -24)) / st.counts[live].astype(np.float32)
+        np.testing.assert_array_equal(st.vc[live, d], vc)
+        U += sum(int(s) ** 2 // int(c) for s, c in zip(sums[d][live], st.counts[live]))
+    T = sum(int(s) ** 2 for s in S.reshape(-1))
+    assert abs(float(st.sigma) / np.sqrt((T - U) * 2.0 ** -48 / (3 * sim.cfg.n)) - 1) < 1e-7
+    m = np.sort(st.codes().T[0]), np.sort(Q[0])
+    np.testing.assert_array_equal(*m)
+    sim.close()
+
+
+def test_column_flags_a_node_past_32_bits():
+    # 4096 particles on one node: more than 2^32 of its 2^-21 units
+    need_gpu()
+    from paper_2003_03931_gb300._lib import PMPM_EOVERFLOW, PmpmError
+    sim = make_sim(np=16, nc=32, a_init=0.1, a_final=0.5, n_steps=2)
+    Q = np.full((3, sim.cfg.n), 3 * 256 + 32, np.int32)
+    sim.load_qp(Q, np.zeros((3, sim.cfg.n), np.float32), 0.3)
+    with pytest.raises(PmpmError) as e:
+        sim.fetch_force()
+    assert e.value.code == PMPM_EOVERFLOW
+    sim.close()
