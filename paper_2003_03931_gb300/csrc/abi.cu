@@ -15,7 +15,7 @@
 
 #include <new>
 
-#include "pmpm_impl.cuh"
+#include "power.cuh"
 #include "cosmo.h"
 
 namespace pmpm {
@@ -475,6 +475,7 @@ static pmpm_sim* init_common(const pmpm_config* cfg, void* d_workspace, size_t b
     tile_setup();
     fft_setup();
     coarse_setup();
+    pk_setup();
     cudaMemsetAsync(s.err, 0, 4, s.stream);
     float T[256], E[256];
     codec_tables(T, E);

@@ -14,7 +14,7 @@
 // (k_coarse_tiny, k_coarse_small).  Larger ones take five passes over memory, the
 // ends and the Green multiply fused into them.
 #include "pmpm_impl.cuh"
-#include "regfft.cuh"
+#include "fftpass.cuh"
 
 namespace pmpm {
 
@@ -111,23 +111,9 @@ __global__ void __launch_bounds__(256) k_coarse_deposit(int nc, const int32_t* _
     }
 }
 
-__device__ __forceinline__ void kfold(int k, int nc, int& a, float& sg) {
-    if (k == 0) { a = 0; sg = 0.f; }
-    else if (k <= nc / 2) { a = k; sg = 1.f; }
-    else { a = nc - k; sg = -1.f; }
-}
-
 // fl32(rho - mean).  The mean, N 2^27 / nc^3 with powers of two, is an integer of
-// at least 8, so the difference is exact in 64 bits; two halves that float32
-// holds exactly and one multiply-add round it once.  (64-bit conversions and
-// FP64 run at 1/64 of the FP32 rate here: three per cell took 24 us of a 32^3
-// mesh on three SMs.)
-__device__ __forceinline__ float delta_of(long long rho, long long mean) {
-    const long long d = rho - mean;
-    const int hi = (int)(d >> 16);
-    if (d >= (1ll << 40) || d < -(1ll << 40)) return __ll2float_rn(d);
-    return __fmaf_rn((float)hi, 65536.f, (float)((int)d & 0xffff));
-}
+// at least 8, so the difference is exact in 64 bits.
+__device__ __forceinline__ float delta_of(long long rho, long long mean) { return f32_of(rho - mean); }
 
 // ------------------------------------------------------------ up to 16^3 cells
 // The whole chain on a complex mesh in one CTA's shared memory: blockIdx.x = 0
@@ -358,67 +344,16 @@ __global__ void __launch_bounds__(SmallMesh<N>::kThreads) k_coarse_small(long lo
 // multiplies and transforms back without another exchange.  116 bytes a cell
 // over five launches against 212 over twelve: 64^3 cells 73 -> 38 us, 128^3
 // 126 -> 72, 256^3 (HBM-bound) 710 -> 399.
-constexpr int kCoarseThreads = 256;
-constexpr int clog2(int v) { return v <= 1 ? 0 : 1 + clog2(v / 2); }
-
-template <int N1, int N2>
-struct Pass {
-    static constexpr int n = N1 * N2, L1 = clog2(N1), L2 = clog2(N2), LN = L1 + L2;
-    static constexpr int P = 4096 / n < 8 ? 8 : 4096 / n, LP = clog2(P);   // pencils of a block
-    static constexpr int RS = N2 + 1, PS = N1 * RS + 1;                    // see k_fft_pass_r
-    static constexpr size_t kBytes = sizeof(float2) * P * PS;
-};
-
-__device__ __forceinline__ float2 cmulw(float2 a, float2 w) {
-    return make_float2(a.x * w.x - a.y * w.y, a.x * w.y + a.y * w.x);
-}
-
-// N1-point step over n1 of item (p, n2), times W_n^(n2 k1), into the buffer
-template <int N1, int N2>
-__device__ __forceinline__ void pass_first(float2 (&a)[N1], float2* Y, int p, int n2, const float2* tw, int twsh) {
-    using Q = Pass<N1, N2>;
-    fft_dit<N1, -1>(a);
-#pragma unroll
-    for (int k1 = 0; k1 < N1; ++k1) Y[p * Q::PS + k1 * Q::RS + n2] = cmulw(a[k1], tw[(n2 * k1) << twsh]);
-}
-// and the N2-point step of item (p, k1) from it
-template <int N1, int N2>
-__device__ __forceinline__ void pass_second(float2 (&a)[N2], const float2* Y, int p, int k1) {
-    using Q = Pass<N1, N2>;
-#pragma unroll
-    for (int n2 = 0; n2 < N2; ++n2) a[bitrev<Q::L2>(n2)] = Y[p * Q::PS + k1 * Q::RS + n2];
-    fft_dit<N2, -1>(a);
-}
-// inverse: the N2-point step of item (p, k1) into the buffer
-template <int N1, int N2>
-__device__ __forceinline__ void back_first(float2 (&a)[N2], float2* Y, int p, int k1, const float2* tw, int twsh) {
-    using Q = Pass<N1, N2>;
-    fft_dit<N2, 1>(a);
-#pragma unroll
-    for (int n2 = 0; n2 < N2; ++n2) {
-        const float2 w = tw[(n2 * k1) << twsh];
-        Y[p * Q::PS + k1 * Q::RS + n2] = cmulw(a[n2], make_float2(w.x, -w.y));
-    }
-}
-// and the N1-point step of item (p, n2): a[n1]
-template <int N1, int N2>
-__device__ __forceinline__ void back_second(float2 (&a)[N1], const float2* Y, int p, int n2) {
-    using Q = Pass<N1, N2>;
-#pragma unroll
-    for (int k1 = 0; k1 < N1; ++k1) a[bitrev<Q::L1>(k1)] = Y[p * Q::PS + k1 * Q::RS + n2];
-    fft_dit<N1, 1>(a);
-}
-
 // x: integer density rows -> delta -> spectrum
 template <int N1, int N2>
-__global__ void __launch_bounds__(kCoarseThreads) k_coarse_fwd_x(long long mean, const long long* __restrict__ rho,
+__global__ void __launch_bounds__(kPassWidth) k_coarse_fwd_x(long long mean, const long long* __restrict__ rho,
                                                                  float2* __restrict__ out,
                                                                  const float2* __restrict__ tw, int twsh) {
     using Q = Pass<N1, N2>;
     extern __shared__ __align__(16) unsigned char pass_smem[];
     float2* Y = reinterpret_cast<float2*>(pass_smem);
     const int64_t q0 = (int64_t)blockIdx.x * Q::P;
-    for (int it = threadIdx.x; it < Q::P * N2; it += kCoarseThreads) {
+    for (int it = threadIdx.x; it < Q::P * N2; it += kPassWidth) {
         const int p = it >> Q::L2, n2 = it & (N2 - 1);
         const long long* src = rho + ((q0 + p) << Q::LN) + n2;
         float2 a[N1];
@@ -428,7 +363,7 @@ __global__ void __launch_bounds__(kCoarseThreads) k_coarse_fwd_x(long long mean,
         pass_first<N1, N2>(a, Y, p, n2, tw, twsh);
     }
     __syncthreads();
-    for (int it = threadIdx.x; it < Q::P * N1; it += kCoarseThreads) {
+    for (int it = threadIdx.x; it < Q::P * N1; it += kPassWidth) {
         const int p = it >> Q::L1, k1 = it & (N1 - 1);
         float2 a[N2];
         pass_second<N1, N2>(a, Y, p, k1);
@@ -440,7 +375,7 @@ __global__ void __launch_bounds__(kCoarseThreads) k_coarse_fwd_x(long long mean,
 
 // y: in place, forward (S = -1) or back; blockIdx.y picks the array
 template <int N1, int N2, int S>
-__global__ void __launch_bounds__(kCoarseThreads) k_coarse_y(float2* d0, float2* d1, const float2* __restrict__ tw,
+__global__ void __launch_bounds__(kPassWidth) k_coarse_y(float2* d0, float2* d1, const float2* __restrict__ tw,
                                                              int twsh) {
     using Q = Pass<N1, N2>;
     extern __shared__ __align__(16) unsigned char pass_smem[];
@@ -448,7 +383,7 @@ __global__ void __launch_bounds__(kCoarseThreads) k_coarse_y(float2* d0, float2*
     const int64_t q0 = (int64_t)blockIdx.x * Q::P;   // pencils (x, z), x fastest
     float2* data = (blockIdx.y ? d1 : d0) + ((q0 >> Q::LN) << (2 * Q::LN)) + (q0 & (Q::n - 1));
     if (S < 0) {
-        for (int it = threadIdx.x; it < Q::P * N2; it += kCoarseThreads) {
+        for (int it = threadIdx.x; it < Q::P * N2; it += kPassWidth) {
             const int p = it & (Q::P - 1), n2 = it >> Q::LP;
             float2 a[N1];
 #pragma unroll
@@ -456,7 +391,7 @@ __global__ void __launch_bounds__(kCoarseThreads) k_coarse_y(float2* d0, float2*
             pass_first<N1, N2>(a, Y, p, n2, tw, twsh);
         }
         __syncthreads();
-        for (int it = threadIdx.x; it < Q::P * N1; it += kCoarseThreads) {
+        for (int it = threadIdx.x; it < Q::P * N1; it += kPassWidth) {
             const int p = it & (Q::P - 1), k1 = it >> Q::LP;
             float2 a[N2];
             pass_second<N1, N2>(a, Y, p, k1);
@@ -464,7 +399,7 @@ __global__ void __launch_bounds__(kCoarseThreads) k_coarse_y(float2* d0, float2*
             for (int k2 = 0; k2 < N2; ++k2) data[p + ((k1 + N1 * k2) << Q::LN)] = a[k2];
         }
     } else {
-        for (int it = threadIdx.x; it < Q::P * N1; it += kCoarseThreads) {
+        for (int it = threadIdx.x; it < Q::P * N1; it += kPassWidth) {
             const int p = it & (Q::P - 1), k1 = it >> Q::LP;
             float2 a[N2];
 #pragma unroll
@@ -472,7 +407,7 @@ __global__ void __launch_bounds__(kCoarseThreads) k_coarse_y(float2* d0, float2*
             back_first<N1, N2>(a, Y, p, k1, tw, twsh);
         }
         __syncthreads();
-        for (int it = threadIdx.x; it < Q::P * N2; it += kCoarseThreads) {
+        for (int it = threadIdx.x; it < Q::P * N2; it += kPassWidth) {
             const int p = it & (Q::P - 1), n2 = it >> Q::LP;
             float2 a[N1];
             back_second<N1, N2>(a, Y, p, n2);
@@ -484,7 +419,7 @@ __global__ void __launch_bounds__(kCoarseThreads) k_coarse_y(float2* d0, float2*
 
 // z: forward, Green multiply and back for B1 and B2
 template <int N1, int N2>
-__global__ void __launch_bounds__(kCoarseThreads) k_coarse_z(const float4* __restrict__ table,
+__global__ void __launch_bounds__(kPassWidth) k_coarse_z(const float4* __restrict__ table,
                                                              const float2* __restrict__ A, float2* __restrict__ B1,
                                                              float2* __restrict__ B2, const float2* __restrict__ tw,
                                                              int twsh) {
@@ -495,7 +430,7 @@ __global__ void __launch_bounds__(kCoarseThreads) k_coarse_z(const float4* __res
     float2* Y = reinterpret_cast<float2*>(pass_smem);
     float2* Z = Y + Q::P * Q::PS;
     const int64_t q0 = (int64_t)blockIdx.x * Q::P;   // pencils (kx, ky), kx fastest
-    for (int it = threadIdx.x; it < Q::P * N2; it += kCoarseThreads) {
+    for (int it = threadIdx.x; it < Q::P * N2; it += kPassWidth) {
         const int p = it & (Q::P - 1), n2 = it >> Q::LP;
         float2 a[N1];
 #pragma unroll
@@ -509,7 +444,7 @@ __global__ void __launch_bounds__(kCoarseThreads) k_coarse_z(const float4* __res
     kfold(ky, Q::n, ay, sy);
 #pragma unroll 1
     for (int b = 0; b < 2; ++b) {
-        for (int it = threadIdx.x; it < Q::P * N1; it += kCoarseThreads) {
+        for (int it = threadIdx.x; it < Q::P * N1; it += kPassWidth) {
             const int p = it & (Q::P - 1), k1 = it >> Q::LP;
             int ax;
             float sx;
@@ -538,7 +473,7 @@ __global__ void __launch_bounds__(kCoarseThreads) k_coarse_z(const float4* __res
         }
         __syncthreads();
         float2* B = b == 0 ? B1 : B2;
-        for (int it = threadIdx.x; it < Q::P * N2; it += kCoarseThreads) {
+        for (int it = threadIdx.x; it < Q::P * N2; it += kPassWidth) {
             const int p = it & (Q::P - 1), n2 = it >> Q::LP;
             float2 a[N1];
             back_second<N1, N2>(a, Z, p, n2);
@@ -551,7 +486,7 @@ __global__ void __launch_bounds__(kCoarseThreads) k_coarse_z(const float4* __res
 
 // x: back to F_x + i F_y (blockIdx.y = 0) and F_z
 template <int N1, int N2>
-__global__ void __launch_bounds__(kCoarseThreads) k_coarse_inv_x(const float2* __restrict__ B1,
+__global__ void __launch_bounds__(kPassWidth) k_coarse_inv_x(const float2* __restrict__ B1,
                                                                  const float2* __restrict__ B2,
                                                                  float* __restrict__ Fl,
                                                                  const float2* __restrict__ tw, int twsh) {
@@ -561,7 +496,7 @@ __global__ void __launch_bounds__(kCoarseThreads) k_coarse_inv_x(const float2* _
     float2* Y = reinterpret_cast<float2*>(pass_smem);
     const int64_t q0 = (int64_t)blockIdx.x * Q::P;
     const float2* B = blockIdx.y ? B2 : B1;
-    for (int it = threadIdx.x; it < Q::P * N1; it += kCoarseThreads) {
+    for (int it = threadIdx.x; it < Q::P * N1; it += kPassWidth) {
         const int p = it >> Q::L1, k1 = it & (N1 - 1);
         const float2* src = B + ((q0 + p) << Q::LN) + k1;
         float2 a[N2];
@@ -570,7 +505,7 @@ __global__ void __launch_bounds__(kCoarseThreads) k_coarse_inv_x(const float2* _
         back_first<N1, N2>(a, Y, p, k1, tw, twsh);
     }
     __syncthreads();
-    for (int it = threadIdx.x; it < Q::P * N2; it += kCoarseThreads) {
+    for (int it = threadIdx.x; it < Q::P * N2; it += kPassWidth) {
         const int p = it >> Q::L2, n2 = it & (N2 - 1);
         float2 a[N1];
         back_second<N1, N2>(a, Y, p, n2);
@@ -618,11 +553,11 @@ void launch_passes(Sim& s, long long mean) {
     int twsh = 0;
     while ((Q::n << twsh) < s.fft_max) ++twsh;   // W_n^e = tw[e << twsh]
     const size_t sm = Q::kBytes;
-    k_coarse_fwd_x<N1, N2><<<groups, kCoarseThreads, sm, s.stream>>>(mean, s.rho_c, s.cA, s.tw_f, twsh);
-    k_coarse_y<N1, N2, -1><<<groups, kCoarseThreads, sm, s.stream>>>(s.cA, s.cA, s.tw_f, twsh);
-    k_coarse_z<N1, N2><<<groups, kCoarseThreads, 2 * sm, s.stream>>>(s.green_coarse, s.cA, s.cB1, s.cB2, s.tw_f, twsh);
-    k_coarse_y<N1, N2, 1><<<dim3(groups, 2), kCoarseThreads, sm, s.stream>>>(s.cB1, s.cB2, s.tw_f, twsh);
-    k_coarse_inv_x<N1, N2><<<dim3(groups, 2), kCoarseThreads, sm, s.stream>>>(s.cB1, s.cB2, s.Fl, s.tw_f, twsh);
+    k_coarse_fwd_x<N1, N2><<<groups, kPassWidth, sm, s.stream>>>(mean, s.rho_c, s.cA, s.tw_f, twsh);
+    k_coarse_y<N1, N2, -1><<<groups, kPassWidth, sm, s.stream>>>(s.cA, s.cA, s.tw_f, twsh);
+    k_coarse_z<N1, N2><<<groups, kPassWidth, 2 * sm, s.stream>>>(s.green_coarse, s.cA, s.cB1, s.cB2, s.tw_f, twsh);
+    k_coarse_y<N1, N2, 1><<<dim3(groups, 2), kPassWidth, sm, s.stream>>>(s.cB1, s.cB2, s.tw_f, twsh);
+    k_coarse_inv_x<N1, N2><<<dim3(groups, 2), kPassWidth, sm, s.stream>>>(s.cB1, s.cB2, s.Fl, s.tw_f, twsh);
     s.launches += 5;
 }
 

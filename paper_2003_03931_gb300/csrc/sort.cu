@@ -17,7 +17,7 @@
 //           Eq. 3 code u (Eq. 4 guess + edge fix-up) written to the new store
 // Within-cell order is not specified; every quantity above is independent of
 // it, so the encoded store is the same multiset per cell on every run.
-#include "pmpm_impl.cuh"
+#include "power.cuh"
 
 namespace pmpm {
 
@@ -530,27 +530,35 @@ __global__ void k_decode(int64_t n, int nc, const int64_t* __restrict__ offsets,
 
 }  // namespace
 
-// Offsets of `counts`; MEANS: with the rest of k_scan_apply for buffer nxt.
+// Offsets of `counts`; MEANS: with the rest of k_scan_apply.
 template <bool MEANS>
-static int scan(Sim& s, const int32_t* counts, int64_t* offsets, int nxt) {
-    const int items = scan_items(s.ncells);
-    const unsigned nb = (unsigned)(s.ncells / (kScanThreads * items));
-    if (s.ncells > kScanDirect) {
-        k_scan_reduce<<<nb, kScanThreads, 0, s.stream>>>(s.ncells, counts, s.blocksums, items);
-        s.launches++;
+static void scan(cudaStream_t st, int64_t ncells, const int32_t* counts, long long* blocksums, int64_t* offsets,
+                 int64_t n, uint32_t* err, const unsigned long long* S, float* vc, int32_t* fill,
+                 unsigned long long* d2, float* sigma, int64_t* launches) {
+    const int items = scan_items(ncells);
+    const unsigned nb = (unsigned)(ncells / (kScanThreads * items));
+    if (ncells > kScanDirect) {
+        k_scan_reduce<<<nb, kScanThreads, 0, st>>>(ncells, counts, blocksums, items);
+        *launches += 1;
         if (nb > kScanFew) {
-            k_scan_top<<<1, 1024, 0, s.stream>>>(nb, s.blocksums);
-            s.launches++;
+            k_scan_top<<<1, 1024, 0, st>>>(nb, blocksums);
+            *launches += 1;
         }
     }
     auto k = items == 1 ? k_scan_apply<MEANS, 1> : (items == 4 ? k_scan_apply<MEANS, 4> : k_scan_apply<MEANS, 8>);
-    k<<<nb, kScanThreads, 0, s.stream>>>(s.ncells, counts, s.blocksums, offsets, s.n, s.err, s.S, s.vc[nxt], s.fill,
-                                         s.d2, s.sigma_d[nxt]);
-    s.launches++;
-    return check_launch(s, "scan");
+    k<<<nb, kScanThreads, 0, st>>>(ncells, counts, blocksums, offsets, n, err, S, vc, fill, d2, sigma);
+    *launches += 1;
 }
 
-int scan_counts(Sim& s, const int32_t* counts, int64_t* offsets) { return scan<false>(s, counts, offsets, 0); }
+void scan_raw(cudaStream_t st, int64_t ncells, const int32_t* counts, long long* blocksums, int64_t* offsets,
+              int64_t n, uint32_t* err, int64_t* launches) {
+    scan<false>(st, ncells, counts, blocksums, offsets, n, err, nullptr, nullptr, nullptr, nullptr, nullptr, launches);
+}
+
+int scan_counts(Sim& s, const int32_t* counts, int64_t* offsets) {
+    scan_raw(s.stream, s.ncells, counts, s.blocksums, offsets, s.n, s.err, &s.launches);
+    return check_launch(s, "scan");
+}
 
 // Check of loaded counts on the device, before any kernel indexes the store
 // through them: every count >= 0 and their sum N.  acc[0] gathers the sum,
@@ -601,7 +609,11 @@ void check_loaded_counts(Sim& s) {
 
 // Offsets of the new counts, zeroed slot counters, the new cell means
 // v_c = fl32(fl32(S 2^-24) / count) of buffer nxt and its sigma (Eq. 3).
-int scan_and_means(Sim& s, int nxt) { return scan<true>(s, s.counts[nxt], s.offsets[nxt], nxt); }
+int scan_and_means(Sim& s, int nxt) {
+    scan<true>(s.stream, s.ncells, s.counts[nxt], s.blocksums, s.offsets[nxt], s.n, s.err, s.S, s.vc[nxt], s.fill, s.d2,
+               s.sigma_d[nxt], &s.launches);
+    return check_launch(s, "scan");
+}
 
 // Encode s.Qn / s.Pn into the other store buffer and make it current.  With
 // counts_ready the new counts and momentum sums were accumulated already

@@ -93,6 +93,77 @@ def test_scan_of_every_form(nc):
     sim.close()
 
 
+def _mean_k(nmesh, nbins, box):
+    """Mean |k| of every shell, summed exactly over the distinct |n|^2."""
+    import math
+    s = np.arange(-nmesh // 2, nmesh // 2) ** 2
+    two = np.add.outer(s, s).reshape(-1)
+    pairs = np.bincount(two)
+    many = np.zeros(pairs.size + s.max(), np.int64)
+    for v in s:
+        many[v:v + pairs.size] += pairs
+    out = []
+    for j in range(1, nbins + 1):
+        m = np.arange(j * j - j + 1, j * j + j + 1)
+        out.append(2 * math.pi / box * math.fsum(many[m] * np.sqrt(m)) / many[m].sum())
+    return np.array(out)
+
+
+@pytest.mark.parametrize("nc,nmesh,pos_bytes", [(8, 8, 1), (8, 32, 2), (16, 16, 1), (16, 32, 2), (32, 32, 1),
+                                                (16, 64, 1), (32, 64, 2), (64, 64, 1), (32, 128, 1), (64, 128, 2),
+                                                (64, 256, 1), (128, 512, 1)])
+def test_power_spectrum_forms(nc, nmesh, pos_bytes):
+    # every node spacing (1, 2 and 4 fine cells), position format and mesh form (one
+    # CTA up to 32^3, three passes from 64^3) against the oracle; a tenth of the
+    # particles in one cell
+    need_gpu()
+    from oracle import power
+    bins = 256 if pos_bytes == 1 else 65536
+    rng = np.random.default_rng(nmesh + nc)
+    sim = make_sim(np=32, nc=nc, a_init=0.02, a_final=1.0, n_steps=4, pos_bytes=pos_bytes)
+    Q = synth.clustered_codes(rng, sim.cfg.n, nc, bins=bins)
+    Q[:, :3000] = rng.integers(0, bins, size=(3, 3000)) + bins * np.array([[nc - 1], [0], [nc // 2]])
+    sim.load_qp(Q.astype(np.int32), synth.momenta(rng, sim.cfg.n), 0.3)
+    nbins = nmesh // 2 - 1
+    k, pk, nm = sim.power_spectrum(nmesh, nbins)
+    ko, po, no = power.power_spectrum(Q.T.astype(np.int64), nmesh, nbins, 4 * nc, pos_bytes=pos_bytes)
+    np.testing.assert_array_equal(nm, no)
+    # (the oracle's k is a running sum of up to 4e5 roots, itself 1e-12 off)
+    np.testing.assert_allclose(k, _mean_k(nmesh, nbins, 4.0 * nc), rtol=1e-12)
+    # float32 transforms of a field whose strongest modes lead the weakest ones
+    np.testing.assert_allclose(pk, po, rtol=1e-4, atol=1e-6 * po.max())
+    sim.close()
+
+
+@pytest.mark.parametrize("n,nc,nmesh", [(1000, 8, 32), (4097, 16, 64)])
+def test_noalloc_any_number_of_particles(n, nc, nmesh):
+    # the entry point on a caller's store takes any n, not only a sim's powers of two
+    need_gpu()
+    import ctypes
+
+    import torch
+
+    from oracle import power
+    from paper_2003_03931_gb300 import _lib
+    lib = _lib.load()
+    rng = np.random.default_rng(n)
+    Q = synth.uniform_codes(rng, n, nc)
+    cell = (Q[0] >> 8) + nc * ((Q[1] >> 8) + nc * (Q[2] >> 8).astype(np.int64))
+    Q = Q[:, np.argsort(cell, kind="stable")]
+    m = [torch.from_numpy((Q[d] & 255).astype(np.uint8)).cuda() for d in range(3)]
+    counts = torch.from_numpy(np.bincount(cell, minlength=nc ** 3).astype(np.int32)).cuda()
+    nbins = nmesh // 2
+    k, pk, nm = np.zeros(nbins), np.zeros(nbins), np.zeros(nbins, np.int64)
+    rc = lib.pmpm_power_spectrum_noalloc(nc, n, m[0].data_ptr(), m[1].data_ptr(), m[2].data_ptr(), counts.data_ptr(),
+                                         nmesh, nbins, k.ctypes.data, pk.ctypes.data, nm.ctypes.data,
+                                         ctypes.c_void_p(torch.cuda.current_stream().cuda_stream))
+    assert rc == 0, lib.pmpm_noalloc_last_error()
+    ko, po, no = power.power_spectrum(Q.T.astype(np.int64), nmesh, nbins, 4 * nc)
+    np.testing.assert_array_equal(nm, no)
+    np.testing.assert_allclose(k, ko, rtol=1e-12)
+    np.testing.assert_allclose(pk, po, rtol=1e-4, atol=1e-6 * po.max())
+
+
 def test_column_flags_a_node_past_32_bits():
     # 4096 particles on one node: more than 2^32 of its 2^-21 units
     need_gpu()
