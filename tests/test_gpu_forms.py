@@ -175,3 +175,21 @@ def test_column_flags_a_node_past_32_bits():
         sim.fetch_force()
     assert e.value.code == PMPM_EOVERFLOW
     sim.close()
+
+
+@pytest.mark.parametrize("np_,nc,pos_bytes", [(4, 8, 1), (8, 8, 2), (16, 8, 1), (32, 8, 1), (64, 32, 2), (128, 32, 1)])
+def test_initial_conditions_sizes(np_, nc, pos_bytes):
+    # every split of the float64 passes up to 128 points, against the oracle's
+    # transforms: the same cells and codes, momenta to float32 rounding
+    need_gpu()
+    from oracle import ic
+    sim = make_sim(np=np_, nc=nc, a_init=0.02, a_final=1.0, n_steps=4, pos_bytes=pos_bytes)
+    sim.ic_zeldovich(9, **synth.IC_SPECTRUM)
+    got = oracle_state(sim)
+    ref, _, _ = ic.zeldovich(9, np_, nc, 0.02, pos_bytes=pos_bytes, **synth.IC_SPECTRUM)
+    np.testing.assert_array_equal(got.counts, ref.counts)
+    for d in range(3):
+        np.testing.assert_array_equal(np.sort(got.codes().T[d]), np.sort(ref.codes().T[d]))
+    np.testing.assert_allclose(got.vc, ref.vc, rtol=1e-5, atol=1e-6 * np.abs(ref.vc).max())
+    np.testing.assert_allclose(float(got.sigma), float(ref.sigma), rtol=1e-6)
+    sim.close()
