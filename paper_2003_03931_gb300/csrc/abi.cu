@@ -279,13 +279,12 @@ __global__ void k_twiddles(int n, float2* tf, double2* td) {
     }
 }
 
+// Waits for the stream and reports the error word, one round trip.
 static int sync_and_check(Sim& s) {
-    cudaError_t e = cudaStreamSynchronize(s.stream);
-    if (e != cudaSuccess) return set_error(s, PMPM_ECUDA, "stream: %s", cudaGetErrorString(e));
     uint32_t flags = 0;
-    e = cudaMemcpyAsync(&flags, s.err, 4, cudaMemcpyDeviceToHost, s.stream);
+    cudaError_t e = cudaMemcpyAsync(&flags, s.err, 4, cudaMemcpyDeviceToHost, s.stream);
     if (e == cudaSuccess) e = cudaStreamSynchronize(s.stream);
-    if (e != cudaSuccess) return set_error(s, PMPM_ECUDA, "error word: %s", cudaGetErrorString(e));
+    if (e != cudaSuccess) return set_error(s, PMPM_ECUDA, "stream: %s", cudaGetErrorString(e));
     if (flags) {
         cudaMemsetAsync(s.err, 0, 4, s.stream);
         cudaStreamSynchronize(s.stream);
@@ -659,9 +658,10 @@ int pmpm_power_spectrum(pmpm_sim* h, int32_t nmesh, int32_t nbins, double* k, do
         s.offsets_valid = true;
     }
     s.qp_step = false;
-    int rc = power_spectrum(s, nmesh, nbins, k, pk, nmodes);
+    bool flagged = false;
+    int rc = power_spectrum(s, nmesh, nbins, k, pk, nmodes, &flagged);
     if (rc) return rc;
-    return sync_and_check(s);
+    return flagged ? sync_and_check(s) : PMPM_OK;
 }
 
 static int copy_out(Sim& s, void* dst, const void* src, size_t bytes) {
@@ -707,15 +707,15 @@ int pmpm_fetch(pmpm_sim* h, int32_t what, void* dst, size_t bytes) {
         case PMPM_SCALARS: {
             float sig = 0.f;
             cudaError_t e = cudaMemcpyAsync(&sig, s.sigma_d[s.cur], 4, cudaMemcpyDeviceToHost, s.stream);
-            if (e == cudaSuccess) e = cudaStreamSynchronize(s.stream);
             if (e != cudaSuccess) return set_error(s, PMPM_ECUDA, "fetch: %s", cudaGetErrorString(e));
+            if ((rc = sync_and_check(s))) return rc;
             pmpm_scalars sc;
             sc.a = s.a;
             sc.sigma = sig;
             sc.step = s.step;
             sc.n = s.n;
             memcpy(dst, &sc, sizeof(sc));
-            break;
+            return PMPM_OK;
         }
         case PMPM_DECODED_Q:
         case PMPM_DECODED_P:
@@ -778,6 +778,7 @@ int pmpm_load(pmpm_sim* h, int32_t what, const void* src, size_t bytes) {
     s.qp_step = false;
     const size_t N = (size_t)s.n, C = (size_t)s.ncells;
     cudaError_t e = cudaSuccess;
+    float sig = 0.f;   // (outlives its copy: the stream is waited for below)
     switch (what) {
         case PMPM_STREAMS:
             if (bytes != store_bytes(s))
@@ -815,9 +816,8 @@ int pmpm_load(pmpm_sim* h, int32_t what, const void* src, size_t bytes) {
             memcpy(&sc, src, sizeof(sc));
             if (sc.n != s.n) return set_error(s, PMPM_EINVAL, "scalars n=%lld != %lld", (long long)sc.n, (long long)s.n);
             if (sc.step < 0 || sc.step > s.cfg.n_steps) return set_error(s, PMPM_EINVAL, "scalars step");
-            const float sig = (float)sc.sigma;
+            sig = (float)sc.sigma;
             e = cudaMemcpyAsync(s.sigma_d[s.cur], &sig, 4, cudaMemcpyHostToDevice, s.stream);
-            if (e == cudaSuccess) e = cudaStreamSynchronize(s.stream);
             s.a = sc.a;
             s.step = sc.step;
             set_device_step(s, sc.step);

@@ -20,19 +20,18 @@ namespace pmpm {
 
 namespace {
 
-constexpr int kBX = 8, kBY = 8, kBZ = 4;
-constexpr int kNX = kBX + 2, kNY = kBY + 2, kNZ = kBZ + 2;
-
 // One thread per coarse cell: the cell's particles reach only the 3^3 nodes
 // around it, so their weights are summed in 27 registers and added to the
-// brick's shared accumulator once per cell.
-template <int PB>
-__global__ void __launch_bounds__(256) k_coarse_deposit(int nc, const int32_t* __restrict__ counts,
+// brick's shared accumulator once per cell.  Bricks of 8 x 8 x 4 cells; boxes up to
+// 32^3 cells take 4^3, four times the blocks (16^3 cells: 64 and not 16).
+template <int PB, int kBX, int kBY, int kBZ>
+__global__ void __launch_bounds__(kBX * kBY * kBZ) k_coarse_deposit(int nc, const int32_t* __restrict__ counts,
                                                         const int64_t* __restrict__ offsets,
                                                         const uint8_t* __restrict__ m0,
                                                         const uint8_t* __restrict__ m1,
                                                         const uint8_t* __restrict__ m2,
                                                         unsigned long long* rho) {
+    constexpr int kNX = kBX + 2, kNY = kBY + 2, kNZ = kBZ + 2;
     // the brick's node sums as 32-bit halves: a native 32-bit shared atomic on
     // the low word, and the high word counts its wraps (at most one per add)
     __shared__ uint32_t acc_lo[kNX * kNY * kNZ], acc_hi[kNX * kNY * kNZ];
@@ -565,11 +564,13 @@ void launch_passes(Sim& s, long long mean) {
 
 int coarse_deposit(Sim& s, bool cleared) {
     if (!cleared) cudaMemsetAsync(s.rho_c, 0, sizeof(long long) * s.ncells, s.stream);
-    const int nb = (s.nc / kBX) * (s.nc / kBY) * (s.nc / kBZ);
-    auto k = s.pb == 2 ? k_coarse_deposit<2> : k_coarse_deposit<1>;
-    k<<<nb, 256, 0, s.stream>>>(s.nc, s.counts[s.cur], s.offsets[s.cur], m_stream(s, s.cur, 0),
-                                m_stream(s, s.cur, 1), m_stream(s, s.cur, 2),
-                                reinterpret_cast<unsigned long long*>(s.rho_c));
+    const bool small = s.nc <= 32;
+    const unsigned nb = (unsigned)(s.ncells / (small ? 64 : 256)), threads = small ? 64 : 256;
+    auto k = s.pb == 2 ? (small ? k_coarse_deposit<2, 4, 4, 4> : k_coarse_deposit<2, 8, 8, 4>)
+                       : (small ? k_coarse_deposit<1, 4, 4, 4> : k_coarse_deposit<1, 8, 8, 4>);
+    k<<<nb, threads, 0, s.stream>>>(s.nc, s.counts[s.cur], s.offsets[s.cur], m_stream(s, s.cur, 0),
+                                    m_stream(s, s.cur, 1), m_stream(s, s.cur, 2),
+                                    reinterpret_cast<unsigned long long*>(s.rho_c));
     s.launches++;
     return check_launch(s, "coarse deposit");
 }

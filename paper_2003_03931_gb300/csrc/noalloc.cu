@@ -4,8 +4,6 @@
 // entry point serves boxes of at most kNaMaxNc coarse cells per side and
 // meshes of at most kNaMaxMesh points per side.  The computation follows
 // pmpm_power_spectrum step for step.
-#include <string.h>
-
 #include <mutex>
 
 #include "power.cuh"
@@ -20,7 +18,7 @@ constexpr int kNaMaxBins = kNaMaxMesh / 2;
 constexpr int kNaMaxDevices = 64;
 constexpr size_t kNaOffsetsBytes = 8 * ((size_t)kNaMaxNc * kNaMaxNc * kNaMaxNc + 1);
 constexpr size_t kNaMeshBytes = 8 * (size_t)kNaMaxMesh * kNaMaxMesh * kNaMaxMesh;
-constexpr size_t kNaBinsBytes = 8 * 3 * kNaMaxBins + 8;   // and the error word of the scan
+constexpr size_t kNaBinsBytes = 8 * 3 * kNaMaxBins + 16;   // and the scan's error word, twice
 constexpr size_t kNaTwBytes = 8 * kNaMaxMesh;
 constexpr size_t kA = 256;
 constexpr size_t kNaOffOffsets = 0;
@@ -105,13 +103,13 @@ extern "C" int pmpm_power_spectrum_noalloc(int32_t nc, int64_t n, const uint8_t*
     if (rc) return rc;
     int64_t* offsets = reinterpret_cast<int64_t*>(base + kNaOffOffsets);
     double* bins = reinterpret_cast<double*>(base + kNaOffBins);
-    uint32_t* err = reinterpret_cast<uint32_t*>(bins + 3 * nbins);
+    uint32_t* err = reinterpret_cast<uint32_t*>(bins + 3 * kNaMaxBins + 1);
     const int64_t ncells = (int64_t)nc * nc * nc;
     int64_t launches = 0;
     cudaMemsetAsync(err, 0, 8, st);
     scan_raw(st, ncells, d_counts, reinterpret_cast<long long*>(base + kNaOffSums), offsets, n, err, &launches);
     const PkStore store = {nc, 1, n, offsets, d_counts, {d_m0, d_m1, d_m2}};
-    cudaError_t e = pk_enqueue(st, store, nmesh, nbins, reinterpret_cast<float2*>(base + kNaOffMesh), nullptr, bins,
+    cudaError_t e = pk_enqueue(st, store, nmesh, nbins, reinterpret_cast<float2*>(base + kNaOffMesh), nullptr, bins, err,
                                reinterpret_cast<const float2*>(base + kNaOffTw), kNaMaxMesh, &launches);
     double hb[3 * kNaMaxBins + 1];
     if (e == cudaSuccess)
@@ -120,9 +118,7 @@ extern "C" int pmpm_power_spectrum_noalloc(int32_t nc, int64_t n, const uint8_t*
     if (e != cudaSuccess) return na_fail(PMPM_ECUDA, cudaGetErrorString(e));
     // counts that do not add up to n put particles in the wrong cells and the
     // mean density is wrong: refuse the result
-    uint32_t flags;
-    memcpy(&flags, hb + 3 * nbins, sizeof(flags));
-    if (flags) {
+    if (hb[3 * nbins] != 0.0) {
         long long total = -1;
         cudaMemcpyAsync(&total, offsets + ncells, sizeof(total), cudaMemcpyDeviceToHost, st);
         cudaStreamSynchronize(st);

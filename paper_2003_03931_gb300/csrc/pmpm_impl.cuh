@@ -63,7 +63,7 @@ struct Sim {
     float* d_factors = nullptr;                 // [2 n_steps] kick, drift (codes) per step
     int* d_step = nullptr;                      // index of the next step (k_step_begin)
     float* d_kd = nullptr;                      // [2] kick and drift factors of the step under way
-    double* pk_bins = nullptr;                  // [3][pk_max/2 + 1] power-spectrum sums
+    double* pk_bins = nullptr;                  // [3][nbins] power-spectrum sums, then the error word
 
     // transient scratch (step, init, ICs and power spectrum share it)
     uint8_t* scratch = nullptr;
@@ -135,11 +135,13 @@ void lowmem_bind(Sim& s, int nxt);    // low-memory layout: S and F_l in store n
 int encode_from_psi(Sim& s, const double* scale);   // low-memory ICs -> store 0
 int decode_state(Sim& s);              // -> s.Qn, s.Pn
 int ic_zeldovich(Sim& s, uint64_t seed, double slope, double kc, double rms);
-int power_spectrum(Sim& s, int nmesh, int nbins, double* k, double* pk, int64_t* nm);
+// *flagged: the error word is set (it comes back with the sums)
+int power_spectrum(Sim& s, int nmesh, int nbins, double* k, double* pk, int64_t* nm, bool* flagged);
 // The same in two halves: enqueue the kernels and an async copy of the raw
-// [3][nbins] sums into host_bins (pinned for a truly async copy), then, once
+// [3][nbins] sums, and with `word` the error word as one more double, into
+// host_bins (pinned for a truly async copy), then, once
 // the stream has reached that point, turn the sums into k, P(k), mode counts.
-int power_spectrum_enqueue(Sim& s, int nmesh, int nbins, double* host_bins);
+int power_spectrum_enqueue(Sim& s, int nmesh, int nbins, double* host_bins, bool word = false);
 void power_spectrum_finish(const double* host_bins, int nbins, double* k, double* pk, int64_t* nm);
 void prof_mark(Sim& s, int stage);     // records an event closing `stage` (-1: opening)
 void set_device_step(Sim& s, int64_t step);

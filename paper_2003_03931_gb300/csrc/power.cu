@@ -238,7 +238,9 @@ __device__ __forceinline__ void block_shell(int nmesh, int nbins, int j, double 
 }
 
 // for meshes whose shells are not the z pass's
-__global__ void __launch_bounds__(kPassWidth) k_pk_shells(int nmesh, int nbins, double kf, double* __restrict__ bins) {
+__global__ void __launch_bounds__(kPassWidth) k_pk_shells(int nmesh, int nbins, double kf, double* __restrict__ bins,
+                                                          const uint32_t* __restrict__ err) {
+    if (blockIdx.x == 0 && threadIdx.x == 0) bins[3 * nbins] = (double)*err;
     block_shell(nmesh, nbins, blockIdx.x + 1, kf, bins);
 }
 
@@ -266,13 +268,15 @@ __device__ __forceinline__ double limbs_value(uint32_t l0, uint32_t l1, uint32_t
 // x, from real deltas or in place; clears the sums that the z pass adds to
 template <int N1, int N2, bool REAL>
 __global__ void __launch_bounds__(kPassWidth) k_pk_x(const float* __restrict__ delta, float2* mesh, int nbins,
-                                                     double* __restrict__ bins, const float2* __restrict__ tw,
-                                                     int twsh) {
+                                                     double* __restrict__ bins, const uint32_t* __restrict__ err,
+                                                     const float2* __restrict__ tw, int twsh) {
     using Q = Pass<N1, N2>;
     extern __shared__ __align__(16) unsigned char pass_smem[];
     float2* Y = reinterpret_cast<float2*>(pass_smem);
-    if (blockIdx.x == 0)
+    if (blockIdx.x == 0) {
         for (int j = threadIdx.x; j < nbins; j += kPassWidth) bins[j] = 0.0;
+        if (threadIdx.x == 0) bins[3 * nbins] = (double)*err;
+    }
     const int64_t q0 = (int64_t)blockIdx.x * Q::P;
     for (int it = threadIdx.x; it < Q::P * N2; it += kPassWidth) {
         const int p = it >> Q::L2, n2 = it & (N2 - 1);
@@ -420,7 +424,8 @@ struct PkSmall {
 template <int N>
 __global__ void __launch_bounds__(PkSmall<N>::kThreads) k_pk_small(int nbins, double norm, double kf,
                                                                    const float* __restrict__ delta,
-                                                                   double* __restrict__ bins) {
+                                                                   double* __restrict__ bins,
+                                                                   const uint32_t* __restrict__ err) {
     using M = PkSmall<N>;
     constexpr int H = M::kH, P = M::kP, T = M::kThreads, L = M::kLog;
     extern __shared__ __align__(16) unsigned char pass_smem[];
@@ -429,6 +434,7 @@ __global__ void __launch_bounds__(PkSmall<N>::kThreads) k_pk_small(int nbins, do
     __shared__ uint32_t limb[3][H][H + 1];
     __shared__ float mx[32];
     const int tid = threadIdx.x;
+    if (tid == 0) bins[3 * nbins] = (double)*err;
     for (int i = tid; i < 3 * H * (H + 1); i += T) (&limb[0][0][0])[i] = 0u;
 #pragma unroll 8
     for (int i = tid; i < N * N * N; i += T) R[(i >> L) * (2 * P) + (i & (N - 1))] = delta[i];
@@ -573,22 +579,23 @@ size_t z_bytes() {
 
 template <int N1, int N2>
 void launch_transforms(cudaStream_t stream, int nbins, double norm, double kf, float2* mesh, const float* delta, double* bins,
-                       const float2* tw, int tw_n) {
+                       const uint32_t* err, const float2* tw, int tw_n) {
     using Q = Pass<N1, N2>;
     const unsigned groups = (unsigned)((int64_t)Q::n * Q::n / Q::P);
     int twsh = 0;
     while ((Q::n << twsh) < tw_n) ++twsh;
-    if (delta) k_pk_x<N1, N2, true><<<groups, kPassWidth, Q::kBytes, stream>>>(delta, mesh, nbins, bins, tw, twsh);
-    else k_pk_x<N1, N2, false><<<groups, kPassWidth, Q::kBytes, stream>>>(nullptr, mesh, nbins, bins, tw, twsh);
+    if (delta) k_pk_x<N1, N2, true><<<groups, kPassWidth, Q::kBytes, stream>>>(delta, mesh, nbins, bins, err, tw, twsh);
+    else k_pk_x<N1, N2, false><<<groups, kPassWidth, Q::kBytes, stream>>>(nullptr, mesh, nbins, bins, err, tw, twsh);
     k_pk_y<N1, N2><<<groups, kPassWidth, Q::kBytes, stream>>>(mesh, tw, twsh);
     const unsigned gz = groups < 152 * 6 ? groups : 152 * 6;
     k_pk_z<N1, N2><<<gz, kPassWidth, z_bytes<N1, N2>(), stream>>>(nbins, norm, kf, mesh, bins, tw, twsh);
 }
 
 template <int N>
-void launch_small(cudaStream_t stream, int nbins, double norm, double kf, const float* delta, double* bins) {
+void launch_small(cudaStream_t stream, int nbins, double norm, double kf, const float* delta, double* bins,
+                  const uint32_t* err) {
     using M = PkSmall<N>;
-    k_pk_small<N><<<1, M::kThreads, M::kBytes, stream>>>(nbins, norm, kf, delta, bins);
+    k_pk_small<N><<<1, M::kThreads, M::kBytes, stream>>>(nbins, norm, kf, delta, bins, err);
 }
 
 template <int N1, int N2>
@@ -618,7 +625,7 @@ void pk_setup() {
 }
 
 cudaError_t pk_enqueue(cudaStream_t stream, const PkStore& st, int nmesh, int nbins, float2* mesh, float* delta,
-                       double* bins, const float2* tw, int tw_n, int64_t* launches) {
+                       double* bins, const uint32_t* err, const float2* tw, int tw_n, int64_t* launches) {
     const int64_t m3 = (int64_t)nmesh * nmesh * nmesh;
     int lh = 0;
     while ((nmesh << lh) < 4 * st.nc) ++lh;
@@ -641,21 +648,21 @@ cudaError_t pk_enqueue(cudaStream_t stream, const PkStore& st, int nmesh, int nb
     else deposit(stream, st, lh, mean, mesh);
     *launches += 1;
     if (small) {
-        if (nmesh == 8) launch_small<8>(stream, nbins, norm, kf, real, bins);
-        else launch_small<16>(stream, nbins, norm, kf, real, bins);
+        if (nmesh == 8) launch_small<8>(stream, nbins, norm, kf, real, bins, err);
+        else launch_small<16>(stream, nbins, norm, kf, real, bins, err);
         *launches += 1;
         return cudaGetLastError();
     }
     *launches += 3;
-    if (nmesh == 32) launch_transforms<4, 8>(stream, nbins, norm, kf, mesh, real, bins, tw, tw_n);
-    else if (nmesh == 64) launch_transforms<8, 8>(stream, nbins, norm, kf, mesh, real, bins, tw, tw_n);
-    else if (nmesh == 128) launch_transforms<8, 16>(stream, nbins, norm, kf, mesh, real, bins, tw, tw_n);
-    else if (nmesh == 256) launch_transforms<16, 16>(stream, nbins, norm, kf, mesh, real, bins, tw, tw_n);
-    else if (nmesh == 512) launch_transforms<16, 32>(stream, nbins, norm, kf, mesh, real, bins, tw, tw_n);
-    else if (nmesh == 1024) launch_transforms<32, 32>(stream, nbins, norm, kf, mesh, real, bins, tw, tw_n);
+    if (nmesh == 32) launch_transforms<4, 8>(stream, nbins, norm, kf, mesh, real, bins, err, tw, tw_n);
+    else if (nmesh == 64) launch_transforms<8, 8>(stream, nbins, norm, kf, mesh, real, bins, err, tw, tw_n);
+    else if (nmesh == 128) launch_transforms<8, 16>(stream, nbins, norm, kf, mesh, real, bins, err, tw, tw_n);
+    else if (nmesh == 256) launch_transforms<16, 16>(stream, nbins, norm, kf, mesh, real, bins, err, tw, tw_n);
+    else if (nmesh == 512) launch_transforms<16, 32>(stream, nbins, norm, kf, mesh, real, bins, err, tw, tw_n);
+    else if (nmesh == 1024) launch_transforms<32, 32>(stream, nbins, norm, kf, mesh, real, bins, err, tw, tw_n);
     else {
         cudaMemsetAsync(bins, 0, sizeof(double) * nbins, stream);
-        k_pk_shells<<<nbins, kPassWidth, 0, stream>>>(nmesh, nbins, kf, bins);
+        k_pk_shells<<<nbins, kPassWidth, 0, stream>>>(nmesh, nbins, kf, bins, err);
         const cudaError_t e = fft3d_float_raw(stream, mesh, nmesh, -1, tw, tw_n);
         if (e != cudaSuccess) return e;
         k_pk_modes<<<grid_for(m3, kPassWidth, 152 * 4), kPassWidth, sizeof(double) * (nbins + 1), stream>>>(
@@ -665,7 +672,7 @@ cudaError_t pk_enqueue(cudaStream_t stream, const PkStore& st, int nmesh, int nb
     return cudaGetLastError();
 }
 
-int power_spectrum_enqueue(Sim& s, int nmesh, int nbins, double* host_bins) {
+int power_spectrum_enqueue(Sim& s, int nmesh, int nbins, double* host_bins, bool word) {
     if (nmesh < 2 || (nmesh & (nmesh - 1)) || nmesh > s.pk_max || s.nf % nmesh)
         return set_error(s, PMPM_EINVAL, "nmesh %d must be a power of two dividing %d, <= %d",
                          nmesh, s.nf, s.pk_max);
@@ -677,9 +684,9 @@ int power_spectrum_enqueue(Sim& s, int nmesh, int nbins, double* host_bins) {
     float* delta = reinterpret_cast<float*>(align_up(reinterpret_cast<uintptr_t>(mesh + m3)));
     const PkStore st = {s.nc, s.pb, s.n, s.offsets[s.cur], s.counts[s.cur],
                         {m_stream(s, s.cur, 0), m_stream(s, s.cur, 1), m_stream(s, s.cur, 2)}};
-    cudaError_t e = pk_enqueue(s.stream, st, nmesh, nbins, mesh, delta, s.pk_bins, s.tw_f, s.fft_max, &s.launches);
+    cudaError_t e = pk_enqueue(s.stream, st, nmesh, nbins, mesh, delta, s.pk_bins, s.err, s.tw_f, s.fft_max, &s.launches);
     if (e == cudaSuccess)
-        e = cudaMemcpyAsync(host_bins, s.pk_bins, sizeof(double) * 3 * nbins, cudaMemcpyDeviceToHost, s.stream);
+        e = cudaMemcpyAsync(host_bins, s.pk_bins, sizeof(double) * (3 * nbins + word), cudaMemcpyDeviceToHost, s.stream);
     if (e != cudaSuccess) return set_error(s, PMPM_ECUDA, "power spectrum: %s", cudaGetErrorString(e));
     return PMPM_OK;
 }
@@ -693,15 +700,18 @@ void power_spectrum_finish(const double* hb, int nbins, double* k, double* pk, i
     }
 }
 
-int power_spectrum(Sim& s, int nmesh, int nbins, double* k, double* pk, int64_t* nm) {
-    double* hb = new (std::nothrow) double[3 * (size_t)(nbins > 0 ? nbins : 1)];
+int power_spectrum(Sim& s, int nmesh, int nbins, double* k, double* pk, int64_t* nm, bool* flagged) {
+    double* hb = new (std::nothrow) double[3 * (size_t)(nbins > 0 ? nbins : 1) + 1];
     if (!hb) return set_error(s, PMPM_ENOMEM, "host bins");
-    int rc = power_spectrum_enqueue(s, nmesh, nbins, hb);
+    int rc = power_spectrum_enqueue(s, nmesh, nbins, hb, true);
     if (!rc) {
         const cudaError_t e = cudaStreamSynchronize(s.stream);
         if (e != cudaSuccess) rc = set_error(s, PMPM_ECUDA, "power spectrum: %s", cudaGetErrorString(e));
     }
-    if (!rc) power_spectrum_finish(hb, nbins, k, pk, nm);
+    if (!rc) {
+        power_spectrum_finish(hb, nbins, k, pk, nm);
+        *flagged = hb[3 * nbins] != 0.0;
+    }
     delete[] hb;
     return rc;
 }
