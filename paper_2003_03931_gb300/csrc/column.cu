@@ -24,11 +24,11 @@
 // whose barriers do not meet.  Register transforms take 128 registers a thread,
 // so there is no room for a third.
 //
-// What bounds it: issue (50% of the slots, 16k warp instructions a layer, 6.5k of
-// them floating point) and the waits between the three barriers of a layer;
-// memory moves 41 B a particle.  Short-range pass of a step on a GB300 against
-// the 32^3-box tiles of one CTA a SM before: 512^3 particles 36.5 -> 19.2 ms,
-// 256^3 4.57 -> 2.58 ms, 128^3 607 -> 431 us, 64^3 125 -> 98 us.
+// What bounds it: issue (49% of the slots, 16.5k warp instructions a layer, 6.3k of
+// them floating point) and the waits between the three barriers of a layer and
+// for the particles' bytes; memory moves 41 B a particle.  Short-range pass of a step on a GB300 against
+// the 32^3-box tiles of one CTA a SM before: 512^3 particles 36.5 -> 19.1 ms,
+// 256^3 4.57 -> 2.54 ms, 128^3 607 -> 404 us, 64^3 125 -> 84 us.
 #include "pmpm_impl.cuh"
 #include "tile_core.cuh"
 
@@ -416,8 +416,9 @@ __device__ __forceinline__ float2 col_pack(int lane, float2 G) {
 
 // a0, a1: the first and last two of the four new spectra; o0, o1: the planes of
 // the four new force planes likewise
-__device__ __forceinline__ void col_zsum(int warp, int lane, const float2* a0, const float2* a1, float2* o0,
-                                         float2* o1, uint32_t tm, bool emit) {
+// The new spectra's places start again as density.
+__device__ __forceinline__ void col_zsum(int warp, int lane, float2* a0, float2* a1, float2* o0, float2* o1,
+                                         uint32_t tm, bool emit) {
     constexpr int kP = kColPlane / 2, kC = kColSlots * kP;
 #pragma unroll 1
     for (int s = 0; s < 2; ++s) {
@@ -429,6 +430,7 @@ __device__ __forceinline__ void col_zsum(int warp, int lane, const float2* a0, c
         tmem_ld16(ta + 32, t + 32);
         tmem_ld8(ta + 48, t + 48);
         float2 z[4] = {a0[i], a0[kColDens / 2 + i], a1[i], a1[kColDens / 2 + i]};   // planes 4l-1 .. 4l+2
+        a0[i] = a0[kColDens / 2 + i] = a1[i] = a1[kColDens / 2 + i] = make_float2(0.f, 0.f);
         if (kx == 0)
 #pragma unroll
             for (int q = 0; q < 4; ++q) z[q] = col_unpack(lane, z[q]);
@@ -767,7 +769,7 @@ __global__ void __launch_bounds__(kColThreads, 2) k_column(const ColParams CP) {
         PMPM_MARK(1);
         // B. the sum along z
         if (fwd) {
-            const float2* const C = reinterpret_cast<const float2*>(S.A);
+            float2* const C = reinterpret_cast<float2*>(S.A);
             col_zsum(warp, lane, C + ab * (kColDens / 2), C + slot6(ab, 2) * (kColDens / 2),
                      S.O + ob * (kColPlane / 2), S.O + slot6(ob, 2) * (kColPlane / 2), tm, emit);
         }
@@ -775,9 +777,8 @@ __global__ void __launch_bounds__(kColThreads, 2) k_column(const ColParams CP) {
         PMPM_MARK(2);
         __syncthreads();
         PMPM_MARK(3);
-        // C. inverse transforms, two warps a component; the other two clear the
-        //    transformed planes; then all deposit layer l + 1, whose first particles
-        //    are loaded before the transforms
+        // C. inverse transforms, two warps a component, and deposit of layer l + 1, most of
+        //    it by the other two; its first particles are loaded before the transforms
         const int total = l <= ze ? S.halo.pre[kColHalo] : 0;
         const bool check = max(S.cmax[(l + 1) & 3], S.cmax[l & 3]) > 255;
         const int ndep = warp < 6 ? kColDepBusy : kColDepFree;
@@ -801,17 +802,6 @@ __global__ void __launch_bounds__(kColThreads, 2) k_column(const ColParams CP) {
                 }
                 PMPM_MARK(5);
             }
-            asm volatile("bar.sync 5, 256;" ::: "memory");
-        } else {
-            if (fwd) {
-#pragma unroll
-                for (int h = 0; h < 2; ++h) {
-                    uint4* z = reinterpret_cast<uint4*>(S.A + slot6(ab, 2 * (warp - 6) + h) * kColDens);
-                    for (int i = lane; i < 32 * kColPitch / 4; i += 32) z[i] = make_uint4(0u, 0u, 0u, 0u);
-                }
-            }
-            asm volatile("bar.sync 6, 64;" ::: "memory");
-            asm volatile("bar.arrive 5, 256;" ::: "memory");
         }
         PMPM_MARK(6);
         ab = slot6(ab, 4);

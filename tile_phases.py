@@ -22,7 +22,7 @@ PKG = os.path.join(ROOT, "paper_2003_03931_gb300")
 PROF_LIB = os.path.join(PKG, "_build_phases", "libpmpm_phases.so")
 
 # the intervals that the marks of k_column close, in a layer's order
-PHASES = ["forward, tables | gather", "  wait", "z sum", "  wait", "inverse y", "inverse x", "  wait | clear",
+PHASES = ["forward, tables | gather", "  wait", "z sum", "  wait", "inverse y", "inverse x", "  (deposit loads)",
           "deposit", "own loads", "  wait"]
 N_MARKS, WARPS = 12, 8
 
