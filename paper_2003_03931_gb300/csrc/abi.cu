@@ -83,6 +83,7 @@ static void derive(Sim& s, const pmpm_config* c) {
     s.nf = 4 * c->nc;
     s.n = (int64_t)c->np * c->np * c->np;
     s.ncells = (int64_t)c->nc * c->nc * c->nc;
+    s.chained = s.ncells <= kChainCells;
     s.tile_max = c->tile_max;
     s.nt = tile_count(c->nc, c->tile_max);
     s.pk_max = c->pk_mesh_max ? c->pk_mesh_max : (s.nf < 512 ? s.nf : 512);
@@ -313,6 +314,7 @@ __global__ void k_step_set(int* step, int v) { *step = v; }
 __global__ void __launch_bounds__(256) k_step_begin(int* step, float* kd, const float* factors, int n_steps,
                                                     int64_t ncells, uint4* rho, uint4* counts, uint4* S,
                                                     unsigned long long* d2) {
+    chain_begin();
     if (blockIdx.x == 0) {
         if (threadIdx.x < 9) d2[threadIdx.x] = 0;
         if (threadIdx.x == 32) {
@@ -373,9 +375,9 @@ static int enqueue_step(Sim& s) {
     int rc;
     prof_mark(s, -1);
     if (s.lowmem) lowmem_bind(s, 1 - s.cur);   // S and F_l in the next store's region
-    k_step_begin<<<grid_for(3 * s.ncells / 2, 256), 256, 0, s.stream>>>(
-        s.d_step, s.d_kd, s.d_factors, s.cfg.n_steps, s.ncells, reinterpret_cast<uint4*>(s.rho_c),
-        reinterpret_cast<uint4*>(s.counts[1 - s.cur]), reinterpret_cast<uint4*>(s.S), s.d2);
+    chain(s.chained, k_step_begin, grid_for(3 * s.ncells / 2, 256), 256, 0, s.stream, s.d_step, s.d_kd, s.d_factors,
+          s.cfg.n_steps, s.ncells, reinterpret_cast<uint4*>(s.rho_c), reinterpret_cast<uint4*>(s.counts[1 - s.cur]),
+          reinterpret_cast<uint4*>(s.S), s.d2);
     s.launches++;
     if ((rc = coarse_deposit(s, true))) return rc;
     prof_mark(s, 0);

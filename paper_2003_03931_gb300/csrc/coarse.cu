@@ -31,6 +31,7 @@ __global__ void __launch_bounds__(kBX * kBY * kBZ) k_coarse_deposit(int nc, cons
                                                         const uint8_t* __restrict__ m1,
                                                         const uint8_t* __restrict__ m2,
                                                         unsigned long long* rho) {
+    chain_begin();
     constexpr int kNX = kBX + 2, kNY = kBY + 2, kNZ = kBZ + 2;
     // the brick's node sums as 32-bit halves: a native 32-bit shared atomic on
     // the low word, and the high word counts its wraps (at most one per add)
@@ -158,6 +159,7 @@ template <int N>
 __global__ void __launch_bounds__(N * N) k_coarse_tiny(long long mean, const long long* __restrict__ rho,
                                                        const float4* __restrict__ table, float* __restrict__ Fl,
                                                        const float2* __restrict__ twiddles, int twsh) {
+    chain_wait();
     constexpr int P = N + 1, h = N / 2 + 1, cells = N * N * N;
     __shared__ float2 C[N * N * P];
     const int tid = threadIdx.x, x = tid % N, y = tid / N;   // (y, z) for the x pencils, (x, z) and (x, y)
@@ -197,6 +199,8 @@ __global__ void __launch_bounds__(N * N) k_coarse_tiny(long long mean, const lon
     __syncthreads();
     tiny_pencil<N, 1>(C + y * N * P + x, P, tw);
     __syncthreads();
+    // only now: the tile pass takes whole SMs, and its CTAs would keep other streams out
+    chain_next();
 #pragma unroll
     for (int z = 0; z < N; ++z) a[z] = col[z * (N * P)];
     autosort<N, 1>(a, tw);
@@ -239,6 +243,7 @@ template <int N>
 __global__ void __launch_bounds__(SmallMesh<N>::kThreads) k_coarse_small(long long mean, const long long* __restrict__ rho,
                                                                          const float4* __restrict__ table,
                                                                          float* __restrict__ Fl) {
+    chain_wait();
     using M = SmallMesh<N>;
     constexpr int H = M::kH, P = M::kP, T = M::kThreads, L = M::kLog;
     extern __shared__ __align__(16) unsigned char small_smem[];
@@ -332,6 +337,7 @@ __global__ void __launch_bounds__(SmallMesh<N>::kThreads) k_coarse_small(long lo
         for (int k = 0; k < H; ++k) row[k] = make_float2(0.5f * x[2 * k], 0.5f * x[2 * k + 1]);   // rfftx2 doubles
     }
     __syncthreads();
+    chain_next();
     for (int i = tid; i < N * N * N; i += T) Fl[(int64_t)comp * N * N * N + i] = R[(i >> L) * (2 * P) + (i & (N - 1))];
 }
 
@@ -348,6 +354,7 @@ template <int N1, int N2>
 __global__ void __launch_bounds__(kPassWidth) k_coarse_fwd_x(long long mean, const long long* __restrict__ rho,
                                                                  float2* __restrict__ out,
                                                                  const float2* __restrict__ tw, int twsh) {
+    chain_begin();
     using Q = Pass<N1, N2>;
     extern __shared__ __align__(16) unsigned char pass_smem[];
     float2* Y = reinterpret_cast<float2*>(pass_smem);
@@ -376,6 +383,7 @@ __global__ void __launch_bounds__(kPassWidth) k_coarse_fwd_x(long long mean, con
 template <int N1, int N2, int S>
 __global__ void __launch_bounds__(kPassWidth) k_coarse_y(float2* d0, float2* d1, const float2* __restrict__ tw,
                                                              int twsh) {
+    chain_begin();
     using Q = Pass<N1, N2>;
     extern __shared__ __align__(16) unsigned char pass_smem[];
     float2* Y = reinterpret_cast<float2*>(pass_smem);
@@ -422,6 +430,7 @@ __global__ void __launch_bounds__(kPassWidth) k_coarse_z(const float4* __restric
                                                              const float2* __restrict__ A, float2* __restrict__ B1,
                                                              float2* __restrict__ B2, const float2* __restrict__ tw,
                                                              int twsh) {
+    chain_begin();
     using Q = Pass<N1, N2>;
     constexpr int64_t plane = (int64_t)Q::n * Q::n;
     constexpr int h = Q::n / 2 + 1;
@@ -489,6 +498,7 @@ __global__ void __launch_bounds__(kPassWidth) k_coarse_inv_x(const float2* __res
                                                                  const float2* __restrict__ B2,
                                                                  float* __restrict__ Fl,
                                                                  const float2* __restrict__ tw, int twsh) {
+    chain_wait();
     using Q = Pass<N1, N2>;
     constexpr int64_t cells = (int64_t)Q::n * Q::n * Q::n;
     extern __shared__ __align__(16) unsigned char pass_smem[];
@@ -504,6 +514,7 @@ __global__ void __launch_bounds__(kPassWidth) k_coarse_inv_x(const float2* __res
         back_first<N1, N2>(a, Y, p, k1, tw, twsh);
     }
     __syncthreads();
+    chain_next();
     for (int it = threadIdx.x; it < Q::P * N2; it += kPassWidth) {
         const int p = it >> Q::L2, n2 = it & (N2 - 1);
         float2 a[N1];
@@ -537,12 +548,12 @@ template <int N>
 void launch_tiny(Sim& s, long long mean) {
     int twsh = 0;
     while ((N << twsh) < s.fft_max) ++twsh;
-    k_coarse_tiny<N><<<2, N * N, 0, s.stream>>>(mean, s.rho_c, s.green_coarse, s.Fl, s.tw_f, twsh);
+    chain(s.chained, k_coarse_tiny<N>, 2, N * N, 0, s.stream, mean, s.rho_c, s.green_coarse, s.Fl, s.tw_f, twsh);
     s.launches++;
 }
 void launch_small(Sim& s, long long mean) {
     using M = SmallMesh<32>;
-    k_coarse_small<32><<<3, M::kThreads, M::kBytes, s.stream>>>(mean, s.rho_c, s.green_coarse, s.Fl);
+    chain(s.chained, k_coarse_small<32>, 3, M::kThreads, M::kBytes, s.stream, mean, s.rho_c, s.green_coarse, s.Fl);
     s.launches++;
 }
 template <int N1, int N2>
@@ -552,11 +563,11 @@ void launch_passes(Sim& s, long long mean) {
     int twsh = 0;
     while ((Q::n << twsh) < s.fft_max) ++twsh;   // W_n^e = tw[e << twsh]
     const size_t sm = Q::kBytes;
-    k_coarse_fwd_x<N1, N2><<<groups, kPassWidth, sm, s.stream>>>(mean, s.rho_c, s.cA, s.tw_f, twsh);
-    k_coarse_y<N1, N2, -1><<<groups, kPassWidth, sm, s.stream>>>(s.cA, s.cA, s.tw_f, twsh);
-    k_coarse_z<N1, N2><<<groups, kPassWidth, 2 * sm, s.stream>>>(s.green_coarse, s.cA, s.cB1, s.cB2, s.tw_f, twsh);
-    k_coarse_y<N1, N2, 1><<<dim3(groups, 2), kPassWidth, sm, s.stream>>>(s.cB1, s.cB2, s.tw_f, twsh);
-    k_coarse_inv_x<N1, N2><<<dim3(groups, 2), kPassWidth, sm, s.stream>>>(s.cB1, s.cB2, s.Fl, s.tw_f, twsh);
+    chain(s.chained, k_coarse_fwd_x<N1, N2>, groups, kPassWidth, sm, s.stream, mean, s.rho_c, s.cA, s.tw_f, twsh);
+    chain(s.chained, k_coarse_y<N1, N2, -1>, groups, kPassWidth, sm, s.stream, s.cA, s.cA, s.tw_f, twsh);
+    chain(s.chained, k_coarse_z<N1, N2>, groups, kPassWidth, 2 * sm, s.stream, s.green_coarse, s.cA, s.cB1, s.cB2, s.tw_f, twsh);
+    chain(s.chained, k_coarse_y<N1, N2, 1>, dim3(groups, 2), kPassWidth, sm, s.stream, s.cB1, s.cB2, s.tw_f, twsh);
+    chain(s.chained, k_coarse_inv_x<N1, N2>, dim3(groups, 2), kPassWidth, sm, s.stream, s.cB1, s.cB2, s.Fl, s.tw_f, twsh);
     s.launches += 5;
 }
 
@@ -568,9 +579,9 @@ int coarse_deposit(Sim& s, bool cleared) {
     const unsigned nb = (unsigned)(s.ncells / (small ? 64 : 256)), threads = small ? 64 : 256;
     auto k = s.pb == 2 ? (small ? k_coarse_deposit<2, 4, 4, 4> : k_coarse_deposit<2, 8, 8, 4>)
                        : (small ? k_coarse_deposit<1, 4, 4, 4> : k_coarse_deposit<1, 8, 8, 4>);
-    k<<<nb, threads, 0, s.stream>>>(s.nc, s.counts[s.cur], s.offsets[s.cur], m_stream(s, s.cur, 0),
-                                    m_stream(s, s.cur, 1), m_stream(s, s.cur, 2),
-                                    reinterpret_cast<unsigned long long*>(s.rho_c));
+    chain(s.chained, k, nb, threads, 0, s.stream, s.nc, s.counts[s.cur], s.offsets[s.cur],
+          m_stream(s, s.cur, 0), m_stream(s, s.cur, 1), m_stream(s, s.cur, 2),
+          reinterpret_cast<unsigned long long*>(s.rho_c));
     s.launches++;
     return check_launch(s, "coarse deposit");
 }

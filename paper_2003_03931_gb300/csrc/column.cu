@@ -689,6 +689,7 @@ __device__ unsigned long long g_phase[8 * kMarks];
 // ------------------------------------------------------------------ the walk
 template <bool LM, int PB>
 __global__ void __launch_bounds__(kColThreads, 2) k_column(const ColParams CP) {
+    chain_begin();
     extern __shared__ __align__(16) unsigned char col_smem[];
     ColShared& S = *reinterpret_cast<ColShared*>(col_smem);
     const TileParams& P = CP.t;
@@ -895,15 +896,15 @@ static int column_layers(int nc, int nt) {
     return best;
 }
 
-void column_pass(cudaStream_t st, const TileParams& P, const float* table, bool lowmem, int pb) {
+void column_pass(cudaStream_t st, const TileParams& P, const float* table, bool lowmem, int pb, bool chained) {
     ColParams C;
     C.t = P;
     C.table = table;
     C.lz = column_layers(P.nc, P.nt);
     const unsigned grid = (unsigned)(P.nt * P.nt * ((P.nc + C.lz - 1) / C.lz));
-    if (lowmem) k_column<true, 1><<<grid, kColThreads, sizeof(ColShared), st>>>(C);
-    else if (pb == 2) k_column<false, 2><<<grid, kColThreads, sizeof(ColShared), st>>>(C);
-    else k_column<false, 1><<<grid, kColThreads, sizeof(ColShared), st>>>(C);
+    if (lowmem) chain(chained, k_column<true, 1>, grid, kColThreads, sizeof(ColShared), st, C);
+    else if (pb == 2) chain(chained, k_column<false, 2>, grid, kColThreads, sizeof(ColShared), st, C);
+    else chain(chained, k_column<false, 1>, grid, kColThreads, sizeof(ColShared), st, C);
 }
 
 }  // namespace pmpm

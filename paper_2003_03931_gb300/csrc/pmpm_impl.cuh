@@ -78,6 +78,7 @@ struct Sim {
     float* ic_psi = nullptr;                    // [3][N] float32 displacement field
 
     // captured steps, one per buffer parity
+    bool chained = false;                       // launches may overlap (chain())
     bool graphs = false;
     bool graph_ready[2] = {false, false};
     cudaGraphExec_t graph_exec[2] = {nullptr, nullptr};
@@ -103,6 +104,39 @@ inline int grid_for(int64_t n, int block, int cap = 152 * 64) {
     if (g < 1) g = 1;
     if (g > cap) g = cap;
     return (int)g;
+}
+
+// Launches a kernel; ahead: it may become resident while the stream's kernel before
+// it drains, which takes off most of the 2 us between two kernels.  For meshes of up
+// to kChainCells cells on a GPU of their own (Sim::chained): ten steps and P(k) of a
+// box of 16^3 cells 1040 -> 914 us on a GB300, a step of 32^3 cells 335 -> 327, but
+// 64^3 cells 6.27 -> 6.28 ms a run.  Among other boxes the CTAs that wait take the
+// place of theirs (sixteen served at once: 24.5 ms, 24.8 chained).
+constexpr int64_t kChainCells = 32 * 32 * 32;
+template <typename... P, typename... A>
+void chain(bool ahead, void (*kernel)(P...), dim3 grid, unsigned block, size_t smem, cudaStream_t stream, A... args) {
+    cudaLaunchAttribute attr{};
+    attr.id = cudaLaunchAttributeProgrammaticStreamSerialization;
+    attr.val.programmaticStreamSerializationAllowed = 1;
+    cudaLaunchConfig_t c{};
+    c.gridDim = grid;
+    c.blockDim = dim3(block);
+    c.dynamicSmemBytes = smem;
+    c.stream = stream;
+    c.attrs = &attr;
+    c.numAttrs = ahead ? 1 : 0;
+    cudaLaunchKernelEx(&c, kernel, static_cast<P>(args)...);
+}
+
+// First thing in a kernel launched by chain(): nothing of memory is touched before
+// the kernels before it are complete.
+__device__ __forceinline__ void chain_wait() { asm volatile("griddepcontrol.wait;" ::: "memory"); }
+// The stream's next kernel may come in, to wait.  After chain_wait(), so that a kernel
+// two places on cannot run ahead of this one.
+__device__ __forceinline__ void chain_next() { asm volatile("griddepcontrol.launch_dependents;" ::: "memory"); }
+__device__ __forceinline__ void chain_begin() {
+    chain_wait();
+    chain_next();
 }
 
 int set_error(Sim& s, int code, const char* fmt, ...);

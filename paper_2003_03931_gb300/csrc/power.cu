@@ -80,6 +80,7 @@ __device__ __forceinline__ int pk_row(const PkStore& st, int64_t base, int x, bo
 template <int PB, int LH, bool SMALL, typename OUT>
 __global__ void __launch_bounds__(Brick<LH, SMALL>::kThreads) k_pk_deposit(const PkStore st, PkMean mean,
                                                                            OUT* __restrict__ out) {
+    chain_begin();
     using B = Brick<LH, SMALL>;
     using F = PosFmt<PB>;
     constexpr int U = F::kCodesPerFine << LH, W = 2 * U, T = B::kThreads;
@@ -270,6 +271,7 @@ template <int N1, int N2, bool REAL>
 __global__ void __launch_bounds__(kPassWidth) k_pk_x(const float* __restrict__ delta, float2* mesh, int nbins,
                                                      double* __restrict__ bins, const uint32_t* __restrict__ err,
                                                      const float2* __restrict__ tw, int twsh) {
+    chain_begin();
     using Q = Pass<N1, N2>;
     extern __shared__ __align__(16) unsigned char pass_smem[];
     float2* Y = reinterpret_cast<float2*>(pass_smem);
@@ -300,6 +302,7 @@ __global__ void __launch_bounds__(kPassWidth) k_pk_x(const float* __restrict__ d
 
 template <int N1, int N2>
 __global__ void __launch_bounds__(kPassWidth) k_pk_y(float2* mesh, const float2* __restrict__ tw, int twsh) {
+    chain_begin();
     using Q = Pass<N1, N2>;
     extern __shared__ __align__(16) unsigned char pass_smem[];
     float2* Y = reinterpret_cast<float2*>(pass_smem);
@@ -342,6 +345,7 @@ __global__ void __launch_bounds__(kPassWidth) k_pk_z(int nbins, double norm, dou
                                                      const float2* __restrict__ mesh,
                                                      double* __restrict__ bins, const float2* __restrict__ tw,
                                                      int twsh) {
+    chain_begin();
     using Q = Pass<N1, N2>;
     constexpr int64_t plane = (int64_t)Q::n * Q::n;
     constexpr int h = Q::n / 2, kItems = (Q::P * N1 + kPassWidth - 1) / kPassWidth;
@@ -426,6 +430,7 @@ __global__ void __launch_bounds__(PkSmall<N>::kThreads) k_pk_small(int nbins, do
                                                                    const float* __restrict__ delta,
                                                                    double* __restrict__ bins,
                                                                    const uint32_t* __restrict__ err) {
+    chain_begin();
     using M = PkSmall<N>;
     constexpr int H = M::kH, P = M::kP, T = M::kThreads, L = M::kLog;
     extern __shared__ __align__(16) unsigned char pass_smem[];
@@ -554,7 +559,7 @@ template <int PB, int LH, bool SMALL, typename OUT>
 void launch_deposit(cudaStream_t stream, const PkStore& st, const PkMean& mean, OUT* out) {
     using B = Brick<LH, SMALL>;
     const unsigned nb = (unsigned)((st.nc / B::CX) * (st.nc / B::CY) * (st.nc / B::CZ));
-    k_pk_deposit<PB, LH, SMALL, OUT><<<nb, B::kThreads, B::kBytes, stream>>>(st, mean, out);
+    chain(st.chained, k_pk_deposit<PB, LH, SMALL, OUT>, nb, B::kThreads, B::kBytes, stream, st, mean, out);
 }
 template <int PB, bool SMALL, typename OUT>
 void deposit_of(cudaStream_t stream, const PkStore& st, int lh, const PkMean& mean, OUT* out) {
@@ -578,24 +583,28 @@ size_t z_bytes() {
 }
 
 template <int N1, int N2>
-void launch_transforms(cudaStream_t stream, int nbins, double norm, double kf, float2* mesh, const float* delta, double* bins,
-                       const uint32_t* err, const float2* tw, int tw_n) {
+void launch_transforms(cudaStream_t stream, bool chained, int nbins, double norm, double kf, float2* mesh,
+                       const float* delta, double* bins, const uint32_t* err, const float2* tw, int tw_n) {
     using Q = Pass<N1, N2>;
     const unsigned groups = (unsigned)((int64_t)Q::n * Q::n / Q::P);
+    const bool ahead = chained && (int64_t)Q::n * Q::n * Q::n <= kChainCells;
     int twsh = 0;
     while ((Q::n << twsh) < tw_n) ++twsh;
-    if (delta) k_pk_x<N1, N2, true><<<groups, kPassWidth, Q::kBytes, stream>>>(delta, mesh, nbins, bins, err, tw, twsh);
-    else k_pk_x<N1, N2, false><<<groups, kPassWidth, Q::kBytes, stream>>>(nullptr, mesh, nbins, bins, err, tw, twsh);
-    k_pk_y<N1, N2><<<groups, kPassWidth, Q::kBytes, stream>>>(mesh, tw, twsh);
+    if (delta)
+        chain(ahead, k_pk_x<N1, N2, true>, groups, kPassWidth, Q::kBytes, stream, delta, mesh, nbins, bins, err, tw, twsh);
+    else
+        chain(ahead, k_pk_x<N1, N2, false>, groups, kPassWidth, Q::kBytes, stream, nullptr, mesh, nbins, bins, err, tw,
+              twsh);
+    chain(ahead, k_pk_y<N1, N2>, groups, kPassWidth, Q::kBytes, stream, mesh, tw, twsh);
     const unsigned gz = groups < 152 * 6 ? groups : 152 * 6;
-    k_pk_z<N1, N2><<<gz, kPassWidth, z_bytes<N1, N2>(), stream>>>(nbins, norm, kf, mesh, bins, tw, twsh);
+    chain(ahead, k_pk_z<N1, N2>, gz, kPassWidth, z_bytes<N1, N2>(), stream, nbins, norm, kf, mesh, bins, tw, twsh);
 }
 
 template <int N>
-void launch_small(cudaStream_t stream, int nbins, double norm, double kf, const float* delta, double* bins,
-                  const uint32_t* err) {
+void launch_small(cudaStream_t stream, bool chained, int nbins, double norm, double kf, const float* delta,
+                  double* bins, const uint32_t* err) {
     using M = PkSmall<N>;
-    k_pk_small<N><<<1, M::kThreads, M::kBytes, stream>>>(nbins, norm, kf, delta, bins, err);
+    chain(chained, k_pk_small<N>, 1, M::kThreads, M::kBytes, stream, nbins, norm, kf, delta, bins, err);
 }
 
 template <int N1, int N2>
@@ -648,18 +657,18 @@ cudaError_t pk_enqueue(cudaStream_t stream, const PkStore& st, int nmesh, int nb
     else deposit(stream, st, lh, mean, mesh);
     *launches += 1;
     if (small) {
-        if (nmesh == 8) launch_small<8>(stream, nbins, norm, kf, real, bins, err);
-        else launch_small<16>(stream, nbins, norm, kf, real, bins, err);
+        if (nmesh == 8) launch_small<8>(stream, st.chained, nbins, norm, kf, real, bins, err);
+        else launch_small<16>(stream, st.chained, nbins, norm, kf, real, bins, err);
         *launches += 1;
         return cudaGetLastError();
     }
     *launches += 3;
-    if (nmesh == 32) launch_transforms<4, 8>(stream, nbins, norm, kf, mesh, real, bins, err, tw, tw_n);
-    else if (nmesh == 64) launch_transforms<8, 8>(stream, nbins, norm, kf, mesh, real, bins, err, tw, tw_n);
-    else if (nmesh == 128) launch_transforms<8, 16>(stream, nbins, norm, kf, mesh, real, bins, err, tw, tw_n);
-    else if (nmesh == 256) launch_transforms<16, 16>(stream, nbins, norm, kf, mesh, real, bins, err, tw, tw_n);
-    else if (nmesh == 512) launch_transforms<16, 32>(stream, nbins, norm, kf, mesh, real, bins, err, tw, tw_n);
-    else if (nmesh == 1024) launch_transforms<32, 32>(stream, nbins, norm, kf, mesh, real, bins, err, tw, tw_n);
+    if (nmesh == 32) launch_transforms<4, 8>(stream, st.chained, nbins, norm, kf, mesh, real, bins, err, tw, tw_n);
+    else if (nmesh == 64) launch_transforms<8, 8>(stream, st.chained, nbins, norm, kf, mesh, real, bins, err, tw, tw_n);
+    else if (nmesh == 128) launch_transforms<8, 16>(stream, st.chained, nbins, norm, kf, mesh, real, bins, err, tw, tw_n);
+    else if (nmesh == 256) launch_transforms<16, 16>(stream, st.chained, nbins, norm, kf, mesh, real, bins, err, tw, tw_n);
+    else if (nmesh == 512) launch_transforms<16, 32>(stream, st.chained, nbins, norm, kf, mesh, real, bins, err, tw, tw_n);
+    else if (nmesh == 1024) launch_transforms<32, 32>(stream, st.chained, nbins, norm, kf, mesh, real, bins, err, tw, tw_n);
     else {
         cudaMemsetAsync(bins, 0, sizeof(double) * nbins, stream);
         k_pk_shells<<<nbins, kPassWidth, 0, stream>>>(nmesh, nbins, kf, bins, err);
@@ -683,7 +692,7 @@ int power_spectrum_enqueue(Sim& s, int nmesh, int nbins, double* host_bins, bool
     float2* mesh = reinterpret_cast<float2*>(s.scratch);
     float* delta = reinterpret_cast<float*>(align_up(reinterpret_cast<uintptr_t>(mesh + m3)));
     const PkStore st = {s.nc, s.pb, s.n, s.offsets[s.cur], s.counts[s.cur],
-                        {m_stream(s, s.cur, 0), m_stream(s, s.cur, 1), m_stream(s, s.cur, 2)}};
+                        {m_stream(s, s.cur, 0), m_stream(s, s.cur, 1), m_stream(s, s.cur, 2)}, s.chained};
     cudaError_t e = pk_enqueue(s.stream, st, nmesh, nbins, mesh, delta, s.pk_bins, s.err, s.tw_f, s.fft_max, &s.launches);
     if (e == cudaSuccess)
         e = cudaMemcpyAsync(host_bins, s.pk_bins, sizeof(double) * (3 * nbins + word), cudaMemcpyDeviceToHost, s.stream);

@@ -12,6 +12,7 @@ struct PkStore {
     const int64_t* offsets;      // [nc^3 + 1]
     const int32_t* counts;       // [nc^3]
     const uint8_t* m[3];         // position bins, storage order
+    bool chained;                // launches may overlap (chain())
 };
 
 // Enqueues P(k) sums of `st` on an nmesh^3 mesh (a power of two from nc to 4 nc,
@@ -24,7 +25,7 @@ cudaError_t pk_enqueue(cudaStream_t stream, const PkStore& st, int nmesh, int nb
 void pk_setup();
 
 // offsets[0..nc^3] of `counts` (sort.cu); blocksums: nc^3 / 256 words
-void scan_raw(cudaStream_t stream, int64_t ncells, const int32_t* counts, long long* blocksums, int64_t* offsets,
+void scan_raw(cudaStream_t stream, bool chained, int64_t ncells, const int32_t* counts, long long* blocksums, int64_t* offsets,
               int64_t n, uint32_t* err, int64_t* launches);
 // in place, forward or back, for sizes without a fused pass (fft.cu)
 cudaError_t fft3d_float_raw(cudaStream_t st, float2* data, int n, int sign, const float2* tw, int tw_n);

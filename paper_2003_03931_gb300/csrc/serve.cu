@@ -297,6 +297,7 @@ bool admit(pmpm_batch& b, Job* j) {
         fail(b, j, rc, "init");
         return true;
     }
+    j->sim->s.chained = false;   // other boxes fill the gaps between its launches
     if (!refs) {
         b.stats.table_builds += 1;
         size_t part[3], off = 0;

@@ -55,6 +55,7 @@ __device__ __forceinline__ long long block_exclusive_scan(long long v, long long
 
 __global__ void __launch_bounds__(kScanThreads) k_scan_reduce(int64_t ncells, const int32_t* __restrict__ counts,
                                                               long long* __restrict__ blocksums, int items) {
+    chain_begin();
     __shared__ long long sh[32];
     const int64_t b0 = (int64_t)blockIdx.x * kScanThreads * items;
     long long acc = 0;
@@ -65,6 +66,7 @@ __global__ void __launch_bounds__(kScanThreads) k_scan_reduce(int64_t ncells, co
 }
 
 __global__ void __launch_bounds__(1024) k_scan_top(int64_t nb, long long* blocksums) {
+    chain_begin();
     __shared__ long long sh[32];
     long long carry = 0;
     for (int64_t base = 0; base < nb; base += blockDim.x) {
@@ -144,6 +146,7 @@ __global__ void __launch_bounds__(kScanThreads) k_scan_apply(int64_t ncells, con
                                                              const unsigned long long* __restrict__ S,
                                                              float* __restrict__ vc, int32_t* __restrict__ fill,
                                                              unsigned long long* d2, float* __restrict__ sigma) {
+    chain_begin();
     constexpr int kTile = kScanThreads * ITEMS;
     __shared__ long long sh[32];
     __shared__ long long buf[kTile + kTile / 16];
@@ -381,6 +384,7 @@ __global__ void k_scatter(Src src, int64_t n, int nc, const float* __restrict__ 
                           const int64_t* __restrict__ offsets, int32_t* fill,
                           const float* __restrict__ sigma_p, const float* __restrict__ E,
                           uint8_t* __restrict__ out, uint32_t* err) {
+    chain_begin();
     const int64_t ncells = (int64_t)nc * nc * nc;
     const float sigma = *sigma_p;
     const int lane = threadIdx.x & 31;
@@ -427,6 +431,7 @@ k_scatter_parked(int64_t n, int nc, const int64_t* __restrict__ offs_old,
                  const int64_t* __restrict__ offsets, int32_t* fill,
                  const float* __restrict__ sigma_p, const float* __restrict__ E,
                  uint8_t* __restrict__ out, uint32_t* err) {
+    chain_begin();
     __shared__ float Es[256];
     const int tid = threadIdx.x, lane = tid & 31;
     for (int k = tid; k < 256; k += kParkThreads) Es[k] = E[k];
@@ -532,31 +537,31 @@ __global__ void k_decode(int64_t n, int nc, const int64_t* __restrict__ offsets,
 
 // Offsets of `counts`; MEANS: with the rest of k_scan_apply.
 template <bool MEANS>
-static void scan(cudaStream_t st, int64_t ncells, const int32_t* counts, long long* blocksums, int64_t* offsets,
+static void scan(cudaStream_t st, bool chained, int64_t ncells, const int32_t* counts, long long* blocksums, int64_t* offsets,
                  int64_t n, uint32_t* err, const unsigned long long* S, float* vc, int32_t* fill,
                  unsigned long long* d2, float* sigma, int64_t* launches) {
     const int items = scan_items(ncells);
     const unsigned nb = (unsigned)(ncells / (kScanThreads * items));
     if (ncells > kScanDirect) {
-        k_scan_reduce<<<nb, kScanThreads, 0, st>>>(ncells, counts, blocksums, items);
+        chain(chained, k_scan_reduce, nb, kScanThreads, 0, st, ncells, counts, blocksums, items);
         *launches += 1;
         if (nb > kScanFew) {
-            k_scan_top<<<1, 1024, 0, st>>>(nb, blocksums);
+            chain(chained, k_scan_top, 1, 1024, 0, st, nb, blocksums);
             *launches += 1;
         }
     }
     auto k = items == 1 ? k_scan_apply<MEANS, 1> : (items == 4 ? k_scan_apply<MEANS, 4> : k_scan_apply<MEANS, 8>);
-    k<<<nb, kScanThreads, 0, st>>>(ncells, counts, blocksums, offsets, n, err, S, vc, fill, d2, sigma);
+    chain(chained, k, nb, kScanThreads, 0, st, ncells, counts, blocksums, offsets, n, err, S, vc, fill, d2, sigma);
     *launches += 1;
 }
 
-void scan_raw(cudaStream_t st, int64_t ncells, const int32_t* counts, long long* blocksums, int64_t* offsets,
+void scan_raw(cudaStream_t st, bool chained, int64_t ncells, const int32_t* counts, long long* blocksums, int64_t* offsets,
               int64_t n, uint32_t* err, int64_t* launches) {
-    scan<false>(st, ncells, counts, blocksums, offsets, n, err, nullptr, nullptr, nullptr, nullptr, nullptr, launches);
+    scan<false>(st, chained, ncells, counts, blocksums, offsets, n, err, nullptr, nullptr, nullptr, nullptr, nullptr, launches);
 }
 
 int scan_counts(Sim& s, const int32_t* counts, int64_t* offsets) {
-    scan_raw(s.stream, s.ncells, counts, s.blocksums, offsets, s.n, s.err, &s.launches);
+    scan_raw(s.stream, s.chained, s.ncells, counts, s.blocksums, offsets, s.n, s.err, &s.launches);
     return check_launch(s, "scan");
 }
 
@@ -610,7 +615,7 @@ void check_loaded_counts(Sim& s) {
 // Offsets of the new counts, zeroed slot counters, the new cell means
 // v_c = fl32(fl32(S 2^-24) / count) of buffer nxt and its sigma (Eq. 3).
 int scan_and_means(Sim& s, int nxt) {
-    scan<true>(s.stream, s.ncells, s.counts[nxt], s.blocksums, s.offsets[nxt], s.n, s.err, s.S, s.vc[nxt], s.fill, s.d2,
+    scan<true>(s.stream, s.chained, s.ncells, s.counts[nxt], s.blocksums, s.offsets[nxt], s.n, s.err, s.S, s.vc[nxt], s.fill, s.d2,
                s.sigma_d[nxt], &s.launches);
     return check_launch(s, "scan");
 }
@@ -634,9 +639,8 @@ int encode_from_qp(Sim& s, bool counts_ready) {
     if (rc) return rc;
     prof_mark(s, 3);
     auto kc = s.pb == 2 ? k_scatter<2, QPArrays> : k_scatter<1, QPArrays>;
-    kc<<<grid_for(s.n, 256), 256, 0, st>>>(QPArrays{s.Qn, s.Pn, s.n}, s.n, s.nc, s.vc[nxt],
-                                           s.offsets[nxt], s.fill, s.sigma_d[nxt], s.Eedge,
-                                           s.streams[nxt], s.err);
+    chain(s.chained, kc, grid_for(s.n, 256), 256, 0, st, QPArrays{s.Qn, s.Pn, s.n}, s.n, s.nc, s.vc[nxt], s.offsets[nxt],
+          s.fill, s.sigma_d[nxt], s.Eedge, s.streams[nxt], s.err);
     s.launches++;
     prof_mark(s, 5);
     s.cur = nxt;
@@ -684,9 +688,8 @@ int encode_from_parked(Sim& s) {
     if (rc) return rc;
     prof_mark(s, 3);
     const int grid = grid_for((int64_t)s.nc * s.nc, kParkThreads / 32, 152 * 4);
-    k_scatter_parked<<<grid, kParkThreads, 0, s.stream>>>(
-        s.n, s.nc, s.offsets[s.cur], s.streams[s.cur], s.Pn, s.d_kd, s.vc[nxt], s.offsets[nxt],
-        s.fill, s.sigma_d[nxt], s.Eedge, s.streams[nxt], s.err);
+    chain(s.chained, k_scatter_parked, grid, kParkThreads, 0, s.stream, s.n, s.nc, s.offsets[s.cur], s.streams[s.cur], s.Pn,
+          s.d_kd, s.vc[nxt], s.offsets[nxt], s.fill, s.sigma_d[nxt], s.Eedge, s.streams[nxt], s.err);
     s.launches++;
     prof_mark(s, 5);
     s.cur = nxt;

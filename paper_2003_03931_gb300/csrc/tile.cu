@@ -9,7 +9,7 @@
 namespace pmpm {
 
 void column_setup();
-void column_pass(cudaStream_t st, const TileParams& P, const float* table, bool lowmem, int pb);
+void column_pass(cudaStream_t st, const TileParams& P, const float* table, bool lowmem, int pb, bool chained);
 
 template <int D, bool LM, int PB, typename CT>
 __device__ __forceinline__ void tile_component(int tid, const TileGeom& g, const TileParams& P,
@@ -116,6 +116,7 @@ __device__ __forceinline__ void tile_body(int tile, const TileParams& P,
 // low-memory step.
 template <int PB, typename CT, bool LM = false>
 __global__ void __launch_bounds__(kTileThreads, 1) k_tile(TileParams P) {
+    chain_begin();
     extern __shared__ __align__(16) unsigned char tile_smem[];
     tile_body<LM, PB, CT>((int)blockIdx.x, P, tile_smem);
 }
@@ -200,12 +201,12 @@ int tile_pass(Sim& s, int mode, float* G) {
     // against 88; 64^3 cells: 607 against 413.
     constexpr int kTileCells = 16;
     const int grid = s.nt * s.nt * s.nt;
-    if (!s.fp16 && s.nc > kTileCells) column_pass(s.stream, P, s.green_col, s.lowmem, s.pb);
-    else if (s.lowmem) k_tile<1, float2, true><<<grid, kTileThreads, kTileSmemBytes, s.stream>>>(P);
-    else if (s.fp16 && s.pb == 2) k_tile<2, __half2><<<grid, kTileThreads, kTileSmemBytes, s.stream>>>(P);
-    else if (s.fp16) k_tile<1, __half2><<<grid, kTileThreads, kTileSmemBytes, s.stream>>>(P);
-    else if (s.pb == 2) k_tile<2, float2><<<grid, kTileThreads, kTileSmemBytes, s.stream>>>(P);
-    else k_tile<1, float2><<<grid, kTileThreads, kTileSmemBytes, s.stream>>>(P);
+    if (!s.fp16 && s.nc > kTileCells) column_pass(s.stream, P, s.green_col, s.lowmem, s.pb, s.chained);
+    else if (s.lowmem) chain(s.chained, k_tile<1, float2, true>, grid, kTileThreads, kTileSmemBytes, s.stream, P);
+    else if (s.fp16 && s.pb == 2) chain(s.chained, k_tile<2, __half2>, grid, kTileThreads, kTileSmemBytes, s.stream, P);
+    else if (s.fp16) chain(s.chained, k_tile<1, __half2>, grid, kTileThreads, kTileSmemBytes, s.stream, P);
+    else if (s.pb == 2) chain(s.chained, k_tile<2, float2>, grid, kTileThreads, kTileSmemBytes, s.stream, P);
+    else chain(s.chained, k_tile<1, float2>, grid, kTileThreads, kTileSmemBytes, s.stream, P);
     s.launches++;
     return check_launch(s, "tile pass");
 }
