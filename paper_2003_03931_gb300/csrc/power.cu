@@ -14,10 +14,11 @@
 // FP64 runs at 1/64 of the FP32 rate here, so shell sums are exact integers of
 // 21-bit limbs of the float32 squares, and only a block's totals become doubles.
 //
-// On a GB300: 256^3 particles on 512^3 points 10.5 -> 1.95 ms (a search per
+// On a GB300: 256^3 particles on 512^3 points 10.5 -> 1.47 ms (a search per
 // particle, 64-bit global atomics and three double shared atomics a mode before):
-// deposit 0.65, x 0.27, y 0.43, z with the shells 0.54, of 0.8 ms for 40 bytes a
-// point at the copy bandwidth; 32^3 on 32^3, without allocation, 115 -> 76 us.
+// deposit 0.65 (shared atomics), x 0.21, y 0.21, z with the shells 0.34, of 0.48 ms for
+// 24 bytes a point at the copy bandwidth (1.95 ms with planes of their own, 40 bytes);
+// 32^3 on 32^3, without allocation, 115 -> 70 us.
 #include "power.cuh"
 
 #include <new>
@@ -266,10 +267,13 @@ __device__ __forceinline__ double limbs_value(uint32_t l0, uint32_t l1, uint32_t
 }
 
 // ------------------------------------------------------------ transforms
-// x, from real deltas or in place; clears the sums that the z pass adds to
-template <int N1, int N2, bool REAL>
-__global__ void __launch_bounds__(kPassWidth) k_pk_x(const float* __restrict__ delta, float2* mesh, int nbins,
-                                                     double* __restrict__ bins, const uint32_t* __restrict__ err,
+// The deltas are real, so planes z = 2m and 2m + 1 go through x and y as the real and
+// the imaginary part of one plane: half the points.  The z pass takes them apart again.
+// x; clears the sums that the z pass adds to
+template <int N1, int N2>
+__global__ void __launch_bounds__(kPassWidth) k_pk_x(const float* __restrict__ delta, float2* __restrict__ mesh,
+                                                     int nbins, double* __restrict__ bins,
+                                                     const uint32_t* __restrict__ err,
                                                      const float2* __restrict__ tw, int twsh) {
     chain_begin();
     using Q = Pass<N1, N2>;
@@ -282,11 +286,12 @@ __global__ void __launch_bounds__(kPassWidth) k_pk_x(const float* __restrict__ d
     const int64_t q0 = (int64_t)blockIdx.x * Q::P;
     for (int it = threadIdx.x; it < Q::P * N2; it += kPassWidth) {
         const int p = it >> Q::L2, n2 = it & (N2 - 1);
-        const int64_t i = ((q0 + p) << Q::LN) + n2;
+        const int64_t m = q0 >> Q::LN, plane = 1ll << (2 * Q::LN);
+        const float* src = delta + m * plane + ((q0 + p) << Q::LN) + n2;   // row q - m n of plane 2 m
         float2 a[N1];
 #pragma unroll
         for (int n1 = 0; n1 < N1; ++n1)
-            a[bitrev<Q::L1>(n1)] = REAL ? make_float2(delta[i + N2 * n1], 0.f) : mesh[i + N2 * n1];
+            a[bitrev<Q::L1>(n1)] = make_float2(src[N2 * n1], src[plane + N2 * n1]);
         pass_first<N1, N2>(a, Y, p, n2, tw, twsh);
     }
     __syncthreads();
@@ -336,10 +341,14 @@ __device__ __forceinline__ float block_max(float v, float* sh) {
     return v;
 }
 
-// z, and the shells: the mesh's own sums first (a shell a block).  Blocks take groups of P pencils (one ky, P neighbouring kx)
-// in turn and keep their shells in double precision, one owner thread each.  A
-// shell takes at most 2 sqrt(2 j) + 1 modes of a pencil, so a limb's 2048 hold a
-// group at every size.
+// z, and the shells: the mesh's own sums first (a shell a block).  Blocks take groups of
+// P pencils (one ky, P neighbouring kx) in turn and keep their shells in double
+// precision, one owner thread each.  A shell takes at most 2 sqrt(2 j) + 1 modes of a
+// pencil, so a limb's 2048 hold a group at every size.
+// Of the packed planes' spectra C, twice the even planes' is C(kx, ky) +
+// conj C(-kx, -ky) and twice the odd ones' -i times the difference: a pencil's input.  A
+// mode's square is that of its mirror image, so rows 0 < ky < n/2 count twice and those
+// past n/2 are left out.
 template <int N1, int N2>
 __global__ void __launch_bounds__(kPassWidth) k_pk_z(int nbins, double norm, double kf,
                                                      const float2* __restrict__ mesh,
@@ -349,7 +358,7 @@ __global__ void __launch_bounds__(kPassWidth) k_pk_z(int nbins, double norm, dou
     using Q = Pass<N1, N2>;
     constexpr int64_t plane = (int64_t)Q::n * Q::n;
     constexpr int h = Q::n / 2, kItems = (Q::P * N1 + kPassWidth - 1) / kPassWidth;
-    constexpr int kGroups = (int)(plane / Q::P);
+    constexpr int kGroups = (h + 1) * (Q::n / Q::P);
     extern __shared__ __align__(16) unsigned char pass_smem[];
     double* acc = reinterpret_cast<double*>(pass_smem);
     uint32_t* limb = reinterpret_cast<uint32_t*>(acc + h + 1);
@@ -363,15 +372,24 @@ __global__ void __launch_bounds__(kPassWidth) k_pk_z(int nbins, double norm, dou
     }
     for (int g = blockIdx.x; g < kGroups; g += gridDim.x) {
         const int64_t q0 = (int64_t)g * Q::P;
-        const int ky = (int)(q0 >> Q::LN), ny = ky < h ? ky : ky - Q::n;
+        const int ky = (int)(q0 >> Q::LN), kx0 = (int)(q0 & (Q::n - 1));
         for (int it = tid; it < Q::P * N2; it += kPassWidth) {
-            const int p = it & (Q::P - 1), n2 = it >> Q::LP;
+            const int p = it & (Q::P - 1), n2 = it >> Q::LP, kx = kx0 + p;
+            const float2* at = mesh + (n2 >> 1) * plane;
+            const float2* c = at + q0 + p;
+            const float2* mirror = at + ((((Q::n - ky) & (Q::n - 1)) << Q::LN) + ((Q::n - kx) & (Q::n - 1)));
+            const float sg = (n2 & 1) ? -1.f : 1.f;
             float2 a[N1];
 #pragma unroll
-            for (int n1 = 0; n1 < N1; ++n1) a[bitrev<Q::L1>(n1)] = mesh[q0 + p + (N2 * n1 + n2) * plane];
+            for (int n1 = 0; n1 < N1; ++n1) {
+                const float2 u = c[(N2 / 2 * n1) * plane], w = mirror[(N2 / 2 * n1) * plane];
+                const float x = __fmaf_rn(sg, w.x, u.x), y = __fmaf_rn(-sg, w.y, u.y);
+                a[bitrev<Q::L1>(n1)] = (n2 & 1) ? make_float2(y, -x) : make_float2(x, y);
+            }
             pass_first<N1, N2>(a, Y, p, n2, tw, twsh);
         }
         __syncthreads();
+        const float weight = ky == 0 || ky == h ? 1.f : 2.f;
         float v[kItems][N2], big = 0.f;
 #pragma unroll
         for (int u = 0; u < kItems; ++u) {
@@ -381,7 +399,7 @@ __global__ void __launch_bounds__(kPassWidth) k_pk_z(int nbins, double norm, dou
                 pass_second<N1, N2>(a, Y, p, k1);
 #pragma unroll
                 for (int k2 = 0; k2 < N2; ++k2) {
-                    v[u][k2] = a[k2].x * a[k2].x + a[k2].y * a[k2].y;
+                    v[u][k2] = weight * (a[k2].x * a[k2].x + a[k2].y * a[k2].y);
                     big = fmaxf(big, v[u][k2]);
                 }
             }
@@ -391,8 +409,8 @@ __global__ void __launch_bounds__(kPassWidth) k_pk_z(int nbins, double norm, dou
         for (int u = 0; u < kItems; ++u) {
             const int it = tid + u * kPassWidth, p = it & (Q::P - 1), k1 = it >> Q::LP;
             if (it < Q::P * N1) {
-                const int kx = (int)(q0 & (Q::n - 1)) + p, nx = kx < h ? kx : kx - Q::n;
-                const int m0 = nx * nx + ny * ny;
+                const int kx = kx0 + p, nx = kx < h ? kx : kx - Q::n;
+                const int m0 = nx * nx + ky * ky;
 #pragma unroll
                 for (int k2 = 0; k2 < N2; ++k2) {
                     const int kz = k1 + N1 * k2, nz = kz < h ? kz : kz - Q::n;
@@ -412,7 +430,7 @@ __global__ void __launch_bounds__(kPassWidth) k_pk_z(int nbins, double norm, dou
         // (the next group's writes to limb and mx come after its own barrier)
     }
     for (int j = tid; j <= nbins; j += kPassWidth)
-        if (j >= 1 && acc[j] != 0.0) atomicAdd(&bins[j - 1], norm * acc[j]);
+        if (j >= 1 && acc[j] != 0.0) atomicAdd(&bins[j - 1], 0.25 * norm * acc[j]);   // of twice the input
 }
 
 // Up to 16^3 points: transforms, shells and the mesh's own sums in one CTA.  Real
@@ -586,17 +604,13 @@ template <int N1, int N2>
 void launch_transforms(cudaStream_t stream, bool chained, int nbins, double norm, double kf, float2* mesh,
                        const float* delta, double* bins, const uint32_t* err, const float2* tw, int tw_n) {
     using Q = Pass<N1, N2>;
-    const unsigned groups = (unsigned)((int64_t)Q::n * Q::n / Q::P);
+    const unsigned groups = (unsigned)((int64_t)Q::n * Q::n / (2 * Q::P));
     const bool ahead = chained && (int64_t)Q::n * Q::n * Q::n <= kChainCells;
     int twsh = 0;
     while ((Q::n << twsh) < tw_n) ++twsh;
-    if (delta)
-        chain(ahead, k_pk_x<N1, N2, true>, groups, kPassWidth, Q::kBytes, stream, delta, mesh, nbins, bins, err, tw, twsh);
-    else
-        chain(ahead, k_pk_x<N1, N2, false>, groups, kPassWidth, Q::kBytes, stream, nullptr, mesh, nbins, bins, err, tw,
-              twsh);
+    chain(ahead, k_pk_x<N1, N2>, groups, kPassWidth, Q::kBytes, stream, delta, mesh, nbins, bins, err, tw, twsh);
     chain(ahead, k_pk_y<N1, N2>, groups, kPassWidth, Q::kBytes, stream, mesh, tw, twsh);
-    const unsigned gz = groups < 152 * 6 ? groups : 152 * 6;
+    const unsigned gz = groups + Q::n / Q::P < 152 * 6 ? groups + Q::n / Q::P : 152 * 6;
     chain(ahead, k_pk_z<N1, N2>, gz, kPassWidth, z_bytes<N1, N2>(), stream, nbins, norm, kf, mesh, bins, tw, twsh);
 }
 
@@ -611,8 +625,7 @@ template <int N1, int N2>
 void setup_transforms() {
     using Q = Pass<N1, N2>;
     const auto smem = cudaFuncAttributeMaxDynamicSharedMemorySize;
-    cudaFuncSetAttribute(k_pk_x<N1, N2, true>, smem, (int)Q::kBytes);
-    cudaFuncSetAttribute(k_pk_x<N1, N2, false>, smem, (int)Q::kBytes);
+    cudaFuncSetAttribute(k_pk_x<N1, N2>, smem, (int)Q::kBytes);
     cudaFuncSetAttribute(k_pk_y<N1, N2>, smem, (int)Q::kBytes);
     cudaFuncSetAttribute(k_pk_z<N1, N2>, smem, (int)z_bytes<N1, N2>());
 }
@@ -633,7 +646,7 @@ void pk_setup() {
     setup_transforms<32, 32>();
 }
 
-cudaError_t pk_enqueue(cudaStream_t stream, const PkStore& st, int nmesh, int nbins, float2* mesh, float* delta,
+cudaError_t pk_enqueue(cudaStream_t stream, const PkStore& st, int nmesh, int nbins, float2* mesh,
                        double* bins, const uint32_t* err, const float2* tw, int tw_n, int64_t* launches) {
     const int64_t m3 = (int64_t)nmesh * nmesh * nmesh;
     int lh = 0;
@@ -652,8 +665,9 @@ cudaError_t pk_enqueue(cudaStream_t stream, const PkStore& st, int nmesh, int nb
     }
     const double L = 4.0 * st.nc, norm = L * L * L / ((double)m3 * (double)m3), kf = 2.0 * kPi / L;
     const bool small = nmesh <= 16;
-    float* real = small ? reinterpret_cast<float*>(mesh) : (nmesh <= 1024 ? delta : nullptr);
-    if (real) deposit(stream, st, lh, mean, real);
+    // the packed planes take the first half of `mesh`, the deltas the second
+    float* real = reinterpret_cast<float*>(small ? mesh : mesh + m3 / 2);
+    if (nmesh <= 1024) deposit(stream, st, lh, mean, real);
     else deposit(stream, st, lh, mean, mesh);
     *launches += 1;
     if (small) {
@@ -688,12 +702,10 @@ int power_spectrum_enqueue(Sim& s, int nmesh, int nbins, double* host_bins, bool
     if (nbins < 1 || nbins > nmesh / 2)
         return set_error(s, PMPM_EINVAL, "nbins %d must be in [1, nmesh/2]", nbins);
     if (nmesh < s.nc) return set_error(s, PMPM_EINVAL, "nmesh below nf/4 is not supported");
-    const int64_t m3 = (int64_t)nmesh * nmesh * nmesh;
     float2* mesh = reinterpret_cast<float2*>(s.scratch);
-    float* delta = reinterpret_cast<float*>(align_up(reinterpret_cast<uintptr_t>(mesh + m3)));
     const PkStore st = {s.nc, s.pb, s.n, s.offsets[s.cur], s.counts[s.cur],
                         {m_stream(s, s.cur, 0), m_stream(s, s.cur, 1), m_stream(s, s.cur, 2)}, s.chained};
-    cudaError_t e = pk_enqueue(s.stream, st, nmesh, nbins, mesh, delta, s.pk_bins, s.err, s.tw_f, s.fft_max, &s.launches);
+    cudaError_t e = pk_enqueue(s.stream, st, nmesh, nbins, mesh, s.pk_bins, s.err, s.tw_f, s.fft_max, &s.launches);
     if (e == cudaSuccess)
         e = cudaMemcpyAsync(host_bins, s.pk_bins, sizeof(double) * (3 * nbins + word), cudaMemcpyDeviceToHost, s.stream);
     if (e != cudaSuccess) return set_error(s, PMPM_ECUDA, "power spectrum: %s", cudaGetErrorString(e));
