@@ -15,11 +15,13 @@
 //          nothing waits for the fields
 //   y      back, three components
 //   x      back, two fields as one complex pencil, straight to codes and momenta
-// FP64 bounds it: about 240 operations a particle at 1/64 of the FP32 rate.  On a
+// FP64 bounds it: about 180 operations a particle at 1/64 of the FP32 rate.  On a
 // GB300, 256^3 particles with their encode: 17.2 ms with complex radix-2 transforms
-// and a pass per operation, 7.4 now (x with the noise 2.2, y 0.35, z 1.5, y back 1.1,
-// x back 1.8); 32^3: 0.44 -> 0.13 ms.
+// and a pass per operation, 5.8 now (x with the noise 1.2, y 0.35, z 1.2, y back 1.1,
+// x back 1.8); 7.4 with the library's logarithm and cosine and three fields through
+// the inverse z transform.
 #include "pmpm_impl.cuh"
+#include "ic_noise.cuh"
 #include "regfftd.cuh"
 
 namespace pmpm {
@@ -28,23 +30,7 @@ namespace {
 
 constexpr double kPi = 3.141592653589793238462643383279502884;
 
-// SplitMix64 output for counter j (Steele, Lea & Flood 2014)
-__device__ __forceinline__ unsigned long long splitmix64(unsigned long long seed,
-                                                         unsigned long long j) {
-    unsigned long long z = seed + (j + 1ull) * 0x9E3779B97F4A7C15ull;
-    z = (z ^ (z >> 30)) * 0xBF58476D1CE4E5B9ull;
-    z = (z ^ (z >> 27)) * 0x94D049BB133111EBull;
-    return z ^ (z >> 31);
-}
-
-// unit Gaussian of lattice point i (Box-Muller; cos(2 pi u) by cospi)
-__device__ __forceinline__ double ic_noise(unsigned long long seed, unsigned long long i) {
-    const unsigned long long z1 = splitmix64(seed, 2ull * i);
-    const unsigned long long z2 = splitmix64(seed, 2ull * i + 1ull);
-    const double u1 = ((double)(z1 >> 11) + 1.0) * 0x1p-53;
-    const double u2 = (double)(z2 >> 11) * 0x1p-52;
-    return sqrt(-2.0 * log(u1)) * cospi(u2);
-}
+__device__ constexpr NoiseTables kNoise{};
 
 // kf sqrt(P(k)) / k^2 (0 at k = 0), shared by the three displacement components.
 // The amplitude depends on the mode only through m = nx^2 + ny^2 + nz^2
@@ -59,12 +45,12 @@ __global__ void k_ic_amp_table(int mmax, int nf, double slope, double kc, double
             const double k = sqrt(k2);
             c = kf * (sqrt(pow(k, slope) * exp(-(k / kc) * (k / kc))) / k2);
         }
-        tab[m] = c;
+        tab[m] = 0.5 * c;   // the x pass gives twice the noise's spectrum
     }
 }
 
 // x: rows 2q and 2q + 1 of the noise as one complex pencil, then their spectra
-// (kx < n/2) apart: A = (Z + conj Z') / 2, B = (Z - conj Z') / 2i with Z' at -kx
+// (kx < n/2) apart: 2 A = Z + conj Z', 2 B = -i (Z - conj Z') with Z' at -kx
 template <int N1, int N2>
 __global__ void __launch_bounds__(PassD<N1, N2>::T) k_ic_x(unsigned long long seed, double2* __restrict__ out,
                                                            const double2* __restrict__ tw, int twsh) {
@@ -82,7 +68,7 @@ __global__ void __launch_bounds__(PassD<N1, N2>::T) k_ic_x(unsigned long long se
         for (int n1 = 0; n1 < N1; ++n1) {
             // (one copy of the noise's code; the values wait in the buffer's own places)
             const unsigned long long j = i + N2 * n1 + n2;
-            Y[p * Q::PS + n1 * Q::RS + n2] = make_double2(ic_noise(seed, j), ic_noise(seed, j + Q::n));
+            Y[p * Q::PS + n1 * Q::RS + n2] = make_double2(noise_at(seed, j, kNoise), noise_at(seed, j + Q::n, kNoise));
         }
 #pragma unroll
         for (int n1 = 0; n1 < N1; ++n1) a[bitrev<Q::L1>(n1)] = Y[p * Q::PS + n1 * Q::RS + n2];
@@ -110,26 +96,29 @@ __global__ void __launch_bounds__(PassD<N1, N2>::T) k_ic_x(unsigned long long se
         const int p = it / Q::H, k = it & (Q::H - 1);
         const double2 z = Y[p * Q::PS + k], w = Y[p * Q::PS + ((Q::n - k) & (Q::n - 1))];
         double2* row = out + (2 * (q0 + p)) * Q::H + k;
-        row[0] = make_double2(0.5 * (z.x + w.x), 0.5 * (z.y - w.y));
-        row[Q::H] = make_double2(0.5 * (z.y + w.y), 0.5 * (w.x - z.x));
+        row[0] = make_double2(z.x + w.x, z.y - w.y);
+        row[Q::H] = make_double2(z.y + w.y, w.x - z.x);
     }
 }
 
-// y, in place: pencils (kx, z), stride n/2; the inverse for component blockIdx.y
+// y: pencils (kx, z), stride n/2; forward in place, back of component blockIdx.y from
+// w (0; times ky: 1) or in place (2)
 template <int N1, int N2, int S>
-__global__ void __launch_bounds__(PassD<N1, N2>::T) k_ic_y(double2* __restrict__ field, const double2* __restrict__ tw,
-                                                           int twsh) {
+__global__ void __launch_bounds__(PassD<N1, N2>::T) k_ic_y(const double2* w, double2* field,
+                                                           const double2* __restrict__ tw, int twsh) {
     using Q = PassD<N1, N2>;
     extern __shared__ __align__(16) unsigned char ic_smem[];
     double2* Y = reinterpret_cast<double2*>(ic_smem);
     const int64_t q0 = (int64_t)blockIdx.x * Q::P;
-    double2* data = field + (int64_t)blockIdx.y * Q::H * Q::n * Q::n + q0 / Q::H * ((int64_t)Q::H * Q::n) + q0 % Q::H;
+    const int64_t at = q0 / Q::H * ((int64_t)Q::H * Q::n) + q0 % Q::H;
+    double2* data = field + (int64_t)blockIdx.y * Q::H * Q::n * Q::n + at;
+    const double2* src = S > 0 && blockIdx.y < 2 ? w + at : data;
     if (S < 0) {
         for (int it = threadIdx.x; it < Q::P * N2; it += Q::T) {
             const int p = it & (Q::P - 1), n2 = it >> Q::LP;
             double2 a[N1];
 #pragma unroll
-            for (int n1 = 0; n1 < N1; ++n1) a[bitrev<Q::L1>(n1)] = data[p + (N2 * n1 + n2) * Q::H];
+            for (int n1 = 0; n1 < N1; ++n1) a[bitrev<Q::L1>(n1)] = src[p + (N2 * n1 + n2) * Q::H];
             firstd<N1, N2>(a, Y, p, n2, tw, twsh);
         }
         __syncthreads();
@@ -145,7 +134,15 @@ __global__ void __launch_bounds__(PassD<N1, N2>::T) k_ic_y(double2* __restrict__
             const int p = it & (Q::P - 1), k1 = it >> Q::LP;
             double2 a[N2];
 #pragma unroll
-            for (int k2 = 0; k2 < N2; ++k2) a[bitrev<Q::L2>(k2)] = data[p + (k1 + N1 * k2) * Q::H];
+            for (int k2 = 0; k2 < N2; ++k2) {
+                const int k = k1 + N1 * k2;
+                double2 v = src[p + k * Q::H];
+                if (blockIdx.y == 1) {
+                    const double c = small_double(k < Q::H ? k : k - Q::n);
+                    v = make_double2(c * v.x, c * v.y);
+                }
+                a[bitrev<Q::L2>(k2)] = v;
+            }
             back_firstd<N1, N2>(a, Y, p, k1, tw, twsh);
         }
         __syncthreads();
@@ -159,12 +156,13 @@ __global__ void __launch_bounds__(PassD<N1, N2>::T) k_ic_y(double2* __restrict__
     }
 }
 
-// z: forward, Psi~_d = i n_d tab w~ (zero on the Nyquist planes), back into field
-// d; partial[block] = sum of |Psi~|^2 over the whole spectrum (a kx > 0 counts for
-// its mirror image), in a fixed order
+// z: forward, Psi~_d = i n_d tab w~ (zero on the Nyquist planes) and back.  kx and ky do
+// not change along z: without them the x and the y component are one field, which
+// takes w's place; the z component goes to `field`.  partial[block] = sum of |Psi~|^2
+// over the whole spectrum (a kx > 0 counts for its mirror image), in a fixed order
 template <int N1, int N2>
 __global__ void __launch_bounds__(PassD<N1, N2>::T) k_ic_z(const double* __restrict__ tab,
-                                                           const double2* __restrict__ w, double2* __restrict__ field,
+                                                           double2* w, double2* __restrict__ field,
                                                            double* __restrict__ partial,
                                                            const double2* __restrict__ tw, int twsh) {
     using Q = PassD<N1, N2>;
@@ -172,9 +170,7 @@ __global__ void __launch_bounds__(PassD<N1, N2>::T) k_ic_z(const double* __restr
     constexpr int kItems = (Q::P * N1 + Q::T - 1) / Q::T;
     extern __shared__ __align__(16) unsigned char ic_smem[];
     double2* Y = reinterpret_cast<double2*>(ic_smem);
-    __shared__ double nd[Q::n];       // signed wavenumbers, 0 at the Nyquist one
     __shared__ double sums[Q::T / 32];
-    for (int k = threadIdx.x; k < Q::n; k += Q::T) nd[k] = k == Q::H ? 0.0 : (double)(k < Q::H ? k : k - Q::n);
     const int64_t q0 = (int64_t)blockIdx.x * Q::P;   // pencils (kx, ky)
     const int ky = (int)(q0 / Q::H), kx0 = (int)(q0 % Q::H);
     for (int it = threadIdx.x; it < Q::P * N2; it += Q::T) {
@@ -199,13 +195,13 @@ __global__ void __launch_bounds__(PassD<N1, N2>::T) k_ic_z(const double* __restr
                 const int kz = k1 + N1 * k2, nz = kz < Q::H ? kz : kz - Q::n, m = m0 + nz * nz;
                 const double c = ky == Q::H || kz == Q::H ? 0.0 : tab[m];
                 a[u][k2] = make_double2(c * a[u][k2].x, c * a[u][k2].y);
-                e += (double)m * (a[u][k2].x * a[u][k2].x + a[u][k2].y * a[u][k2].y);
+                e += small_double(m) * (a[u][k2].x * a[u][k2].x + a[u][k2].y * a[u][k2].y);
             }
             energy += kx == 0 ? e : 2.0 * e;
         }
     }
 #pragma unroll 1
-    for (int d = 0; d < 3; ++d) {
+    for (int d = 0; d < 2; ++d) {
         __syncthreads();
 #pragma unroll
         for (int u = 0; u < kItems; ++u) {
@@ -214,8 +210,13 @@ __global__ void __launch_bounds__(PassD<N1, N2>::T) k_ic_z(const double* __restr
                 double2 b[N2];
 #pragma unroll
                 for (int k2 = 0; k2 < N2; ++k2) {
-                    const double c = nd[d == 0 ? kx0 + p : (d == 1 ? ky : k1 + N1 * k2)];
-                    b[bitrev<Q::L2>(k2)] = make_double2(-c * a[u][k2].y, c * a[u][k2].x);
+                    b[bitrev<Q::L2>(k2)] = make_double2(-a[u][k2].y, a[u][k2].x);
+                    if (d == 1) {   // (tab is 0 on the Nyquist plane)
+                        const int kz = k1 + N1 * k2;
+                        const double c = small_double(kz < Q::H ? kz : kz - Q::n);
+                        b[bitrev<Q::L2>(k2)].x *= c;
+                        b[bitrev<Q::L2>(k2)].y *= c;
+                    }
                 }
                 back_firstd<N1, N2>(b, Y, p, k1, tw, twsh);
             }
@@ -226,7 +227,7 @@ __global__ void __launch_bounds__(PassD<N1, N2>::T) k_ic_z(const double* __restr
             double2 b[N1];
             back_secondd<N1, N2>(b, Y, p, n2);
 #pragma unroll
-            for (int n1 = 0; n1 < N1; ++n1) field[d * plane * Q::n + q0 + p + (N2 * n1 + n2) * plane] = b[n1];
+            for (int n1 = 0; n1 < N1; ++n1) (d ? field : w)[q0 + p + (N2 * n1 + n2) * plane] = b[n1];
         }
     }
 #pragma unroll
@@ -305,9 +306,11 @@ __global__ void __launch_bounds__(PassD<N1, N2>::T) k_ic_x_back(const double2* _
             if (k != Q::H) {
                 const int kk = k < Q::H ? k : Q::n - k;
                 const double2 x = X[kk], v = V[kk];
-                if (k == 0) r = make_double2(x.x, v.x);
-                else if (k < Q::H) r = make_double2(x.x - v.y, x.y + v.x);
-                else r = make_double2(x.x + v.y, v.x - x.y);
+                // the x component's factor kx
+                const double c = z ? 1.0 : small_double(kk);
+                if (k == 0) r = make_double2(c * x.x, v.x);
+                else if (k < Q::H) r = make_double2(c * x.x - v.y, c * x.y + v.x);
+                else r = make_double2(c * x.x + v.y, v.x - c * x.y);
             }
             a[bitrev<Q::L2>(k2)] = r;
         }
@@ -354,10 +357,10 @@ void ic_passes(Sim& s, uint64_t seed, double rms, const double* tab, double2* w,
     while ((Q::n << twsh) < s.fft_max) ++twsh;
     const unsigned rows = (unsigned)(Q::n * Q::n / Q::P), half = (unsigned)((int64_t)Q::H * Q::n / Q::P);
     k_ic_x<N1, N2><<<half, Q::T, Q::kBytes, st>>>(seed, w, s.tw_d, twsh);
-    k_ic_y<N1, N2, -1><<<half, Q::T, Q::kBytes, st>>>(w, s.tw_d, twsh);
-    k_ic_z<N1, N2><<<half, Q::T, Q::kBytes, st>>>(tab, w, field, partial, s.tw_d, twsh);
+    k_ic_y<N1, N2, -1><<<half, Q::T, Q::kBytes, st>>>(nullptr, w, s.tw_d, twsh);
+    k_ic_z<N1, N2><<<half, Q::T, Q::kBytes, st>>>(tab, w, field + 2 * (s.n / 2), partial, s.tw_d, twsh);
     k_ic_scale_sum<<<1, 256, 0, st>>>((int)half, s.cfg.a_init, rms, partial, scale);
-    k_ic_y<N1, N2, 1><<<dim3(half, 3), Q::T, Q::kBytes, st>>>(field, s.tw_d, twsh);
+    k_ic_y<N1, N2, 1><<<dim3(half, 3), Q::T, Q::kBytes, st>>>(w, field, s.tw_d, twsh);
     k_ic_x_back<N1, N2><<<dim3(rows, 2), Q::T, Q::kBytes, st>>>(field, out, scale, s.tw_d, twsh);
     s.launches += 6;
 }
