@@ -10,9 +10,9 @@
 //  2. delta = rho - mean (float64 subtraction, float32 storage), 3-D FFT;
 //  3. Green multiply: B1 = rho~ (K~_x + i K~_y), B2 = rho~ K~_z (K~ = -i S);
 //  4. two inverse FFTs give F_x + i F_y and F_z.
-// Meshes up to 32^3 fit one SM's shared memory: 2-4 are one launch
-// (k_coarse_tiny, k_coarse_small).  Larger ones take five passes over memory, the
-// ends and the Green multiply fused into them.
+// Meshes up to 16^3 fit one SM's shared memory: 2-4 are one launch
+// (k_coarse_tiny).  Larger ones take five passes over memory, the ends and the
+// Green multiply fused into them.
 #include "pmpm_impl.cuh"
 #include "fftpass.cuh"
 
@@ -215,140 +215,16 @@ __global__ void __launch_bounds__(N * N) k_coarse_tiny(long long mean, const lon
     }
 }
 
-// ------------------------------------------------------------ 32^3 cells
-// The force of one component in one CTA: real transforms along x with the kx = 16
-// plane in the imaginary part of kx = 0 (139 KB of shared memory), rows 17
-// complex apart so that pencils along every axis fall in distinct banks; along
-// z forward, Green multiply and back from the registers.  Three CTAs transform
-// the density each, which is cheaper than twelve launches (69 us on a GB300,
-// against 29).
-template <int N>
-struct SmallMesh {
-    static constexpr int kH = N / 2, kP = kH + 1, kLog = 5;
-    static constexpr int kThreads = N * kH;
-    static constexpr size_t kBytes = sizeof(float2) * N * N * kP;
-};
-
-template <int N, int S>
-__device__ __forceinline__ void small_pencil(float2* c, int stride) {
-    float2 a[N];
-#pragma unroll
-    for (int k = 0; k < N; ++k) a[bitrev<SmallMesh<N>::kLog>(k)] = c[k * stride];
-    fft_dit<N, S>(a);
-#pragma unroll
-    for (int k = 0; k < N; ++k) c[k * stride] = a[k];
-}
-
-template <int N>
-__global__ void __launch_bounds__(SmallMesh<N>::kThreads) k_coarse_small(long long mean, const long long* __restrict__ rho,
-                                                                         const float4* __restrict__ table,
-                                                                         float* __restrict__ Fl) {
-    chain_wait();
-    using M = SmallMesh<N>;
-    constexpr int H = M::kH, P = M::kP, T = M::kThreads, L = M::kLog;
-    extern __shared__ __align__(16) unsigned char small_smem[];
-    float2* C = reinterpret_cast<float2*>(small_smem);
-    float* R = reinterpret_cast<float*>(small_smem);
-    const int tid = threadIdx.x, comp = blockIdx.x;
-#pragma unroll 8
-    for (int i = tid; i < N * N * N; i += T) R[(i >> L) * (2 * P) + (i & (N - 1))] = delta_of(rho[i], mean);
-    __syncthreads();
-    for (int r = tid; r < N * N; r += T) {
-        float2* row = C + r * P;
-        float x[N];
-        float2 X[H + 1];
-#pragma unroll
-        for (int k = 0; k < H; ++k) {
-            x[2 * k] = row[k].x;
-            x[2 * k + 1] = row[k].y;
-        }
-        rfftx2<N>(x, X);
-        row[0] = make_float2(X[0].x, X[H].x);
-#pragma unroll
-        for (int k = 1; k < H; ++k) row[k] = X[k];
-    }
-    __syncthreads();
-    for (int t = tid; t < H * N; t += T)   // along y: kx, z
-        small_pencil<N, -1>(C + (t / H) * (N * P) + t % H, P);
-    __syncthreads();
-    for (int t = tid; t < H * N; t += T) {   // along z: kx = t / N, ky = t mod N
-        const int kx = t / N, ky = t % N;
-        float2* col = C + ky * P + kx;
-        float2 a[N];
-#pragma unroll
-        for (int k = 0; k < N; ++k) a[bitrev<L>(k)] = col[k * (N * P)];
-        fft_dit<N, -1>(a);
-        int ay;
-        float sy;
-        kfold(ky, N, ay, sy);
-        if (kx != 0) {
-#pragma unroll
-            for (int kz = 0; kz < N; ++kz) {
-                const int az = kz <= H ? kz : N - kz;
-                const float sz = kz == 0 ? 0.f : (kz <= H ? 1.f : -1.f);
-                const float4 g = table[(az * (H + 1) + ay) * (H + 1) + kx];
-                const float c = comp == 0 ? g.x : (comp == 1 ? sy * g.y : sz * g.z);
-                a[kz] = make_float2(c * a[kz].y, -(c * a[kz].x));   // -i c a
-            }
-        } else {
-            // Z = A + i B holds kx = 0 and kx = N/2; with the partner Z' at (-ky, -kz),
-            // -i (s0 A + i sH B) = -i [(s0 + sH)/2 Z + (s0 - sH)/2 conj Z'] (the x
-            // component's s0 and sH vanish).  One warp holds the column.
-#pragma unroll
-            for (int kz = 0; kz < N; ++kz) col[kz * (N * P)] = a[kz];
-            __syncwarp();
-            const float2* mate = C + ((N - ky) & (N - 1)) * P;
-            float2 b[N];
-#pragma unroll
-            for (int kz = 0; kz < N; ++kz) b[kz] = mate[((N - kz) & (N - 1)) * (N * P)];
-            __syncwarp();
-#pragma unroll
-            for (int kz = 0; kz < N; ++kz) {
-                const int az = kz <= H ? kz : N - kz;
-                const float sz = kz == 0 ? 0.f : (kz <= H ? 1.f : -1.f);
-                const float4 g0 = table[(az * (H + 1) + ay) * (H + 1)], gH = table[(az * (H + 1) + ay) * (H + 1) + H];
-                const float s0 = comp == 0 ? 0.f : (comp == 1 ? sy * g0.y : sz * g0.z);
-                const float sH = comp == 0 ? 0.f : (comp == 1 ? sy * gH.y : sz * gH.z);
-                const float cA = 0.5f * (s0 + sH), cB = 0.5f * (s0 - sH);
-                const float vx = cA * a[kz].x + cB * b[kz].x, vy = cA * a[kz].y - cB * b[kz].y;
-                a[kz] = make_float2(vy, -vx);
-            }
-        }
-        float2 w[N];
-#pragma unroll
-        for (int k = 0; k < N; ++k) w[bitrev<L>(k)] = a[k];
-        fft_dit<N, 1>(w);
-#pragma unroll
-        for (int k = 0; k < N; ++k) col[k * (N * P)] = w[k];
-    }
-    __syncthreads();
-    for (int t = tid; t < H * N; t += T) small_pencil<N, 1>(C + (t / H) * (N * P) + t % H, P);
-    __syncthreads();
-    for (int r = tid; r < N * N; r += T) {
-        float2* row = C + r * P;
-        float x[N];
-        float2 X[H + 1];
-        X[0] = make_float2(row[0].x, 0.f);
-        X[H] = make_float2(row[0].y, 0.f);
-#pragma unroll
-        for (int k = 1; k < H; ++k) X[k] = row[k];
-        irfft<N>(X, x);
-#pragma unroll
-        for (int k = 0; k < H; ++k) row[k] = make_float2(0.5f * x[2 * k], 0.5f * x[2 * k + 1]);   // rfftx2 doubles
-    }
-    __syncthreads();
-    chain_next();
-    for (int i = tid; i < N * N * N; i += T) Fl[(int64_t)comp * N * N * N + i] = R[(i >> L) * (2 * P) + (i & (N - 1))];
-}
-
-// ------------------------------------------------------------ 64^3 cells and more
+// ------------------------------------------------------------ 32^3 cells and more
 // Passes of n = N1 N2 points per pencil in two register steps with one
 // transpose through shared memory (fft.cu).  With j = N2 n1 + n2 and
 // k = k1 + N1 k2 the forward pass ends with all k2 of one k1 in a thread's
 // registers, which is where the inverse one begins: the z pass transforms,
 // multiplies and transforms back without another exchange.  116 bytes a cell
 // over five launches against 212 over twelve: 64^3 cells 73 -> 38 us, 128^3
-// 126 -> 72, 256^3 (HBM-bound) 710 -> 399.
+// 126 -> 72, 256^3 (HBM-bound) 710 -> 399.  32^3 cells (69 us before) take 32 blocks
+// a pass; one launch of three CTAs with the mesh in shared memory took 29 us, a
+// step 321 us against 310.
 // x: integer density rows -> delta -> spectrum
 template <int N1, int N2>
 __global__ void __launch_bounds__(kPassWidth) k_coarse_fwd_x(long long mean, const long long* __restrict__ rho,
@@ -551,11 +427,6 @@ void launch_tiny(Sim& s, long long mean) {
     chain(s.chained, k_coarse_tiny<N>, 2, N * N, 0, s.stream, mean, s.rho_c, s.green_coarse, s.Fl, s.tw_f, twsh);
     s.launches++;
 }
-void launch_small(Sim& s, long long mean) {
-    using M = SmallMesh<32>;
-    chain(s.chained, k_coarse_small<32>, 3, M::kThreads, M::kBytes, s.stream, mean, s.rho_c, s.green_coarse, s.Fl);
-    s.launches++;
-}
 template <int N1, int N2>
 void launch_passes(Sim& s, long long mean) {
     using Q = Pass<N1, N2>;
@@ -587,7 +458,7 @@ int coarse_deposit(Sim& s, bool cleared) {
 }
 
 void coarse_setup() {
-    cudaFuncSetAttribute(k_coarse_small<32>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)SmallMesh<32>::kBytes);
+    pass_setup<4, 8>();
     pass_setup<8, 8>();
     pass_setup<8, 16>();
     pass_setup<16, 16>();
@@ -601,7 +472,7 @@ int coarse_force(Sim& s) {
     switch (s.nc) {
         case 8: launch_tiny<8>(s, mean); break;
         case 16: launch_tiny<16>(s, mean); break;
-        case 32: launch_small(s, mean); break;
+        case 32: launch_passes<4, 8>(s, mean); break;
         case 64: launch_passes<8, 8>(s, mean); break;
         case 128: launch_passes<8, 16>(s, mean); break;
         case 256: launch_passes<16, 16>(s, mean); break;

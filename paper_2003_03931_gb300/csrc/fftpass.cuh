@@ -13,7 +13,7 @@ namespace pmpm {
 
 // The float32 nearest to d.  Two halves that float32 holds exactly and one
 // multiply-add round it once; 64-bit conversions and FP64 run at 1/64 of the
-// FP32 rate here (three per cell took 24 us of a 32^3 mesh on three SMs).
+// FP32 rate here (three per cell took 24 us for a 32^3 mesh on three SMs).
 __device__ __forceinline__ float f32_of(long long d) {
     if (d >= (1ll << 40) || d < -(1ll << 40)) return __ll2float_rn(d);
     return __fmaf_rn((float)(int)(d >> 16), 65536.f, (float)((int)d & 0xffff));
