@@ -14,9 +14,10 @@
 // FP64 runs at 1/64 of the FP32 rate here, so shell sums are exact integers of
 // 21-bit limbs of the float32 squares, and only a block's totals become doubles.
 //
-// On a GB300: 256^3 particles on 512^3 points 10.5 -> 1.47 ms (a search per
+// On a GB300: 256^3 particles on 512^3 points 10.5 -> 1.37 ms (a search per
 // particle, 64-bit global atomics and three double shared atomics a mode before):
-// deposit 0.65 (shared atomics), x 0.21, y 0.21, z with the shells 0.34, of 0.48 ms for
+// deposit 0.55 (issue: the particles of 2.8 bricks
+// are looked at), x 0.21, y 0.21, z with the shells 0.34, of 0.48 ms for
 // 24 bytes a point at the copy bandwidth (1.95 ms with planes of their own, 40 bytes);
 // 32^3 on 32^3, without allocation, 115 -> 70 us.
 #include "power.cuh"
@@ -57,10 +58,17 @@ struct PkMean {
         if (inv > 0.0) return (float)((double)v * inv - 1.0);
         return f32_of(((long long)v << shift) - mean) * scale;
     }
+    // the same for v < 2^31 where narrow()
+    __device__ __forceinline__ bool narrow() const { return inv <= 0.0 && shift == 0 && mean < (1ll << 31); }
+    __device__ __forceinline__ float delta(uint32_t v) const { return __int2float_rn((int)(v - (uint32_t)mean)) * scale; }
 };
 
-__device__ __forceinline__ void put(float* out, int64_t i, float v) { out[i] = v; }
-__device__ __forceinline__ void put(float2* out, int64_t i, float v) { out[i] = make_float2(v, 0.f); }
+// four nodes from i, a multiple of 4
+__device__ __forceinline__ void put(float* out, int64_t i, float4 v) { *reinterpret_cast<float4*>(out + i) = v; }
+__device__ __forceinline__ void put(float2* out, int64_t i, float4 v) {
+    *reinterpret_cast<float4*>(out + i) = make_float4(v.x, 0.f, v.y, 0.f);
+    *reinterpret_cast<float4*>(out + i + 2) = make_float4(v.z, 0.f, v.w, 0.f);
+}
 
 // the cells x0 - 1 .. of row (by, bz) around the brick, one per lane; never past
 // the store, whatever the counts
@@ -97,7 +105,7 @@ __global__ void __launch_bounds__(Brick<LH, SMALL>::kThreads) k_pk_deposit(const
         const int by = row % (B::CY + 2), bz = row / (B::CY + 2);
         return (int64_t)nc * (wrap1(y0 - 1 + by, nc) + (int64_t)nc * wrap1(z0 - 1 + bz, nc));
     };
-    for (int i = tid; i < 2 * B::kNodes; i += T) pk_smem[i] = 0u;
+    for (int i = tid; i < B::kNodes / 2; i += T) reinterpret_cast<uint4*>(pk_smem)[i] = make_uint4(0u, 0u, 0u, 0u);
     int most = 0;
     for (int row = warp; row < kRows; row += T / 32) {
         int64_t off;
@@ -150,11 +158,22 @@ __global__ void __launch_bounds__(Brick<LH, SMALL>::kThreads) k_pk_deposit(const
         }
     }
     __syncthreads();
+    // four nodes a thread (NX and the mesh's side are multiples of 4); by 32-bit integers
+    // where they hold the sums: half of the kernel's instructions were 64-bit ones here
     const int64_t nm = (int64_t)nc * B::R;
-    for (int i = tid; i < B::kNodes; i += T) {
-        const int x = i % B::NX, y = i / B::NX % B::NY, z = i / (B::NX * B::NY);
-        const unsigned long long v = (unsigned long long)hi[i] << 32 | lo[i];
-        put(out, (x0 * B::R + x) + nm * ((y0 * B::R + y) + nm * (int64_t)(z0 * B::R + z)), mean.delta(v));
+    const bool narrow = safe && mean.narrow();
+    for (int q = tid; q < B::kNodes / 4; q += T) {
+        const int x = 4 * q % B::NX, y = 4 * q / B::NX % B::NY, z = 4 * q / (B::NX * B::NY);
+        const uint4 l = reinterpret_cast<const uint4*>(lo)[q];
+        float4 d;
+        if (narrow && (int)(l.x | l.y | l.z | l.w) >= 0) {
+            d = make_float4(mean.delta(l.x), mean.delta(l.y), mean.delta(l.z), mean.delta(l.w));
+        } else {
+            const uint4 h = reinterpret_cast<const uint4*>(hi)[q];
+            d = make_float4(mean.delta((unsigned long long)h.x << 32 | l.x), mean.delta((unsigned long long)h.y << 32 | l.y),
+                            mean.delta((unsigned long long)h.z << 32 | l.z), mean.delta((unsigned long long)h.w << 32 | l.w));
+        }
+        put(out, (x0 * B::R + x) + nm * ((y0 * B::R + y) + nm * (int64_t)(z0 * B::R + z)), d);
     }
 }
 
@@ -434,8 +453,7 @@ __global__ void __launch_bounds__(kPassWidth) k_pk_z(int nbins, double norm, dou
 }
 
 // Up to 16^3 points: transforms, shells and the mesh's own sums in one CTA.  Real
-// transforms along x with the kx = N/2 plane in the imaginary part of kx = 0, as in
-// k_coarse_small; a mode with 0 < kx < N/2 stands for its mirror image too.
+// transforms along x with the kx = N/2 plane in the imaginary part of kx = 0; a mode with 0 < kx < N/2 stands for its mirror image too.
 template <int N>
 struct PkSmall {
     static constexpr int kH = N / 2, kP = kH + 1, kLog = N == 16 ? 4 : 3;
