@@ -270,24 +270,6 @@ struct Cic1 {
     int w1;      // weight of node i0+1, in 1/(2U) units
 };
 
-// fine mesh: U = 64, weights in 1/128
-PMPM_HD Cic1 cic_fine(int64_t Q) {
-    int64_t s = 2 * Q + 1 - kCodesPerFine;
-    Cic1 c;
-    c.i0 = (int)(s >> 7);
-    c.w1 = (int)(s & 127);
-    return c;
-}
-
-// coarse mesh: U = 256, weights in 1/512
-PMPM_HD Cic1 cic_coarse(int64_t Q) {
-    int64_t s = 2 * Q + 1 - kBins;
-    Cic1 c;
-    c.i0 = (int)(s >> 9);
-    c.w1 = (int)(s & 511);
-    return c;
-}
-
 PMPM_HD int wrap(int i, int n) {
     int r = i % n;
     return r < 0 ? r + n : r;

@@ -60,34 +60,7 @@ __device__ void ewald_real(const Ewald& e, double x, double y, double z, double 
             }
 }
 
-// Fourier sum over |h| <= h_max, h != 0
-__device__ void ewald_fourier(const Ewald& e, double x, double y, double z, double out[3]) {
-    const double pref = 4.0 * kPi / (e.L * e.L * e.L);
-    const double kf = 2.0 * kPi / e.L;
-    const int H = e.h_max;
-    for (int hz = -H; hz <= H; ++hz)
-        for (int hy = -H; hy <= H; ++hy)
-            for (int hx = -H; hx <= H; ++hx) {
-                const int h2 = hx * hx + hy * hy + hz * hz;
-                if (h2 == 0 || h2 > H * H) continue;
-                const double kx = kf * hx, ky = kf * hy, kz = kf * hz;
-                const double k2 = kx * kx + ky * ky + kz * kz;
-                const double c = pref * exp(-k2 / (4.0 * e.alpha * e.alpha)) / k2 *
-                                 sin(kx * x + ky * y + kz * z);
-                out[0] -= c * kx;
-                out[1] -= c * ky;
-                out[2] -= c * kz;
-            }
-}
-
-__device__ void ewald_force(const Ewald& e, double x, double y, double z, double out[3]) {
-    out[0] = out[1] = out[2] = 0.0;
-    if (x == 0.0 && y == 0.0 && z == 0.0) return;
-    ewald_real(e, x, y, z, out);
-    ewald_fourier(e, x, y, z, out);
-}
-
-// The x component of the same force, evaluated by one warp: lane l takes the
+// The x component of the periodic force, evaluated by one warp: lane l takes the
 // images and Fourier vectors with flat index l, l + 32, ...; the lane sums
 // are combined in a fixed order (every lane returns the total).
 __device__ double ewald_force_x_warp(const Ewald& e, double x, double y, double z, int lane) {
