@@ -222,9 +222,8 @@ __global__ void __launch_bounds__(N * N) k_coarse_tiny(long long mean, const lon
 // registers, which is where the inverse one begins: the z pass transforms,
 // multiplies and transforms back without another exchange.  116 bytes a cell
 // over five launches against 212 over twelve: 64^3 cells 73 -> 38 us, 128^3
-// 126 -> 72, 256^3 (HBM-bound) 710 -> 399.  32^3 cells (69 us before) take 32 blocks
-// a pass; one launch of three CTAs with the mesh in shared memory took 29 us, a
-// step 321 us against 310.
+// 126 -> 72, 256^3 (HBM-bound) 710 -> 399.  32^3 cells (69 us before) are 32 blocks
+// a pass and 14 us; one launch of three CTAs with the mesh in shared memory: 29 us.
 // x: integer density rows -> delta -> spectrum
 template <int N1, int N2>
 __global__ void __launch_bounds__(kPassWidth) k_coarse_fwd_x(long long mean, const long long* __restrict__ rho,
