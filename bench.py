@@ -46,7 +46,7 @@ SM_COUNT = 152
 FP32_LANES_PER_SM = 128
 TILE_FFT = 32
 TILE_FILES = ["paper_2003_03931_gb300/csrc/tile_core.cuh", "paper_2003_03931_gb300/csrc/regfft.cuh",
-              "paper_2003_03931_gb300/csrc/tile.cu", "paper_2003_03931_gb300/csrc/common.cuh"]
+              "paper_2003_03931_gb300/csrc/column.cu", "paper_2003_03931_gb300/csrc/common.cuh"]
 
 
 def parse_args(argv=None):
@@ -80,7 +80,8 @@ def parse_args(argv=None):
 def tile_flops_per_launch(nc, tile_max=5):
     """Algorithmic FLOPs of one tile pass: per tile one real 32^3 forward
     transform and three real inverse transforms, 2.5 M log2 M each
-    (M = 32^3 points), over all tiles."""
+    (M = 32^3 points), over all tiles: the conventional count of the method,
+    whatever share of it the kernel avoids."""
     nt = -(-nc // tile_max)
     m = TILE_FFT ** 3
     return 4 * 2.5 * m * math.log2(m) * nt ** 3
@@ -98,10 +99,10 @@ HBM_STAGE_BYTES = {
     "coarse_deposit": (3, 20),
     # density in and spectrum out, spectrum in and F_l out (one pass each way)
     "coarse_fft_green": (0, 36),
-    # counts and momentum sums in; offsets and v_c out
+    # counts and momentum sums in; offsets, v_c and the dispersion out
     "hist_scan_cell_means": (0, 48),
     "scan_cell_means": (0, 48),
-    # per cell: counts and momentum sums in (the cell part of the dispersion)
+    # (a stage of its own only in name: it is part of the one above and takes 0 ms)
     "dispersion": (0, 28),
     "cell_moments_sigma": (0, 28),
     # new codes and momenta in, store out; v_c and offsets in
@@ -428,8 +429,8 @@ def box_roofline(m, workload, fp32_peak, peak_basis, hbm):
     launches = len(tile_stages)
     avg_ms = tile_ms / launches
     achieved = flops / (avg_ms / 1e3) / 1e12
-    kernel = ("k_tile, low-memory form (tile fine PM + kick + drift; new momenta kept, codes not)"
-              if cfg.lowmem else "k_tile (tile fine PM + kick + drift)")
+    kernel = ("k_column, low-memory form (tile fine PM + kick + drift; new momenta kept, codes not)"
+              if cfg.lowmem else "k_column (tile fine PM + kick + drift)")
     roof = {"bound": "alu", "kernel": kernel, "achieved": achieved, "peak": fp32_peak,
             "unit": "TFLOP/s", "frac": achieved / fp32_peak,
             "traffic": recorded_traffic(workload, lowmem=cfg.lowmem),

@@ -1,6 +1,7 @@
 // fft.cu -- batched 1-D FFTs along the three axes of an n^3 complex array
-// (n a power of two), float or double.  Used for the coarse-mesh force of
-// Eq. 1, the Zel'dovich displacement field and the power spectrum.
+// (n a power of two), float or double.  Used for the force tables, the low-memory
+// step's displacement field and power spectra past 1024 points a side; a step's
+// coarse force, the other initial conditions and spectra have passes of their own.
 //
 // One block transforms P neighbouring pencils.  Float pencils of 64 to 1024
 // points take two register steps with one shared-memory transpose
