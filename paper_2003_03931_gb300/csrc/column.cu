@@ -29,6 +29,8 @@
 // for the particles' bytes; memory moves 41 B a particle.  Short-range pass of a step on a GB300 against
 // the 32^3-box tiles of one CTA a SM before: 512^3 particles 36.5 -> 19.1 ms,
 // 256^3 4.57 -> 2.54 ms, 128^3 607 -> 404 us, 64^3 125 -> 84 us.
+#include <algorithm>
+
 #include "pmpm_impl.cuh"
 #include "tile_core.cuh"
 
@@ -881,13 +883,23 @@ void column_setup() {
 // shortest walk: 64^3 particles on 32^3 cells lz = 6 (98 us against 111 at 11
 // and 120 at 3), 128^3 on 64^3 22 (431 us; 509 at 6, 540 at 64), 256^3 on 128^3 64
 // (2.58 ms; 2.83 at 16, 2.93 at 128).
-static int column_layers(int nc, int nt) {
+//
+// Where other boxes fill the SMs (sharers of them in all), the last CTAs of a pass cost
+// nothing and what counts is the sum of all walks: longer ones, but none that would take
+// 1.3 times as long alone.  Sixteen boxes of 32^3 to 128^3 particles 23.7 -> 22.5 ms; 400
+// requests as they come at 1.5 times the capacity, p99 1.98 -> 1.85 s.
+static int column_layers(int nc, int nt, int sharers) {
+    const auto ctas = [=](int lz) { return (int64_t)nt * nt * ((nc + lz - 1) / lz); };
+    const auto alone = [=](int lz) {
+        const int64_t n = ctas(lz), rest = n % 304;
+        return ((double)(n / 304) + (rest == 0 ? 0.0 : (rest <= 152 ? 0.74 : 1.0))) * (lz + 5.5);
+    };
+    double least = 1e30, cost = 1e30;
+    for (int lz = 1; lz <= nc; ++lz) least = std::min(least, alone(lz));
     int best = nc;
-    double cost = 1e30;
     for (int lz = 1; lz <= nc; ++lz) {
-        const int64_t ctas = (int64_t)nt * nt * ((nc + lz - 1) / lz), rest = ctas % 304;
-        const double waves = (double)(ctas / 304) + (rest == 0 ? 0.0 : (rest <= 152 ? 0.74 : 1.0));
-        const double c = waves * (lz + 5.5);
+        if (alone(lz) > (sharers > 1 ? 1.3 : 1.0) * least) continue;
+        const double c = alone(lz) + (sharers - 1) * (double)ctas(lz) / 304 * (lz + 5.5);
         if (c < cost) {
             cost = c;
             best = lz;
@@ -896,11 +908,12 @@ static int column_layers(int nc, int nt) {
     return best;
 }
 
-void column_pass(cudaStream_t st, const TileParams& P, const float* table, bool lowmem, int pb, bool chained) {
+void column_pass(cudaStream_t st, const TileParams& P, const float* table, bool lowmem, int pb, bool chained,
+                 int sharers) {
     ColParams C;
     C.t = P;
     C.table = table;
-    C.lz = column_layers(P.nc, P.nt);
+    C.lz = column_layers(P.nc, P.nt, sharers);
     const unsigned grid = (unsigned)(P.nt * P.nt * ((P.nc + C.lz - 1) / C.lz));
     if (lowmem) chain(chained, k_column<true, 1>, grid, kColThreads, sizeof(ColShared), st, C);
     else if (pb == 2) chain(chained, k_column<false, 2>, grid, kColThreads, sizeof(ColShared), st, C);

@@ -79,6 +79,7 @@ struct Sim {
 
     // captured steps, one per buffer parity
     bool chained = false;                       // launches may overlap (chain())
+    int sharers = 1;                            // boxes that run on the GPU at once
     bool graphs = false;
     bool graph_ready[2] = {false, false};
     cudaGraphExec_t graph_exec[2] = {nullptr, nullptr};

@@ -338,6 +338,7 @@ bool admit(pmpm_batch& b, Job* j) {
 bool advance(pmpm_batch& b, Job* j, bool* did) {
     while (!j->finishing && j->enq < j->r.n_steps && (int)j->inflight.size() < b.c.chunks_in_flight) {
         const int k = std::min(b.c.steps_per_chunk, j->r.n_steps - j->enq);
+        j->sim->s.sharers = (int)b.active.size();
         int rc = pmpm_step(j->sim, k);
         cudaEvent_t e = rc ? nullptr : take_event(b);
         if (!rc && (!e || cudaEventRecord(e, j->st) != cudaSuccess)) rc = PMPM_ECUDA;

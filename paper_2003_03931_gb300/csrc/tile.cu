@@ -9,7 +9,8 @@
 namespace pmpm {
 
 void column_setup();
-void column_pass(cudaStream_t st, const TileParams& P, const float* table, bool lowmem, int pb, bool chained);
+void column_pass(cudaStream_t st, const TileParams& P, const float* table, bool lowmem, int pb, bool chained,
+                 int sharers);
 
 template <int D, bool LM, int PB, typename CT>
 __device__ __forceinline__ void tile_component(int tid, const TileGeom& g, const TileParams& P,
@@ -201,7 +202,7 @@ int tile_pass(Sim& s, int mode, float* G) {
     // against 88; 64^3 cells: 607 against 413.
     constexpr int kTileCells = 16;
     const int grid = s.nt * s.nt * s.nt;
-    if (!s.fp16 && s.nc > kTileCells) column_pass(s.stream, P, s.green_col, s.lowmem, s.pb, s.chained);
+    if (!s.fp16 && s.nc > kTileCells) column_pass(s.stream, P, s.green_col, s.lowmem, s.pb, s.chained, s.sharers);
     else if (s.lowmem) chain(s.chained, k_tile<1, float2, true>, grid, kTileThreads, kTileSmemBytes, s.stream, P);
     else if (s.fp16 && s.pb == 2) chain(s.chained, k_tile<2, __half2>, grid, kTileThreads, kTileSmemBytes, s.stream, P);
     else if (s.fp16) chain(s.chained, k_tile<1, __half2>, grid, kTileThreads, kTileSmemBytes, s.stream, P);
