@@ -11,8 +11,8 @@
 //  3. Green multiply: B1 = rho~ (K~_x + i K~_y), B2 = rho~ K~_z (K~ = -i S);
 //  4. two inverse FFTs give F_x + i F_y and F_z.
 // Meshes up to 16^3 fit one SM's shared memory: 2-4 are one launch
-// (k_coarse_tiny).  Larger ones take five passes over memory, the ends and the
-// Green multiply fused into them.
+// (k_coarse_tiny).  32^3 cells take four launches of a warp a plane or row, larger
+// meshes five passes over memory, the ends and the Green multiply fused into them.
 #include "pmpm_impl.cuh"
 #include "fftpass.cuh"
 
@@ -155,6 +155,13 @@ __device__ __forceinline__ void tiny_pencil(float2* c, int stride, const float2 
     for (int k = 0; k < N; ++k) c[k * stride] = a[k];
 }
 
+// a (S_y - i S_x), or a (-i S_z)
+__device__ __forceinline__ float2 green_times(float2 a, float4 g, float sx, float sy, float sz, bool xy) {
+    const float Sx = sx * g.x, Sy = sy * g.y, Sz = sz * g.z;
+    return xy ? make_float2(__fmaf_rn(a.x, Sy, __fmul_rn(a.y, Sx)), __fmaf_rn(a.y, Sy, -__fmul_rn(a.x, Sx)))
+              : make_float2(a.y * Sz, -a.x * Sz);
+}
+
 template <int N>
 __global__ void __launch_bounds__(N * N) k_coarse_tiny(long long mean, const long long* __restrict__ rho,
                                                        const float4* __restrict__ table, float* __restrict__ Fl,
@@ -187,12 +194,7 @@ __global__ void __launch_bounds__(N * N) k_coarse_tiny(long long mean, const lon
         int az;
         float sz;
         kfold(z, N, az, sz);
-        const float4 g = table[(az * h + ay) * h + ax];
-        const float Sx = sx * g.x, Sy = sy * g.y, Sz = sz * g.z;
-        // a (S_y - i S_x) or a (-i S_z)
-        col[z * (N * P)] = blockIdx.x == 0 ? make_float2(__fmaf_rn(a[z].x, Sy, __fmul_rn(a[z].y, Sx)),
-                                                         __fmaf_rn(a[z].y, Sy, -__fmul_rn(a[z].x, Sx)))
-                                           : make_float2(a[z].y * Sz, -a[z].x * Sz);
+        col[z * (N * P)] = green_times(a[z], table[(az * h + ay) * h + ax], sx, sy, sz, blockIdx.x == 0);
     }
     __syncthreads();
     tiny_pencil<N, 1>(C + tid * P, 1, tw);
@@ -215,15 +217,135 @@ __global__ void __launch_bounds__(N * N) k_coarse_tiny(long long mean, const lon
     }
 }
 
-// ------------------------------------------------------------ 32^3 cells and more
+// ------------------------------------------------------------ 32^3 cells
+// The same stages, twiddles and roundings (keeps_bits) in four launches: x and y of a
+// plane by one warp, through registers and a plane of shared memory, z with the Green
+// multiply, a pencil a thread, and both back.  Latency bounds it: one warp on an SM walks
+// two pencils' 32 points in a row.  20 us on a GB300; twelve passes of fft.cu 69, the
+// five fused passes of larger meshes, whose order of axes gives other bits, 14.
+constexpr int kC32 = 32, kC32Plane = kC32 * kC32, kC32Cells = kC32 * kC32Plane, kC32Pitch = kC32 + 1;
+
+// the 32-point twiddles of a table of 32 << twsh
+__device__ __forceinline__ void c32_twiddles(const float2* __restrict__ twiddles, int twsh, float2 (&tw)[kC32 / 2]) {
+#pragma unroll
+    for (int k = 0; k < kC32 / 2; ++k) tw[k] = twiddles[k << twsh];
+}
+
+// x and y of plane blockIdx.x: of the density (S = -1) to A, or of A or B (by
+// blockIdx.y), in place, back
+template <int S>
+__global__ void __launch_bounds__(kC32) k_coarse32_plane(long long mean, const long long* rho, float2* A, float2* B,
+                                                         const float2* __restrict__ twiddles, int twsh) {
+    chain_begin();
+    __shared__ float2 C[kC32 * kC32Pitch];
+    const int lane = threadIdx.x;
+    const int64_t at = (int64_t)blockIdx.x * kC32Plane + lane;
+    float2* const data = blockIdx.y ? B : A;
+    float2 tw[kC32 / 2];
+    c32_twiddles(twiddles, twsh, tw);
+#pragma unroll 8
+    for (int y = 0; y < kC32; ++y)
+        C[y * kC32Pitch + lane] = S < 0 ? make_float2(delta_of(rho[at + y * kC32], mean), 0.f) : data[at + y * kC32];
+    __syncwarp();
+    tiny_pencil<kC32, S>(C + lane * kC32Pitch, 1, tw);
+    __syncwarp();
+    float2 a[kC32];
+#pragma unroll
+    for (int y = 0; y < kC32; ++y) a[y] = C[y * kC32Pitch + lane];
+    autosort<kC32, S>(a, tw);
+#pragma unroll
+    for (int y = 0; y < kC32; ++y) data[at + y * kC32] = a[y];
+}
+
+// z: pencils (kx, ky = blockIdx.x); forward from A, Green multiply, to B1 (blockIdx.y = 0) or B2
+__global__ void __launch_bounds__(kC32) k_coarse32_green(const float4* __restrict__ table, const float2* A, float2* B1,
+                                                         float2* B2, const float2* __restrict__ twiddles, int twsh) {
+    chain_begin();
+    constexpr int h = kC32 / 2 + 1;
+    const int x = threadIdx.x, y = blockIdx.x, at = y * kC32 + x;
+    float2 tw[kC32 / 2], a[kC32];
+    c32_twiddles(twiddles, twsh, tw);
+#pragma unroll
+    for (int z = 0; z < kC32; ++z) a[z] = A[z * kC32Plane + at];
+    autosort<kC32, -1>(a, tw);
+    int ax, ay;
+    float sx, sy;
+    kfold(x, kC32, ax, sx);
+    kfold(y, kC32, ay, sy);
+    float2* const out = blockIdx.y ? B2 : B1;
+#pragma unroll
+    for (int z = 0; z < kC32; ++z) {
+        int az;
+        float sz;
+        kfold(z, kC32, az, sz);
+        out[z * kC32Plane + at] = green_times(a[z], table[(az * h + ay) * h + ax], sx, sy, sz, blockIdx.y == 0);
+    }
+}
+
+// z back: F_x + i F_y from B1 (blockIdx.y = 0), F_z from B2
+__global__ void __launch_bounds__(kC32) k_coarse32_back(const float2* B1, const float2* B2, float* Fl,
+                                                        const float2* __restrict__ twiddles, int twsh) {
+    chain_wait();
+    const int at = blockIdx.x * kC32 + threadIdx.x;
+    const float2* const B = blockIdx.y ? B2 : B1;
+    float2 tw[kC32 / 2], a[kC32];
+    c32_twiddles(twiddles, twsh, tw);
+#pragma unroll
+    for (int z = 0; z < kC32; ++z) a[z] = B[z * kC32Plane + at];
+    chain_next();   // (as in k_coarse_tiny)
+    autosort<kC32, 1>(a, tw);
+#pragma unroll
+    for (int z = 0; z < kC32; ++z) {
+        if (blockIdx.y == 0) {
+            Fl[z * kC32Plane + at] = a[z].x;
+            Fl[kC32Cells + z * kC32Plane + at] = a[z].y;
+        } else {
+            Fl[2 * kC32Cells + z * kC32Plane + at] = a[z].x;
+        }
+    }
+}
+
+// ------------------------------------------------------------ sparse boxes, 64^3 cells and more
+// Density to delta, Green multiply and F_l around fft.cu's transforms, for steps that
+// keep their bits (keeps_bits): twelve launches, every pass through memory, 73 us at 64^3
+// cells where the fused passes below take 41.
+__global__ void __launch_bounds__(256) k_coarse_delta(int64_t ncells, long long mean, const long long* rho, float2* out) {
+    for (int64_t i = blockIdx.x * (int64_t)blockDim.x + threadIdx.x; i < ncells; i += (int64_t)gridDim.x * blockDim.x)
+        out[i] = make_float2(delta_of(rho[i], mean), 0.f);
+}
+
+__global__ void __launch_bounds__(256) k_coarse_green(int nc, const float4* table, const float2* A, float2* B1, float2* B2) {
+    const int64_t ncells = (int64_t)nc * nc * nc, h = nc / 2 + 1;
+    for (int64_t i = blockIdx.x * (int64_t)blockDim.x + threadIdx.x; i < ncells; i += (int64_t)gridDim.x * blockDim.x) {
+        int ax, ay, az;
+        float sx, sy, sz;
+        kfold((int)(i % nc), nc, ax, sx);
+        kfold((int)((i / nc) % nc), nc, ay, sy);
+        kfold((int)(i / ((int64_t)nc * nc)), nc, az, sz);
+        const float4 g = table[(az * h + ay) * h + ax];
+        const float2 a = A[i];
+        B1[i] = green_times(a, g, sx, sy, sz, true);
+        B2[i] = green_times(a, g, sx, sy, sz, false);
+    }
+}
+
+__global__ void __launch_bounds__(256) k_coarse_extract(int64_t ncells, const float2* B1, const float2* B2, float* Fl) {
+    for (int64_t i = blockIdx.x * (int64_t)blockDim.x + threadIdx.x; i < ncells; i += (int64_t)gridDim.x * blockDim.x) {
+        const float2 b1 = B1[i];
+        Fl[i] = b1.x;
+        Fl[ncells + i] = b1.y;
+        Fl[2 * ncells + i] = B2[i].x;
+    }
+}
+
+// ------------------------------------------------------------ 64^3 cells and more
 // Passes of n = N1 N2 points per pencil in two register steps with one
 // transpose through shared memory (fft.cu).  With j = N2 n1 + n2 and
 // k = k1 + N1 k2 the forward pass ends with all k2 of one k1 in a thread's
 // registers, which is where the inverse one begins: the z pass transforms,
 // multiplies and transforms back without another exchange.  116 bytes a cell
 // over five launches against 212 over twelve: 64^3 cells 73 -> 38 us, 128^3
-// 126 -> 72, 256^3 (HBM-bound) 710 -> 399.  32^3 cells (69 us before) are 32 blocks
-// a pass and 14 us; one launch of three CTAs with the mesh in shared memory: 29 us.
+// 126 -> 72, 256^3 (HBM-bound) 710 -> 399.
 // x: integer density rows -> delta -> spectrum
 template <int N1, int N2>
 __global__ void __launch_bounds__(kPassWidth) k_coarse_fwd_x(long long mean, const long long* __restrict__ rho,
@@ -426,6 +548,28 @@ void launch_tiny(Sim& s, long long mean) {
     chain(s.chained, k_coarse_tiny<N>, 2, N * N, 0, s.stream, mean, s.rho_c, s.green_coarse, s.Fl, s.tw_f, twsh);
     s.launches++;
 }
+void launch_32(Sim& s, long long mean) {
+    int twsh = 0;
+    while ((kC32 << twsh) < s.fft_max) ++twsh;
+    const dim3 both(kC32, 2);
+    chain(s.chained, k_coarse32_plane<-1>, kC32, kC32, 0, s.stream, mean, s.rho_c, s.cA, s.cA, s.tw_f, twsh);
+    chain(s.chained, k_coarse32_green, both, kC32, 0, s.stream, s.green_coarse, s.cA, s.cB1, s.cB2, s.tw_f, twsh);
+    chain(s.chained, k_coarse32_plane<1>, both, kC32, 0, s.stream, 0, nullptr, s.cB1, s.cB2, s.tw_f, twsh);
+    chain(s.chained, k_coarse32_back, both, kC32, 0, s.stream, s.cB1, s.cB2, s.Fl, s.tw_f, twsh);
+    s.launches += 4;
+}
+int launch_kept(Sim& s, long long mean) {
+    const int grid = grid_for(s.ncells, 256);
+    k_coarse_delta<<<grid, 256, 0, s.stream>>>(s.ncells, mean, s.rho_c, s.cA);
+    int rc = fft3d<float>(s, s.cA, s.nc, -1);
+    if (rc) return rc;
+    k_coarse_green<<<grid, 256, 0, s.stream>>>(s.nc, s.green_coarse, s.cA, s.cB1, s.cB2);
+    if ((rc = fft3d<float>(s, s.cB1, s.nc, 1))) return rc;
+    if ((rc = fft3d<float>(s, s.cB2, s.nc, 1))) return rc;
+    k_coarse_extract<<<grid, 256, 0, s.stream>>>(s.ncells, s.cB1, s.cB2, s.Fl);
+    s.launches += 3;
+    return check_launch(s, "coarse force");
+}
 template <int N1, int N2>
 void launch_passes(Sim& s, long long mean) {
     using Q = Pass<N1, N2>;
@@ -457,7 +601,6 @@ int coarse_deposit(Sim& s, bool cleared) {
 }
 
 void coarse_setup() {
-    pass_setup<4, 8>();
     pass_setup<8, 8>();
     pass_setup<8, 16>();
     pass_setup<16, 16>();
@@ -465,13 +608,14 @@ void coarse_setup() {
     pass_setup<32, 32>();
 }
 
-int coarse_force(Sim& s) {
+int coarse_force(Sim& s, bool step) {
     // N 2^27 / nc^3, all powers of two (N up to 2^36)
     const long long mean = s.n >= s.ncells ? (s.n / s.ncells) << 27 : (1ll << 27) / (s.ncells / s.n);
+    if (step && keeps_bits(s) && s.nc > 32) return launch_kept(s, mean);
     switch (s.nc) {
         case 8: launch_tiny<8>(s, mean); break;
         case 16: launch_tiny<16>(s, mean); break;
-        case 32: launch_passes<4, 8>(s, mean); break;
+        case 32: launch_32(s, mean); break;
         case 64: launch_passes<8, 8>(s, mean); break;
         case 128: launch_passes<8, 16>(s, mean); break;
         case 256: launch_passes<16, 16>(s, mean); break;
