@@ -185,9 +185,14 @@ __global__ void __launch_bounds__(kScanThreads) k_scan_apply(int64_t ncells, con
     long long base = 0;
     if (ncells <= kScanDirect) {
         long long part = 0;
-        for (int i = 4 * t; i < (int)b0; i += 4 * kScanThreads) {
-            const int4 c = *reinterpret_cast<const int4*>(counts + i);
-            part += (long long)c.x + c.y + c.z + c.w;
+        if (reinterpret_cast<uintptr_t>(counts) % 16 == 0) {
+            for (int i = 4 * t; i < (int)b0; i += 4 * kScanThreads) {
+                const int4 c = *reinterpret_cast<const int4*>(counts + i);
+                part += (long long)c.x + c.y + c.z + c.w;
+            }
+        } else {   // a caller's counts (pmpm_power_spectrum_noalloc) may start at any int
+#pragma unroll 8
+            for (int i = t; i < (int)b0; i += kScanThreads) part += counts[i];
         }
         block_exclusive_scan(part, sh, base);
     } else if (gridDim.x > kScanFew) {
