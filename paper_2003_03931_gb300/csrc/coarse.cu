@@ -23,7 +23,9 @@ namespace {
 // One thread per coarse cell: the cell's particles reach only the 3^3 nodes
 // around it, so their weights are summed in 27 registers and added to the
 // brick's shared accumulator once per cell.  Bricks of 8 x 8 x 4 cells; boxes up to
-// 32^3 cells take 4^3, four times the blocks (16^3 cells: 64 and not 16).
+// 16^3 cells take 4^3, four times the blocks (64 and not 16: 128^3 particles 158 us against
+// 200 on a GB300, 32^3 11.5 both).  At 32^3 cells they lose, the more the denser: 64^3
+// particles 15.9 us against 12.2, 128^3 54 against 31, 256^3 497 against 232.
 template <int PB, int kBX, int kBY, int kBZ>
 __global__ void __launch_bounds__(kBX * kBY * kBZ) k_coarse_deposit(int nc, const int32_t* __restrict__ counts,
                                                         const int64_t* __restrict__ offsets,
@@ -589,7 +591,7 @@ void launch_passes(Sim& s, long long mean) {
 
 int coarse_deposit(Sim& s, bool cleared) {
     if (!cleared) cudaMemsetAsync(s.rho_c, 0, sizeof(long long) * s.ncells, s.stream);
-    const bool small = s.nc <= 32;
+    const bool small = s.nc <= 16;
     const unsigned nb = (unsigned)(s.ncells / (small ? 64 : 256)), threads = small ? 64 : 256;
     auto k = s.pb == 2 ? (small ? k_coarse_deposit<2, 4, 4, 4> : k_coarse_deposit<2, 8, 8, 4>)
                        : (small ? k_coarse_deposit<1, 4, 4, 4> : k_coarse_deposit<1, 8, 8, 4>);
