@@ -27,11 +27,11 @@ namespace {
 // 200 on a GB300, 32^3 11.5 both).  At 32^3 cells they lose, the more the denser: 64^3
 // particles 15.9 us against 12.2, 128^3 54 against 31, 256^3 497 against 232.
 template <int PB, int kBX, int kBY, int kBZ>
-__global__ void __launch_bounds__(kBX * kBY * kBZ) k_coarse_deposit(int nc, const int32_t* __restrict__ counts,
-                                                        const int64_t* __restrict__ offsets,
-                                                        const uint8_t* __restrict__ m0,
-                                                        const uint8_t* __restrict__ m1,
-                                                        const uint8_t* __restrict__ m2,
+__global__ void __launch_bounds__(kBX * kBY * kBZ) k_coarse_deposit(int nc, const int32_t* counts,
+                                                        const int64_t* offsets,
+                                                        const uint8_t* m0,
+                                                        const uint8_t* m1,
+                                                        const uint8_t* m2,
                                                         unsigned long long* rho) {
     chain_begin();
     constexpr int kNX = kBX + 2, kNY = kBY + 2, kNZ = kBZ + 2;
@@ -165,8 +165,8 @@ __device__ __forceinline__ float2 green_times(float2 a, float4 g, float sx, floa
 }
 
 template <int N>
-__global__ void __launch_bounds__(N * N) k_coarse_tiny(long long mean, const long long* __restrict__ rho,
-                                                       const float4* __restrict__ table, float* __restrict__ Fl,
+__global__ void __launch_bounds__(N * N) k_coarse_tiny(long long mean, const long long* rho,
+                                                       const float4* __restrict__ table, float* Fl,
                                                        const float2* __restrict__ twiddles, int twsh) {
     chain_wait();
     constexpr int P = N + 1, h = N / 2 + 1, cells = N * N * N;
@@ -350,8 +350,8 @@ __global__ void __launch_bounds__(256) k_coarse_extract(int64_t ncells, const fl
 // 126 -> 72, 256^3 (HBM-bound) 710 -> 399.
 // x: integer density rows -> delta -> spectrum
 template <int N1, int N2>
-__global__ void __launch_bounds__(kPassWidth) k_coarse_fwd_x(long long mean, const long long* __restrict__ rho,
-                                                                 float2* __restrict__ out,
+__global__ void __launch_bounds__(kPassWidth) k_coarse_fwd_x(long long mean, const long long* rho,
+                                                                 float2* out,
                                                                  const float2* __restrict__ tw, int twsh) {
     chain_begin();
     using Q = Pass<N1, N2>;
@@ -426,8 +426,8 @@ __global__ void __launch_bounds__(kPassWidth) k_coarse_y(float2* d0, float2* d1,
 // z: forward, Green multiply and back for B1 and B2
 template <int N1, int N2>
 __global__ void __launch_bounds__(kPassWidth) k_coarse_z(const float4* __restrict__ table,
-                                                             const float2* __restrict__ A, float2* __restrict__ B1,
-                                                             float2* __restrict__ B2, const float2* __restrict__ tw,
+                                                             const float2* A, float2* B1,
+                                                             float2* B2, const float2* __restrict__ tw,
                                                              int twsh) {
     chain_begin();
     using Q = Pass<N1, N2>;
@@ -493,9 +493,9 @@ __global__ void __launch_bounds__(kPassWidth) k_coarse_z(const float4* __restric
 
 // x: back to F_x + i F_y (blockIdx.y = 0) and F_z
 template <int N1, int N2>
-__global__ void __launch_bounds__(kPassWidth) k_coarse_inv_x(const float2* __restrict__ B1,
-                                                                 const float2* __restrict__ B2,
-                                                                 float* __restrict__ Fl,
+__global__ void __launch_bounds__(kPassWidth) k_coarse_inv_x(const float2* B1,
+                                                                 const float2* B2,
+                                                                 float* Fl,
                                                                  const float2* __restrict__ tw, int twsh) {
     chain_wait();
     using Q = Pass<N1, N2>;

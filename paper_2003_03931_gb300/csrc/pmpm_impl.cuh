@@ -142,7 +142,9 @@ void chain(bool ahead, void (*kernel)(P...), dim3 grid, unsigned block, size_t s
 }
 
 // First thing in a kernel launched by chain(): nothing of memory is touched before
-// the kernels before it are complete.
+// the kernels before it are complete.  What they write such a kernel reads through plain
+// pointers: const __restrict__ would promise that nothing writes there while it lives,
+// and it lives already.
 __device__ __forceinline__ void chain_wait() { asm volatile("griddepcontrol.wait;" ::: "memory"); }
 // The stream's next kernel may come in, to wait.  After chain_wait(), so that a kernel
 // two places on cannot run ahead of this one.

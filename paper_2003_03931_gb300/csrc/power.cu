@@ -88,7 +88,7 @@ __device__ __forceinline__ int pk_row(const PkStore& st, int64_t base, int x, bo
 // 1-byte unit (2U_1)^-3.
 template <int PB, int LH, bool SMALL, typename OUT>
 __global__ void __launch_bounds__(Brick<LH, SMALL>::kThreads) k_pk_deposit(const PkStore st, PkMean mean,
-                                                                           OUT* __restrict__ out) {
+                                                                           OUT* out) {
     chain_begin();
     using B = Brick<LH, SMALL>;
     using F = PosFmt<PB>;
@@ -290,9 +290,9 @@ __device__ __forceinline__ double limbs_value(uint32_t l0, uint32_t l1, uint32_t
 // the imaginary part of one plane: half the points.  The z pass takes them apart again.
 // x; clears the sums that the z pass adds to
 template <int N1, int N2>
-__global__ void __launch_bounds__(kPassWidth) k_pk_x(const float* __restrict__ delta, float2* __restrict__ mesh,
-                                                     int nbins, double* __restrict__ bins,
-                                                     const uint32_t* __restrict__ err,
+__global__ void __launch_bounds__(kPassWidth) k_pk_x(const float* delta, float2* mesh,
+                                                     int nbins, double* bins,
+                                                     const uint32_t* err,
                                                      const float2* __restrict__ tw, int twsh) {
     chain_begin();
     using Q = Pass<N1, N2>;
@@ -370,8 +370,8 @@ __device__ __forceinline__ float block_max(float v, float* sh) {
 // past n/2 are left out.
 template <int N1, int N2>
 __global__ void __launch_bounds__(kPassWidth) k_pk_z(int nbins, double norm, double kf,
-                                                     const float2* __restrict__ mesh,
-                                                     double* __restrict__ bins, const float2* __restrict__ tw,
+                                                     const float2* mesh,
+                                                     double* bins, const float2* __restrict__ tw,
                                                      int twsh) {
     chain_begin();
     using Q = Pass<N1, N2>;
@@ -463,9 +463,9 @@ struct PkSmall {
 
 template <int N>
 __global__ void __launch_bounds__(PkSmall<N>::kThreads) k_pk_small(int nbins, double norm, double kf,
-                                                                   const float* __restrict__ delta,
-                                                                   double* __restrict__ bins,
-                                                                   const uint32_t* __restrict__ err) {
+                                                                   const float* delta,
+                                                                   double* bins,
+                                                                   const uint32_t* err) {
     chain_begin();
     using M = PkSmall<N>;
     constexpr int H = M::kH, P = M::kP, T = M::kThreads, L = M::kLog;

@@ -53,8 +53,8 @@ __device__ __forceinline__ long long block_exclusive_scan(long long v, long long
     return before + x - v;
 }
 
-__global__ void __launch_bounds__(kScanThreads) k_scan_reduce(int64_t ncells, const int32_t* __restrict__ counts,
-                                                              long long* __restrict__ blocksums, int items) {
+__global__ void __launch_bounds__(kScanThreads) k_scan_reduce(int64_t ncells, const int32_t* counts,
+                                                              long long* blocksums, int items) {
     chain_begin();
     __shared__ long long sh[32];
     const int64_t b0 = (int64_t)blockIdx.x * kScanThreads * items;
@@ -136,16 +136,16 @@ constexpr int64_t kScanDirect = 32768;
 // U = sum over cells and axes of floor(S^2 / n), into the digits d2[4..7]; the
 // last block done (d2[8] counts them; none waits) writes sigma.  Scan, means and
 // dispersion of a step, with separate passes over counts and S before: 16^3
-// cells 43 -> 10 us (one launch), 64^3 46 -> 21, 256^3 625 -> 363 (of 48 B a
+// cells 43 -> 10 us (one launch), 64^3 46 -> 21, 256^3 625 -> 343 (of 48 B a
 // cell: 119 us at the copy bandwidth; the divisions bound it).
 template <bool MEANS, int ITEMS>
-__global__ void __launch_bounds__(kScanThreads) k_scan_apply(int64_t ncells, const int32_t* __restrict__ counts,
-                                                             const long long* __restrict__ blocksums,
-                                                             int64_t* __restrict__ offsets, int64_t n,
+__global__ void __launch_bounds__(kScanThreads) k_scan_apply(int64_t ncells, const int32_t* counts,
+                                                             const long long* blocksums,
+                                                             int64_t* offsets, int64_t n,
                                                              uint32_t* err,
-                                                             const unsigned long long* __restrict__ S,
-                                                             float* __restrict__ vc, int32_t* __restrict__ fill,
-                                                             unsigned long long* d2, float* __restrict__ sigma) {
+                                                             const unsigned long long* S,
+                                                             float* vc, int32_t* fill,
+                                                             unsigned long long* d2, float* sigma) {
     chain_begin();
     constexpr int kTile = kScanThreads * ITEMS;
     __shared__ long long sh[32];
@@ -163,19 +163,21 @@ __global__ void __launch_bounds__(kScanThreads) k_scan_apply(int64_t ncells, con
     // cell means, dispersion and slot counters, in the striped order
     unsigned long long lo = 0, hi = 0;
     if (MEANS) {
+        long long s[ITEMS][3];
+#pragma unroll
+        for (int k = 0; k < ITEMS; ++k)
+#pragma unroll
+            for (int d = 0; d < 3; ++d) s[k][d] = (long long)S[d * ncells + b0 + k * kScanThreads + t];
 #pragma unroll
         for (int k = 0; k < ITEMS; ++k) {
             const int64_t i = b0 + k * kScanThreads + t;
             fill[i] = 0;
-            long long s[3];
-#pragma unroll
-            for (int d = 0; d < 3; ++d) s[d] = (long long)S[d * ncells + i];
 #pragma unroll
             for (int d = 0; d < 3; ++d) {
                 float v = 0.f;
                 if (cst[k] > 0) {
-                    v = __fdiv_rn(__fmul_rn(__ll2float_rn(s[d]), 0x1p-24f), (float)cst[k]);
-                    add_square_over_n128(s[d], cst[k], lo, hi);
+                    v = __fdiv_rn(__fmul_rn(__ll2float_rn(s[k][d]), 0x1p-24f), (float)cst[k]);
+                    add_square_over_n128(s[k][d], cst[k], lo, hi);
                 }
                 vc[d * ncells + i] = v;
             }
@@ -342,8 +344,8 @@ template <int PB>
 __device__ __forceinline__ void scatter_two(const int32_t (&q)[2][3], const float (&p)[2][3],
                                             const bool (&live)[2], int64_t n, int nc,
                                             const float* const (&vcd)[3],
-                                            const int64_t* __restrict__ offsets, int32_t* fill,
-                                            float sigma, const float* Es, uint8_t* __restrict__ out,
+                                            const int64_t* offsets, int32_t* fill,
+                                            float sigma, const float* Es, uint8_t* out,
                                             uint32_t* err) {
     const int lane = threadIdx.x & 31;
     int64_t off[2], end[2];
@@ -385,10 +387,10 @@ __device__ __forceinline__ void scatter_two(const int32_t (&q)[2][3], const floa
 // Re-encode (Eq. 2-3) of the particles a source gives, in any order.  Each
 // warp handles two particles per lane at a time.
 template <int PB, class Src>
-__global__ void k_scatter(Src src, int64_t n, int nc, const float* __restrict__ vc,
-                          const int64_t* __restrict__ offsets, int32_t* fill,
-                          const float* __restrict__ sigma_p, const float* __restrict__ E,
-                          uint8_t* __restrict__ out, uint32_t* err) {
+__global__ void k_scatter(Src src, int64_t n, int nc, const float* vc,
+                          const int64_t* offsets, int32_t* fill,
+                          const float* sigma_p, const float* __restrict__ E,
+                          uint8_t* out, uint32_t* err) {
     chain_begin();
     const int64_t ncells = (int64_t)nc * nc * nc;
     const float sigma = *sigma_p;
@@ -430,12 +432,12 @@ constexpr int kParkSpan = 64;   // particles per warp iteration (two per lane)
 // cell comes from a window of 32 old offsets, one per lane, searched
 // through shuffles (the next window only where a particle lies beyond it).
 __global__ void __launch_bounds__(kParkThreads, 4)
-k_scatter_parked(int64_t n, int nc, const int64_t* __restrict__ offs_old,
-                 const uint8_t* __restrict__ st_old, const float* __restrict__ Pn,
-                 const float* __restrict__ kd, const float* __restrict__ vc,
-                 const int64_t* __restrict__ offsets, int32_t* fill,
-                 const float* __restrict__ sigma_p, const float* __restrict__ E,
-                 uint8_t* __restrict__ out, uint32_t* err) {
+k_scatter_parked(int64_t n, int nc, const int64_t* offs_old,
+                 const uint8_t* st_old, const float* Pn,
+                 const float* kd, const float* vc,
+                 const int64_t* offsets, int32_t* fill,
+                 const float* sigma_p, const float* __restrict__ E,
+                 uint8_t* out, uint32_t* err) {
     chain_begin();
     __shared__ float Es[256];
     const int tid = threadIdx.x, lane = tid & 31;
