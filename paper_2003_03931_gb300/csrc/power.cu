@@ -11,8 +11,8 @@
 //            all of it (k_pk_small).
 //   shells   mean |k| and the number of modes follow from the mesh alone: integer
 //            arithmetic, one block a shell
-// FP64 runs at 1/64 of the FP32 rate here, so shell sums are exact integers of
-// 21-bit limbs of the float32 squares, and only a block's totals become doubles.
+// FP64 runs at 1/64 of the FP32 rate here, so squares and shell sums are integers
+// (pk_sums.cuh) and only a block's totals become doubles.
 //
 // On a GB300: 256^3 particles on 512^3 points 10.5 -> 1.37 ms (a search per
 // particle, 64-bit global atomics and three double shared atomics a mode before):
@@ -25,6 +25,7 @@
 #include <new>
 
 #include "fftpass.cuh"
+#include "pk_sums.cuh"
 
 namespace pmpm {
 
@@ -265,24 +266,12 @@ __global__ void __launch_bounds__(kPassWidth) k_pk_shells(int nmesh, int nbins, 
     block_shell(nmesh, nbins, blockIdx.x + 1, kf, bins);
 }
 
-// Adds a float32 v >= 0 to a shell as an integer: 62 bits under the largest
-// exponent emax of what is added, in three limbs of 21 bits.  A limb takes 2048
-// values.
-__device__ __forceinline__ void add_limbs(uint32_t* limb, int stride, float v, int emax) {
-    const uint32_t b = __float_as_uint(v);
-    if (b < 0x00800000u) return;   // zero (or below 2^-126)
-    const int sh = 38 - (emax - (int)(b >> 23));
-    if (sh < -24) return;
-    const uint32_t m = (b & 0x7fffffu) | 0x800000u;
-    const unsigned long long x = sh >= 0 ? (unsigned long long)m << sh : (m + (1u << (-sh - 1))) >> -sh;
-    const uint32_t l0 = (uint32_t)x & 0x1fffffu, l1 = (uint32_t)(x >> 21) & 0x1fffffu, l2 = (uint32_t)(x >> 42);
-    if (l0) smem_red(limb, l0);
-    if (l1) smem_red(limb + stride, l1);
-    if (l2) smem_red(limb + 2 * stride, l2);
-}
-__device__ __forceinline__ double limbs_value(uint32_t l0, uint32_t l1, uint32_t l2, int emax) {
-    const double v = (double)((unsigned long long)l0 + ((unsigned long long)l1 << 21)) + (double)l2 * 4398046511104.0;
-    return ldexp(v, emax - 188);
+// Adds an integer of up to 62 bits to a shell (pk_sums.cuh).
+__device__ __forceinline__ void add_limbs(uint32_t* limb, int stride, unsigned long long x) {
+    const Limbs l = limbs_of(x);
+    if (l.v[0]) smem_red(limb, l.v[0]);
+    if (l.v[1]) smem_red(limb + stride, l.v[1]);
+    if (l.v[2]) smem_red(limb + 2 * stride, l.v[2]);
 }
 
 // ------------------------------------------------------------ transforms
@@ -408,19 +397,16 @@ __global__ void __launch_bounds__(kPassWidth) k_pk_z(int nbins, double norm, dou
             pass_first<N1, N2>(a, Y, p, n2, tw, twsh);
         }
         __syncthreads();
-        const float weight = ky == 0 || ky == h ? 1.f : 2.f;
-        float v[kItems][N2], big = 0.f;
+        const int twice = ky == 0 || ky == h ? 0 : 1;
+        float2 a[kItems][N2];
+        float big = 0.f;
 #pragma unroll
         for (int u = 0; u < kItems; ++u) {
             const int it = tid + u * kPassWidth, p = it & (Q::P - 1), k1 = it >> Q::LP;
             if (it < Q::P * N1) {
-                float2 a[N2];
-                pass_second<N1, N2>(a, Y, p, k1);
+                pass_second<N1, N2>(a[u], Y, p, k1);
 #pragma unroll
-                for (int k2 = 0; k2 < N2; ++k2) {
-                    v[u][k2] = weight * (a[k2].x * a[k2].x + a[k2].y * a[k2].y);
-                    big = fmaxf(big, v[u][k2]);
-                }
+                for (int k2 = 0; k2 < N2; ++k2) big = fmaxf(big, fmaxf(fabsf(a[u][k2].x), fabsf(a[u][k2].y)));
             }
         }
         const int emax = (int)(__float_as_uint(block_max(big, mx)) >> 23);
@@ -434,7 +420,9 @@ __global__ void __launch_bounds__(kPassWidth) k_pk_z(int nbins, double norm, dou
                 for (int k2 = 0; k2 < N2; ++k2) {
                     const int kz = k1 + N1 * k2, nz = kz < h ? kz : kz - Q::n;
                     const int j = shell_of(m0 + nz * nz);
-                    if (j >= 1 && j <= nbins) add_limbs(limb + j, h + 1, v[u][k2], emax);
+                    if (j >= 1 && j <= nbins)
+                        add_limbs(limb + j, h + 1,
+                                  (square_of<12>(a[u][k2].x, emax) + square_of<12>(a[u][k2].y, emax)) << twice);
                 }
             }
         }
@@ -442,7 +430,7 @@ __global__ void __launch_bounds__(kPassWidth) k_pk_z(int nbins, double norm, dou
         for (int j = tid; j <= nbins; j += kPassWidth) {
             uint32_t* l = limb + j;
             if (l[0] | l[h + 1] | l[2 * (h + 1)]) {
-                acc[j] += limbs_value(l[0], l[h + 1], l[2 * (h + 1)], emax);
+                acc[j] += limbs_value<12>(l[0], l[h + 1], l[2 * (h + 1)], emax);
                 l[0] = l[h + 1] = l[2 * (h + 1)] = 0u;
             }
         }
@@ -515,38 +503,39 @@ __global__ void __launch_bounds__(PkSmall<N>::kThreads) k_pk_small(int nbins, do
         for (int k = 0; k < N; ++k) col[k * (N * P)] = a[k];
     }
     __syncthreads();
-    // |delta~|^2 (times 4) of mode kz at this kx (twice: its mirror image too), and
-    // for kx = 0 at kx = 0 and N/2: A = (Z + conj Z') / 2, B = (Z - conj Z') / 2i, Z' at
+    // The modes at kz of this kx (they stand for their mirror images too), or for kx = 0
+    // those of kx = 0 and N/2, times two: 2 A = Z + conj Z', 2 B = -i (Z - conj Z'), Z' at
     // (-ky, -kz)
-    auto square = [&](int k, float& at0, float& atH) {
+    auto modes = [&](int k, float2& at0, float2& atH) {
+        at0 = a[k];
+        atH = make_float2(0.f, 0.f);
         if (kx == 0) {
             const float2 b = C[((N - ky) & (N - 1)) * P + ((N - k) & (N - 1)) * (N * P)];
-            const float px = a[k].x + b.x, py = a[k].y - b.y, qx = a[k].x - b.x, qy = a[k].y + b.y;
-            at0 = 0.25f * (px * px + py * py);
-            atH = 0.25f * (qx * qx + qy * qy);
-        } else {
-            at0 = 2.f * (a[k].x * a[k].x + a[k].y * a[k].y);
-            atH = 0.f;
+            at0 = make_float2(a[k].x + b.x, a[k].y - b.y);
+            atH = make_float2(a[k].x - b.x, a[k].y + b.y);
         }
     };
     float big = 0.f;
 #pragma unroll
     for (int k = 0; k < N; ++k) {
-        float v, w;
-        square(k, v, w);
-        big = fmaxf(big, fmaxf(v, w));
+        float2 v, w;
+        modes(k, v, w);
+        big = fmaxf(big, fmaxf(fmaxf(fabsf(v.x), fabsf(v.y)), fmaxf(fabsf(w.x), fabsf(w.y))));
     }
-    const int emax = (int)(__float_as_uint(block_max(big, mx)) >> 23);
+    // |delta~|^2 times 16 (rfftx2 doubles, and so does `modes` at kx = 0)
+    const int emax = (int)(__float_as_uint(block_max(big, mx)) >> 23), times8 = kx == 0 ? 0 : 3;
 #pragma unroll
     for (int k = 0; k < N; ++k) {
-        float v, w;
-        square(k, v, w);
+        float2 v, w;
+        modes(k, v, w);
         const int nz = k < H ? k : k - N, m = kx * kx + ny * ny + nz * nz;
         const int j = shell_of(m);
-        if (j >= 1 && j <= nbins) add_limbs(&limb[0][kx][j], H * (H + 1), v, emax);
+        if (j >= 1 && j <= nbins)
+            add_limbs(&limb[0][kx][j], H * (H + 1), (square_of<10>(v.x, emax) + square_of<10>(v.y, emax)) << times8);
         if (kx == 0) {
             const int i = shell_of(m + H * H);
-            if (i <= nbins) add_limbs(&limb[0][0][i], H * (H + 1), w, emax);
+            if (i <= nbins)
+                add_limbs(&limb[0][0][i], H * (H + 1), square_of<10>(w.x, emax) + square_of<10>(w.y, emax));
         }
     }
     __syncthreads();
@@ -561,8 +550,7 @@ __global__ void __launch_bounds__(PkSmall<N>::kThreads) k_pk_small(int nbins, do
         for (int e = 0; e < 6; ++e) s[e] = warp_sum(s[e]);
         if (lane == 0) {
             // limbs of up to 8 kx: s[2] below 2^35
-            const double v = (double)(s[0] + (s[1] << 21)) + (double)s[2] * 4398046511104.0;
-            bins[j - 1] = ldexp(0.25 * norm * v, emax - 188);   // rfftx2 doubles
+            bins[j - 1] = 0.0625 * norm * limbs_value<10>(s[0], s[1], s[2], emax);
             bins[nbins + j - 1] = kf * ((double)s[3] * 0x1p-14 + (double)s[4] * 0x1p-40);
             bins[2 * nbins + j - 1] = (double)s[5];
         }
