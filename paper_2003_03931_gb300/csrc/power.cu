@@ -9,8 +9,8 @@
 //   x, y, z  register transforms (fftpass.cuh); the z pass adds |delta~|^2 to its
 //            block's shells and writes nothing.  Up to 16^3 points one CTA does
 //            all of it (k_pk_small).
-//   shells   mean |k| and the number of modes follow from the mesh alone: integer
-//            arithmetic, one block a shell
+//   shells   mean |k| and the number of modes follow from the mesh alone: modes counted
+//            by |n|^2, one block a shell
 // FP64 runs at 1/64 of the FP32 rate here, so squares and shell sums are integers
 // (pk_sums.cuh) and only a block's totals become doubles.
 //
@@ -199,15 +199,11 @@ __device__ __forceinline__ int isqrt(int v) {   // floor, v >= 0
     return r;
 }
 
-// Sum of |n| and number of the modes of shell j of an nmesh^3 mesh, over the
-// lanes of warp w of W: octant points (a, b, c), a <= b, with their multiplicities.
-// sqrt(m) = s + e: s the float32 root, e its first-order remainder (the second
-// order is 1e-13 of it); both are added as integers, of 2^-14 and of 2^-40 (e and
-// what s has beyond 2^-14).
-__device__ __forceinline__ void shell_sums(int nmesh, int j, int w, int W, int lane, long long& hi, long long& lo,
-                                           long long& modes) {
+// Modes of shell j of an nmesh^3 mesh by |n|^2: adds to hist[m - (j^2 - j + 1)], m up to
+// j^2 + j, by the lanes of warp w of W.  Octant points (a, b, c), a <= b, with their
+// multiplicities.  A root per m is left, 2 j of them, and not one per mode: in float64.
+__device__ __forceinline__ void count_shell(int nmesh, int j, int w, int W, int lane, uint32_t* hist) {
     const int h = nmesh / 2, mlo = j * j - j + 1, mhi = j * j + j, side = min(h, j);
-    hi = lo = modes = 0;
     for (int b = w; b <= side; b += W) {
         for (int a = lane; a <= b; a += 32) {
             const int m0 = a * a + b * b;
@@ -219,51 +215,56 @@ __device__ __forceinline__ void shell_sums(int nmesh, int j, int w, int W, int l
                 c0 = isqrt(mlo - m0);
                 if (c0 * c0 < mlo - m0) ++c0;
             }
-            for (int c = c0; c <= c1; ++c) {
-                const int k = mult * (c == 0 || c == h ? 1 : 2);
-                const float m = (float)(m0 + c * c);   // below 2^24 (j <= 2048): exact
-                const float s = root(m);
-                const float e = __fdividef(__fmaf_rn(-s, s, m), 2.f * s);
-                const int whole = (int)(s * 16384.f);
-                const float rest = __fmaf_rn((float)whole, -0x1p-14f, s);
-                hi += (long long)(k * whole);          // 16 x 2^25
-                lo += (long long)k * (__float2int_rn(rest * 0x1p40f) + __float2int_rn(e * 0x1p40f));
-                modes += k;
-            }
+            for (int c = c0; c <= c1; ++c) smem_red(&hist[m0 + c * c - mlo], mult * (c == 0 || c == h ? 1 : 2));
         }
     }
 }
-__device__ __forceinline__ long long warp_sum(long long v) {
+template <typename V>
+__device__ __forceinline__ V warp_sum(V v) {
 #pragma unroll
     for (int o = 16; o > 0; o >>= 1) v += __shfl_xor_sync(0xffffffffu, v, o);
     return v;
 }
 
-// k and mode sums of shell j, by one block
-__device__ __forceinline__ void block_shell(int nmesh, int nbins, int j, double kf, double* bins) {
-    __shared__ long long sh[3][kPassWidth / 32];
-    long long s[3];
-    shell_sums(nmesh, j, threadIdx.x >> 5, kPassWidth / 32, threadIdx.x & 31, s[0], s[1], s[2]);
-#pragma unroll
-    for (int e = 0; e < 3; ++e) {
-        s[e] = warp_sum(s[e]);
-        if ((threadIdx.x & 31) == 0) sh[e][threadIdx.x >> 5] = s[e];
+// k and mode sums of shell j, by one block; hist: 2 j words of shared memory
+__device__ __forceinline__ void block_shell(int nmesh, int nbins, int j, double kf, double* bins, uint32_t* hist) {
+    __shared__ double shk[kPassWidth / 32];
+    __shared__ int shm[kPassWidth / 32];
+    const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5, mlo = j * j - j + 1;
+    for (int i = tid; i < 2 * j; i += kPassWidth) hist[i] = 0u;
+    __syncthreads();
+    count_shell(nmesh, j, warp, kPassWidth / 32, lane, hist);
+    __syncthreads();
+    double k = 0.0;
+    int modes = 0;
+    for (int i = tid; i < 2 * j; i += kPassWidth) {
+        k += (double)hist[i] * __dsqrt_rn((double)(mlo + i));
+        modes += (int)hist[i];
+    }
+    k = warp_sum(k);
+    modes = warp_sum(modes);
+    if (lane == 0) {
+        shk[warp] = k;
+        shm[warp] = modes;
     }
     __syncthreads();
-    if (threadIdx.x == 0) {
-        for (int w = 1; w < kPassWidth / 32; ++w)
-            for (int e = 0; e < 3; ++e) s[e] += sh[e][w];
-        bins[nbins + j - 1] = kf * ((double)s[0] * 0x1p-14 + (double)s[1] * 0x1p-40);
-        bins[2 * nbins + j - 1] = (double)s[2];
+    if (tid == 0) {
+        for (int w = 1; w < kPassWidth / 32; ++w) {
+            k += shk[w];
+            modes += shm[w];
+        }
+        bins[nbins + j - 1] = kf * k;
+        bins[2 * nbins + j - 1] = (double)modes;
     }
     __syncthreads();
 }
 
-// for meshes whose shells are not the z pass's
+// for meshes whose shells are not the z pass's; nmesh words of shared memory
 __global__ void __launch_bounds__(kPassWidth) k_pk_shells(int nmesh, int nbins, double kf, double* __restrict__ bins,
                                                           const uint32_t* __restrict__ err) {
+    extern __shared__ uint32_t shell_smem[];
     if (blockIdx.x == 0 && threadIdx.x == 0) bins[3 * nbins] = (double)*err;
-    block_shell(nmesh, nbins, blockIdx.x + 1, kf, bins);
+    block_shell(nmesh, nbins, blockIdx.x + 1, kf, bins, shell_smem);
 }
 
 // Adds an integer of up to 62 bits to a shell (pk_sums.cuh).
@@ -373,7 +374,7 @@ __global__ void __launch_bounds__(kPassWidth) k_pk_z(int nbins, double norm, dou
     float* mx = reinterpret_cast<float*>(limb + 3 * (h + 1));
     float2* Y = reinterpret_cast<float2*>(mx + 33);   // 8-byte aligned: h + 1 is odd
     const int tid = threadIdx.x;
-    for (int j = 1 + blockIdx.x; j <= nbins; j += gridDim.x) block_shell(Q::n, nbins, j, kf, bins);
+    for (int j = 1 + blockIdx.x; j <= nbins; j += gridDim.x) block_shell(Q::n, nbins, j, kf, bins, reinterpret_cast<uint32_t*>(Y));
     for (int j = tid; j <= h; j += kPassWidth) {
         acc[j] = 0.0;
         limb[j] = limb[h + 1 + j] = limb[2 * (h + 1) + j] = 0u;
@@ -460,7 +461,7 @@ __global__ void __launch_bounds__(PkSmall<N>::kThreads) k_pk_small(int nbins, do
     extern __shared__ __align__(16) unsigned char pass_smem[];
     float2* C = reinterpret_cast<float2*>(pass_smem);
     float* R = reinterpret_cast<float*>(pass_smem);
-    __shared__ uint32_t limb[3][H][H + 1];
+    __shared__ uint32_t limb[3][H][H + 1], hist[T / 32][N];
     __shared__ float mx[32];
     const int tid = threadIdx.x;
     if (tid == 0) bins[3 * nbins] = (double)*err;
@@ -542,17 +543,22 @@ __global__ void __launch_bounds__(PkSmall<N>::kThreads) k_pk_small(int nbins, do
     // a warp per shell: its limbs over kx, and the mesh's own sums
     const int lane = tid & 31;
     for (int j = 1 + (tid >> 5); j <= nbins; j += T / 32) {
-        long long s[6];
+        long long s[3];
 #pragma unroll
-        for (int e = 0; e < 3; ++e) s[e] = lane < H ? limb[e][lane][j] : 0;
-        shell_sums(N, j, 0, 1, lane, s[3], s[4], s[5]);
-#pragma unroll
-        for (int e = 0; e < 6; ++e) s[e] = warp_sum(s[e]);
+        for (int e = 0; e < 3; ++e) s[e] = warp_sum(lane < H ? (long long)limb[e][lane][j] : 0ll);
+        uint32_t* const count = hist[tid >> 5];
+        if (lane < N) count[lane] = 0u;
+        __syncwarp();
+        count_shell(N, j, 0, 1, lane, count);
+        __syncwarp();
+        const int m = j * j - j + 1 + lane, n = lane < 2 * j ? (int)count[lane] : 0;
+        const double k = warp_sum((double)n * __dsqrt_rn((double)m));
+        const int modes = warp_sum(n);
+        __syncwarp();
         if (lane == 0) {
-            // limbs of up to 8 kx: s[2] below 2^35
             bins[j - 1] = 0.0625 * norm * limbs_value<10>(s[0], s[1], s[2], emax);
-            bins[nbins + j - 1] = kf * ((double)s[3] * 0x1p-14 + (double)s[4] * 0x1p-40);
-            bins[2 * nbins + j - 1] = (double)s[5];
+            bins[nbins + j - 1] = kf * k;
+            bins[2 * nbins + j - 1] = (double)modes;
         }
     }
 }
@@ -691,7 +697,7 @@ cudaError_t pk_enqueue(cudaStream_t stream, const PkStore& st, int nmesh, int nb
     else if (nmesh == 1024) launch_transforms<32, 32>(stream, st.chained, nbins, norm, kf, mesh, real, bins, err, tw, tw_n);
     else {
         cudaMemsetAsync(bins, 0, sizeof(double) * nbins, stream);
-        k_pk_shells<<<nbins, kPassWidth, 0, stream>>>(nmesh, nbins, kf, bins, err);
+        k_pk_shells<<<nbins, kPassWidth, sizeof(uint32_t) * nmesh, stream>>>(nmesh, nbins, kf, bins, err);
         const cudaError_t e = fft3d_float_raw(stream, mesh, nmesh, -1, tw, tw_n);
         if (e != cudaSuccess) return e;
         k_pk_modes<<<grid_for(m3, kPassWidth, 152 * 4), kPassWidth, sizeof(double) * (nbins + 1), stream>>>(
