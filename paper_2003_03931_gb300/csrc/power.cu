@@ -86,7 +86,18 @@ __device__ __forceinline__ int pk_row(const PkStore& st, int64_t base, int x, bo
 // low word's wraps are counted in the high word.  A warp takes a row of cells (x
 // fastest, CX + 2 of them), its particles 32 at a time; the cell of each comes from
 // the row's prefix counts, one per lane.  2-byte products are rounded to the
-// 1-byte unit (2U_1)^-3.
+// 1-byte unit (2U_1)^-3.  Cells of more than kPkCrowd particles are the whole block's, one
+// after another, four particles a thread at a time: a warp would walk a row for as long as
+// its fullest cell is (128^3 particles, 20000 of them in one cell: CROWD).
+constexpr int kPkCrowd = 1024;
+template <int PB>
+struct PackedBins {
+    using type = uint32_t;
+};
+template <>
+struct PackedBins<2> {
+    using type = unsigned long long;
+};
 template <int PB, int LH, bool SMALL, typename OUT>
 __global__ void __launch_bounds__(Brick<LH, SMALL>::kThreads) k_pk_deposit(const PkStore st, PkMean mean,
                                                                            OUT* out) {
@@ -113,10 +124,37 @@ __global__ void __launch_bounds__(Brick<LH, SMALL>::kThreads) k_pk_deposit(const
         most = max(most, pk_row(st, row_base(row), x0 - 1 + lane, lane < B::CX + 2, off));
     }
     const bool safe = !__syncthreads_or(most > B::kSafe);
+    // particle of cell (bx, by, bz) with bins m to its nodes
+    auto cloud = [&](int bx, int by, int bz, const int (&m)[3]) {
+        const int sx = (bx - 1) * 2 * F::kBins + 2 * m[0] + 1 - U;
+        const int sy = (by - 1) * 2 * F::kBins + 2 * m[1] + 1 - U;
+        const int sz = (bz - 1) * 2 * F::kBins + 2 * m[2] + 1 - U;
+        const int ix = sx >> LW, iy = sy >> LW, iz = sz >> LW;
+        if ((unsigned)(ix + 1) > (unsigned)B::NX || (unsigned)(iy + 1) > (unsigned)B::NY ||
+            (unsigned)(iz + 1) > (unsigned)B::NZ)
+            return;
+        const int wx = sx & (W - 1), wy = sy & (W - 1), wz = sz & (W - 1);
+#pragma unroll
+        for (int c = 0; c < 8; ++c) {
+            const int dx = c & 1, dy = (c >> 1) & 1, dz = c >> 2;
+            const int x = ix + dx, y = iy + dy, z = iz + dz;
+            const uint32_t w = cic_weight3<PB>(dx ? wx : W - wx, dy ? wy : W - wy, dz ? wz : W - wz);
+            if ((unsigned)x < (unsigned)B::NX && (unsigned)y < (unsigned)B::NY && (unsigned)z < (unsigned)B::NZ) {
+                const int i = x + B::NX * (y + B::NY * z);
+                if (safe) {
+                    smem_red(&lo[i], w);
+                } else {
+                    const uint32_t old = atomicAdd(&lo[i], w);
+                    if (old + w < old) atomicAdd(&hi[i], 1u);
+                }
+            }
+        }
+    };
     for (int row = warp; row < kRows; row += T / 32) {
         const int by = row % (B::CY + 2), bz = row / (B::CY + 2);
         int64_t off;
-        const int cnt = pk_row(st, row_base(row), x0 - 1 + lane, lane < B::CX + 2, off);
+        int cnt = pk_row(st, row_base(row), x0 - 1 + lane, lane < B::CX + 2, off);
+        if (cnt > kPkCrowd) cnt = 0;
         int incl = cnt;
 #pragma unroll
         for (int o = 1; o < 16; o <<= 1) {
@@ -133,26 +171,37 @@ __global__ void __launch_bounds__(Brick<LH, SMALL>::kThreads) k_pk_deposit(const
             for (int k = 1; k < B::CX + 2; ++k) bx += v >= __shfl_sync(0xffffffffu, pre, k) ? 1 : 0;
             const int64_t j = __shfl_sync(0xffffffffu, rel, bx) + v;
             if (v >= total) continue;
-            const int sx = (bx - 1) * 2 * F::kBins + 2 * load_bin<PB>(st.m[0], j) + 1 - U;
-            const int sy = (by - 1) * 2 * F::kBins + 2 * load_bin<PB>(st.m[1], j) + 1 - U;
-            const int sz = (bz - 1) * 2 * F::kBins + 2 * load_bin<PB>(st.m[2], j) + 1 - U;
-            const int ix = sx >> LW, iy = sy >> LW, iz = sz >> LW;
-            if ((unsigned)(ix + 1) > (unsigned)B::NX || (unsigned)(iy + 1) > (unsigned)B::NY ||
-                (unsigned)(iz + 1) > (unsigned)B::NZ)
-                continue;
-            const int wx = sx & (W - 1), wy = sy & (W - 1), wz = sz & (W - 1);
+            const int m[3] = {load_bin<PB>(st.m[0], j), load_bin<PB>(st.m[1], j), load_bin<PB>(st.m[2], j)};
+            cloud(bx, by, bz, m);
+        }
+    }
+    if (__syncthreads_or(most > kPkCrowd)) {
+        for (int row = 0; row < kRows; ++row) {
+            int64_t off;
+            const int cnt = pk_row(st, row_base(row), x0 - 1 + lane, lane < B::CX + 2, off);
+            for (unsigned crowded = __ballot_sync(0xffffffffu, cnt > kPkCrowd); crowded; crowded &= crowded - 1u) {
+                const int bx = __ffs(crowded) - 1;
+                const unsigned n = __shfl_sync(0xffffffffu, cnt, bx);
+                const int64_t at = __shfl_sync(0xffffffffu, off, bx);
+                using Bins = typename PackedBins<PB>::type;
+                constexpr int kAhead = PB == 1 ? 4 : 2;
+#pragma unroll 1
+                for (unsigned v0 = tid; v0 < n; v0 += kAhead * T) {
+                    Bins p[kAhead];
 #pragma unroll
-            for (int c = 0; c < 8; ++c) {
-                const int dx = c & 1, dy = (c >> 1) & 1, dz = c >> 2;
-                const int x = ix + dx, y = iy + dy, z = iz + dz;
-                const uint32_t w = cic_weight3<PB>(dx ? wx : W - wx, dy ? wy : W - wy, dz ? wz : W - wz);
-                if ((unsigned)x < (unsigned)B::NX && (unsigned)y < (unsigned)B::NY && (unsigned)z < (unsigned)B::NZ) {
-                    const int i = x + B::NX * (y + B::NY * z);
-                    if (safe) {
-                        smem_red(&lo[i], w);
-                    } else {
-                        const uint32_t old = atomicAdd(&lo[i], w);
-                        if (old + w < old) atomicAdd(&hi[i], 1u);
+                    for (int u = 0; u < kAhead; ++u) {
+                        const int64_t j = at + min(v0 + u * T, n - 1);
+                        p[u] = 0;
+#pragma unroll
+                        for (int e = 0; e < 3; ++e) p[u] |= (Bins)load_bin<PB>(st.m[e], j) << (8 * PB * e);
+                    }
+#pragma unroll 1
+                    for (int u = 0; u < kAhead && v0 + u * T < n; ++u) {
+                        const int m[3] = {(int)(p[0] & (F::kBins - 1)), (int)(p[0] >> 8 * PB & (F::kBins - 1)),
+                                          (int)(p[0] >> 16 * PB)};
+                        cloud(bx, row % (B::CY + 2), row / (B::CY + 2), m);
+#pragma unroll
+                        for (int k = 1; k < kAhead; ++k) p[k - 1] = p[k];
                     }
                 }
             }
