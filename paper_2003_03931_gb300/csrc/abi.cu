@@ -389,6 +389,41 @@ static int enqueue_step(Sim& s) {
     return check_launch(s, "step");
 }
 
+// The captured step of buffer parity s.cur, captured first where it is not yet.
+static int replay_step(Sim& s) {
+    const int c = s.cur;
+    if (!s.graph_ready[c]) {
+        const bool prof = s.prof;
+        const int64_t l0 = s.launches;
+        s.prof = false;
+        cudaGraph_t g = nullptr;
+        cudaError_t e = cudaStreamBeginCapture(s.stream, cudaStreamCaptureModeThreadLocal);
+        if (e != cudaSuccess) {
+            s.prof = prof;
+            return set_error(s, PMPM_ECUDA, "capture: %s", cudaGetErrorString(e));
+        }
+        const int rc = enqueue_step(s);
+        e = cudaStreamEndCapture(s.stream, &g);
+        s.prof = prof;
+        s.cur = c;   // capturing ran nothing
+        s.graph_launches[c] = s.launches - l0;
+        s.launches = l0;
+        if (rc || e != cudaSuccess) {
+            if (g) cudaGraphDestroy(g);
+            return rc ? rc : set_error(s, PMPM_ECUDA, "capture: %s", cudaGetErrorString(e));
+        }
+        e = cudaGraphInstantiate(&s.graph_exec[c], g, 0);
+        cudaGraphDestroy(g);
+        if (e != cudaSuccess) return set_error(s, PMPM_ECUDA, "instantiate: %s", cudaGetErrorString(e));
+        s.graph_ready[c] = true;
+    }
+    const cudaError_t e = cudaGraphLaunch(s.graph_exec[c], s.stream);
+    if (e != cudaSuccess) return set_error(s, PMPM_ECUDA, "graph launch: %s", cudaGetErrorString(e));
+    s.launches += s.graph_launches[c];
+    s.cur = 1 - c;
+    return PMPM_OK;
+}
+
 static int one_step(Sim& s) {
     if (s.step >= s.cfg.n_steps) return set_error(s, PMPM_EINVAL, "schedule exhausted");
     int rc;
@@ -396,39 +431,17 @@ static int one_step(Sim& s) {
         if ((rc = scan_counts(s, s.counts[s.cur], s.offsets[s.cur]))) return rc;
         s.offsets_valid = true;
     }
+    const int c = s.cur;
     s.in_step = true;
-    if (s.graphs) {
-        const int c = s.cur;
-        if (!s.graph_ready[c]) {
-            const bool prof = s.prof;
-            const int64_t l0 = s.launches;
-            s.prof = false;
-            cudaGraph_t g = nullptr;
-            cudaError_t e = cudaStreamBeginCapture(s.stream, cudaStreamCaptureModeThreadLocal);
-            if (e != cudaSuccess) return set_error(s, PMPM_ECUDA, "capture: %s", cudaGetErrorString(e));
-            rc = enqueue_step(s);
-            e = cudaStreamEndCapture(s.stream, &g);
-            s.prof = prof;
-            s.cur = c;   // capturing ran nothing
-            s.graph_launches[c] = s.launches - l0;
-            s.launches = l0;
-            if (rc || e != cudaSuccess) {
-                if (g) cudaGraphDestroy(g);
-                return rc ? rc : set_error(s, PMPM_ECUDA, "capture: %s", cudaGetErrorString(e));
-            }
-            e = cudaGraphInstantiate(&s.graph_exec[c], g, 0);
-            cudaGraphDestroy(g);
-            if (e != cudaSuccess) return set_error(s, PMPM_ECUDA, "instantiate: %s", cudaGetErrorString(e));
-            s.graph_ready[c] = true;
-        }
-        const cudaError_t e = cudaGraphLaunch(s.graph_exec[c], s.stream);
-        if (e != cudaSuccess) return set_error(s, PMPM_ECUDA, "graph launch: %s", cudaGetErrorString(e));
-        s.launches += s.graph_launches[c];
-        s.cur = 1 - c;
-    } else {
-        if ((rc = enqueue_step(s))) return rc;
-    }
+    rc = s.graphs ? replay_step(s) : enqueue_step(s);
     s.in_step = false;
+    if (rc) {
+        // A step writes the other store only: this one stands, and so does the step to
+        // take from it (k_step_begin has moved the device's counter on).
+        s.cur = c;
+        set_device_step(s, s.step);
+        return rc;
+    }
     s.step += 1;
     s.a = sched_a(s, s.step);
     return PMPM_OK;
