@@ -381,7 +381,7 @@ static int enqueue_step(Sim& s) {
     s.launches++;
     if ((rc = coarse_deposit(s, true))) return rc;
     prof_mark(s, 0);
-    if ((rc = coarse_force(s, true))) return rc;
+    if ((rc = coarse_force(s))) return rc;
     prof_mark(s, 1);
     if ((rc = tile_pass(s, 1, nullptr))) return rc;
     prof_mark(s, 2);
@@ -739,7 +739,7 @@ int pmpm_fetch(pmpm_sim* h, int32_t what, void* dst, size_t bytes) {
             break;
         case PMPM_FORCE:
             if ((rc = coarse_deposit(s))) return rc;
-            if ((rc = coarse_force(s, false))) return rc;
+            if ((rc = coarse_force(s))) return rc;
             if ((rc = tile_pass(s, 0, s.Pn))) return rc;
             rc = copy_out(s, dst, s.Pn, need);
             break;

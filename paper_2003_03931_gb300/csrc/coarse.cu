@@ -308,7 +308,7 @@ __global__ void __launch_bounds__(kC32) k_coarse32_back(const float2* B1, const 
 }
 
 // ------------------------------------------------------------ sparse boxes, 64^3 cells and more
-// Density to delta, Green multiply and F_l around fft.cu's transforms, for steps that
+// Density to delta, Green multiply and F_l around fft.cu's transforms, for boxes that
 // keep their bits (keeps_bits): twelve launches, every pass through memory, 73 us at 64^3
 // cells where the fused passes below take 41.
 __global__ void __launch_bounds__(256) k_coarse_delta(int64_t ncells, long long mean, const long long* rho, float2* out) {
@@ -610,10 +610,10 @@ void coarse_setup() {
     pass_setup<32, 32>();
 }
 
-int coarse_force(Sim& s, bool step) {
+int coarse_force(Sim& s) {
     // N 2^27 / nc^3, all powers of two (N up to 2^36)
     const long long mean = s.n >= s.ncells ? (s.n / s.ncells) << 27 : (1ll << 27) / (s.ncells / s.n);
-    if (step && keeps_bits(s) && s.nc > 32) return launch_kept(s, mean);
+    if (s.nc > 32 && keeps_bits(s)) return launch_kept(s, mean);
     switch (s.nc) {
         case 8: launch_tiny<8>(s, mean); break;
         case 16: launch_tiny<16>(s, mean); break;

@@ -1,8 +1,8 @@
 // fft.cu -- batched 1-D FFTs along the three axes of an n^3 complex array
 // (n a power of two), float or double.  Used for the force tables, the low-memory
 // step's displacement field, power spectra past 1024 points a side and the coarse
-// force of sparse boxes' steps; the coarse force otherwise, the other initial
-// conditions and spectra have passes of their own.
+// force of sparse boxes; the coarse force otherwise, the other initial conditions
+// and spectra have passes of their own.
 //
 // One block transforms P neighbouring pencils.  Float pencils of 64 to 1024
 // points take two register steps with one shared-memory transpose

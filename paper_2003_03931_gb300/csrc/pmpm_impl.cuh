@@ -100,16 +100,15 @@ struct Sim {
 
 inline uintptr_t align_up(uintptr_t p, uintptr_t a = 256) { return (p + a - 1) & ~(a - 1); }
 
-// Whether a step's force comes from the 32^3-box tiles and from coarse transforms in
-// fft.cu's order, bit for bit, and not from columns of tiles and the fused passes.
+// Whether the force comes from the 32^3-box tiles and from coarse transforms in fft.cu's
+// order, bit for bit, and not from columns of tiles and the fused passes.
 // A step turns a last bit of a momentum into a velocity bin now and then (in a cell of
 // one particle, whose velocity is its cell's mean, always: the sign of the rounding), and
 // later steps amplify that.  With columns in place of tiles the P(k) of 64^3 particles on
 // 32^3 cells moved by up to 3e-5 after 5 to 10 steps to a = 1 (600 boxes) and by 4e-4
 // after 10 to 40, and sigma of boxes with a particle a cell or fewer by up to 1e-4
 // after 1 to 4.  Denser boxes of 64^3 cells and more average it out: 128^3 particles 2e-6
-// (250 boxes) and 2.5e-5 (80), 256^3 2e-7.  A force on its own (PMPM_FORCE) differs by 1e-7
-// and takes the faster kernels at every size.
+// (250 boxes) and 2.5e-5 (80), 256^3 2e-7.
 inline bool keeps_bits(const Sim& s) { return s.nc <= 32 || s.n <= s.ncells; }
 
 inline int grid_for(int64_t n, int block, int cap = 152 * 64) {
@@ -166,8 +165,7 @@ size_t green_scratch_bytes(int nc);
 template <typename R>
 int fft3d(Sim& s, void* data, int n, int sign);
 int fft_pass_count(int n);
-// FFT + Green of s.rho_c -> s.Fl; step: for a step (keeps_bits)
-int coarse_force(Sim& s, bool step);
+int coarse_force(Sim& s);             // FFT + Green of s.rho_c -> s.Fl
 int coarse_deposit(Sim& s, bool cleared = false);   // -> s.rho_c
 int tile_pass(Sim& s, int mode, float* G);
 int tile_density(Sim& s, int tile, uint32_t* d_out);   // one tile's fine box after the deposit

@@ -184,17 +184,6 @@ static TileParams base_params(Sim& s) {
     return P;
 }
 
-// Columns of tiles (column.cu) or 32^3-box tiles.  Boxes of up to kTileCells cells a side
-// are one wave of tiles, where the depth of walking columns does not pay: 16^3 cells are
-// 64 CTAs and 36 us on a GB300 against 42 to 50 (by how the particles cluster).  Steps that
-// keep their bits (keeps_bits) take tiles too, where columns would be faster: 64^3 particles
-// on 32^3 cells 106 us against 84.  All else takes columns: 128^3 particles on 64^3 cells 607
-// us with tiles, 404 with columns.
-static bool by_columns(const Sim& s, int mode) {
-    constexpr int kTileCells = 16;
-    return !s.fp16 && s.nc > kTileCells && (mode == 0 || !keeps_bits(s));
-}
-
 int tile_pass(Sim& s, int mode, float* G) {
     TileParams P = base_params(s);
     P.mode = mode;
@@ -208,7 +197,11 @@ int tile_pass(Sim& s, int mode, float* G) {
     // derived again by its re-encode
     if (s.lowmem) P.Qn = nullptr;
     const int grid = s.nt * s.nt * s.nt;
-    if (by_columns(s, mode)) column_pass(s.stream, P, s.green_col, s.lowmem, s.pb, s.chained, s.sharers);
+    // Columns of tiles (column.cu), but for boxes that keep their bits (keeps_bits) and FP16
+    // storage.  128^3 particles on 64^3 cells take 404 us on a GB300 by columns, 607 by tiles;
+    // 64^3 on 32^3, which keep tiles, 84 against 106.  Up to 16^3 cells columns would not pay:
+    // tiles are one wave there, 36 us against 42 to 50 (by how the particles cluster).
+    if (!s.fp16 && !keeps_bits(s)) column_pass(s.stream, P, s.green_col, s.lowmem, s.pb, s.chained, s.sharers);
     else if (s.lowmem) chain(s.chained, k_tile<1, float2, true>, grid, kTileThreads, kTileSmemBytes, s.stream, P);
     else if (s.fp16 && s.pb == 2) chain(s.chained, k_tile<2, __half2>, grid, kTileThreads, kTileSmemBytes, s.stream, P);
     else if (s.fp16) chain(s.chained, k_tile<1, __half2>, grid, kTileThreads, kTileSmemBytes, s.stream, P);
