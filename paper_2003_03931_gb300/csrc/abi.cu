@@ -90,7 +90,6 @@ static void derive(Sim& s, const pmpm_config* c) {
     s.fft_max = s.nc;
     if (s.np > s.fft_max) s.fft_max = s.np;
     if (s.pk_max > s.fft_max) s.fft_max = s.pk_max;
-    s.nblocks_scan = s.ncells / (256 * scan_items(s.ncells));
     s.lowmem = (c->flags & PMPM_FLAG_LOWMEM) != 0;
     s.fp16 = (c->flags & PMPM_FLAG_FINE_FP16) != 0;
     s.pb = c->pos_bytes == 2 ? 2 : 1;
@@ -135,8 +134,8 @@ static size_t layout_lowmem(Sim& s, uint8_t* base) {
     s.tw_f = reinterpret_cast<float2*>(take(8 * (size_t)s.fft_max));
     s.tw_d = reinterpret_cast<double2*>(take(16 * (size_t)s.fft_max));
     s.err = reinterpret_cast<uint32_t*>(take(4));
-    s.blocksums = reinterpret_cast<long long*>(take(8 * (size_t)(s.nblocks_scan + 1)));
     s.ic_partial = reinterpret_cast<double*>(take(8 * (3 * 1024 + 1)));
+    s.scan_sums = reinterpret_cast<long long*>(s.ic_partial);
     s.pk_bins = reinterpret_cast<double*>(take(8 * 3 * (size_t)(s.pk_max / 2 + 1)));
     s.d_factors = reinterpret_cast<float*>(take(8 * (size_t)s.cfg.n_steps));
     s.d_step = reinterpret_cast<int*>(take(4));
@@ -218,8 +217,8 @@ size_t layout(Sim& s, uint8_t* base) {
     s.tw_f = reinterpret_cast<float2*>(take(8 * (size_t)s.fft_max));
     s.tw_d = reinterpret_cast<double2*>(take(16 * (size_t)s.fft_max));
     s.err = reinterpret_cast<uint32_t*>(take(4));
-    s.blocksums = reinterpret_cast<long long*>(take(8 * (size_t)(s.nblocks_scan + 1)));
     s.ic_partial = reinterpret_cast<double*>(take(8 * (3 * 1024 + 1)));
+    s.scan_sums = reinterpret_cast<long long*>(s.ic_partial);
     s.pk_bins = reinterpret_cast<double*>(take(8 * 3 * (size_t)(s.pk_max / 2 + 1)));
     s.d_factors = reinterpret_cast<float*>(take(8 * (size_t)s.cfg.n_steps));
     s.d_step = reinterpret_cast<int*>(take(4));

@@ -57,9 +57,8 @@ struct Sim {
     float2* tw_f = nullptr;                     // [fft_max] exp(-2 pi i k / fft_max)
     double2* tw_d = nullptr;
     uint32_t* err = nullptr;
-    long long* blocksums = nullptr;
-    int64_t nblocks_scan = 0;
     double* ic_partial = nullptr;               // [3*1024 + 1] IC rms partial sums
+    long long* scan_sums = nullptr;             // [kScanSums], in the first of them
     float* d_factors = nullptr;                 // [2 n_steps] kick, drift (codes) per step
     int* d_step = nullptr;                      // index of the next step (k_step_begin)
     float* d_kd = nullptr;                      // [2] kick and drift factors of the step under way
@@ -172,7 +171,8 @@ int tile_density(Sim& s, int tile, uint32_t* d_out);   // one tile's fine box af
 void tile_setup();
 void fft_setup();
 void coarse_setup();
-// cells a thread of the scan takes (sort.cu)
+// block sums that a scan keeps beside its arrays, and cells a thread of it takes (sort.cu)
+constexpr int kScanSums = 1024;
 inline int scan_items(int64_t ncells) { return ncells <= (1 << 18) ? 1 : (ncells <= (1 << 24) ? 4 : 8); }
 int scan_counts(Sim& s, const int32_t* counts, int64_t* offsets);
 int encode_from_qp(Sim& s, bool counts_ready);

@@ -24,8 +24,8 @@ cudaError_t pk_enqueue(cudaStream_t stream, const PkStore& st, int nmesh, int nb
                        double* bins, const uint32_t* err, const float2* tw, int tw_n, int64_t* launches);
 void pk_setup();
 
-// offsets[0..nc^3] of `counts` (sort.cu); blocksums: nc^3 / 256 words
-void scan_raw(cudaStream_t stream, bool chained, int64_t ncells, const int32_t* counts, long long* blocksums, int64_t* offsets,
+// offsets[0..nc^3] of `counts` (sort.cu); sums: kScanSums words
+void scan_raw(cudaStream_t stream, bool chained, int64_t ncells, const int32_t* counts, long long* sums, int64_t* offsets,
               int64_t n, uint32_t* err, int64_t* launches);
 // in place, forward or back, for sizes without a fused pass (fft.cu)
 cudaError_t fft3d_float_raw(cudaStream_t st, float2* data, int n, int sign, const float2* tw, int tw_n);

@@ -53,8 +53,9 @@ __device__ __forceinline__ long long block_exclusive_scan(long long v, long long
     return before + x - v;
 }
 
+// the particles of block b's cells, to sums[b stride]
 __global__ void __launch_bounds__(kScanThreads) k_scan_reduce(int64_t ncells, const int32_t* counts,
-                                                              long long* blocksums, int items) {
+                                                              long long* sums, int64_t stride, int items) {
     chain_begin();
     __shared__ long long sh[32];
     const int64_t b0 = (int64_t)blockIdx.x * kScanThreads * items;
@@ -62,19 +63,20 @@ __global__ void __launch_bounds__(kScanThreads) k_scan_reduce(int64_t ncells, co
     for (int k = 0; k < items; ++k) acc += counts[b0 + (int64_t)k * kScanThreads + threadIdx.x];
     long long total;
     block_exclusive_scan(acc, sh, total);
-    if (threadIdx.x == 0) blocksums[blockIdx.x] = total;
+    if (threadIdx.x == 0) sums[blockIdx.x * stride] = total;
 }
 
-__global__ void __launch_bounds__(1024) k_scan_top(int64_t nb, long long* blocksums) {
+// those sums in place to what lies before each block
+__global__ void __launch_bounds__(1024) k_scan_top(int64_t nb, long long* sums, int64_t stride) {
     chain_begin();
     __shared__ long long sh[32];
     long long carry = 0;
     for (int64_t base = 0; base < nb; base += blockDim.x) {
         const int64_t i = base + threadIdx.x;
-        const long long v = i < nb ? blocksums[i] : 0;
+        const long long v = i < nb ? sums[i * stride] : 0;
         long long total;
         const long long ex = block_exclusive_scan(v, sh, total);
-        if (i < nb) blocksums[i] = carry + ex;
+        if (i < nb) sums[i * stride] = carry + ex;
         carry += total;
     }
 }
@@ -121,9 +123,10 @@ __device__ float sigma_of(const unsigned long long* d2, int64_t n) {
 }
 
 // Where a block takes the particles before it from: it adds up the counts
-// itself (up to 32^3 cells), or up to kScanFew blocks' sums, or finds the prefix
-// that k_scan_top made of them.
-constexpr int kScanFew = 1024;
+// itself (up to 32^3 cells), or up to kScanFew blocks' sums (kScanSums of pmpm_impl.cuh), or
+// finds the prefix that k_scan_top made of them: it waits in the offsets, at the
+// block's first cell, where the block writes it again.
+constexpr int kScanFew = kScanSums;
 constexpr int64_t kScanDirect = 32768;
 
 // One tile of kScanThreads ITEMS cells per block (the cells, at least 512 and a
@@ -140,7 +143,7 @@ constexpr int64_t kScanDirect = 32768;
 // cell: 119 us at the copy bandwidth; the divisions bound it).
 template <bool MEANS, int ITEMS>
 __global__ void __launch_bounds__(kScanThreads) k_scan_apply(int64_t ncells, const int32_t* counts,
-                                                             const long long* blocksums,
+                                                             const long long* sums,
                                                              int64_t* offsets, int64_t n,
                                                              uint32_t* err,
                                                              const unsigned long long* S,
@@ -198,10 +201,10 @@ __global__ void __launch_bounds__(kScanThreads) k_scan_apply(int64_t ncells, con
         }
         block_exclusive_scan(part, sh, base);
     } else if (gridDim.x > kScanFew) {
-        base = blocksums[blockIdx.x];
+        base = offsets[b0];
     } else {
         long long part = 0;
-        for (int b = t; b < (int)blockIdx.x; b += kScanThreads) part += blocksums[b];
+        for (int b = t; b < (int)blockIdx.x; b += kScanThreads) part += sums[b];
         block_exclusive_scan(part, sh, base);
     }
     __syncthreads();
@@ -544,31 +547,34 @@ __global__ void k_decode(int64_t n, int nc, const int64_t* __restrict__ offsets,
 
 // Offsets of `counts`; MEANS: with the rest of k_scan_apply.
 template <bool MEANS>
-static void scan(cudaStream_t st, bool chained, int64_t ncells, const int32_t* counts, long long* blocksums, int64_t* offsets,
+static void scan(cudaStream_t st, bool chained, int64_t ncells, const int32_t* counts, long long* sums, int64_t* offsets,
                  int64_t n, uint32_t* err, const unsigned long long* S, float* vc, int32_t* fill,
                  unsigned long long* d2, float* sigma, int64_t* launches) {
     const int items = scan_items(ncells);
     const unsigned nb = (unsigned)(ncells / (kScanThreads * items));
     if (ncells > kScanDirect) {
-        chain(chained, k_scan_reduce, nb, kScanThreads, 0, st, ncells, counts, blocksums, items);
+        const bool many = nb > kScanFew;
+        long long* const to = many ? reinterpret_cast<long long*>(offsets) : sums;
+        const int64_t stride = many ? kScanThreads * items : 1;
+        chain(chained, k_scan_reduce, nb, kScanThreads, 0, st, ncells, counts, to, stride, items);
         *launches += 1;
-        if (nb > kScanFew) {
-            chain(chained, k_scan_top, 1, 1024, 0, st, nb, blocksums);
+        if (many) {
+            chain(chained, k_scan_top, 1, 1024, 0, st, nb, to, stride);
             *launches += 1;
         }
     }
     auto k = items == 1 ? k_scan_apply<MEANS, 1> : (items == 4 ? k_scan_apply<MEANS, 4> : k_scan_apply<MEANS, 8>);
-    chain(chained, k, nb, kScanThreads, 0, st, ncells, counts, blocksums, offsets, n, err, S, vc, fill, d2, sigma);
+    chain(chained, k, nb, kScanThreads, 0, st, ncells, counts, sums, offsets, n, err, S, vc, fill, d2, sigma);
     *launches += 1;
 }
 
-void scan_raw(cudaStream_t st, bool chained, int64_t ncells, const int32_t* counts, long long* blocksums, int64_t* offsets,
+void scan_raw(cudaStream_t st, bool chained, int64_t ncells, const int32_t* counts, long long* sums, int64_t* offsets,
               int64_t n, uint32_t* err, int64_t* launches) {
-    scan<false>(st, chained, ncells, counts, blocksums, offsets, n, err, nullptr, nullptr, nullptr, nullptr, nullptr, launches);
+    scan<false>(st, chained, ncells, counts, sums, offsets, n, err, nullptr, nullptr, nullptr, nullptr, nullptr, launches);
 }
 
 int scan_counts(Sim& s, const int32_t* counts, int64_t* offsets) {
-    scan_raw(s.stream, s.chained, s.ncells, counts, s.blocksums, offsets, s.n, s.err, &s.launches);
+    scan_raw(s.stream, s.chained, s.ncells, counts, s.scan_sums, offsets, s.n, s.err, &s.launches);
     return check_launch(s, "scan");
 }
 
@@ -622,7 +628,7 @@ void check_loaded_counts(Sim& s) {
 // Offsets of the new counts, zeroed slot counters, the new cell means
 // v_c = fl32(fl32(S 2^-24) / count) of buffer nxt and its sigma (Eq. 3).
 int scan_and_means(Sim& s, int nxt) {
-    scan<true>(s.stream, s.chained, s.ncells, s.counts[nxt], s.blocksums, s.offsets[nxt], s.n, s.err, s.S, s.vc[nxt], s.fill, s.d2,
+    scan<true>(s.stream, s.chained, s.ncells, s.counts[nxt], s.scan_sums, s.offsets[nxt], s.n, s.err, s.S, s.vc[nxt], s.fill, s.d2,
                s.sigma_d[nxt], &s.launches);
     return check_launch(s, "scan");
 }
