@@ -103,12 +103,14 @@ inline uintptr_t align_up(uintptr_t p, uintptr_t a = 256) { return (p + a - 1) &
 // order, bit for bit, and not from columns of tiles and the fused passes.
 // A step turns a last bit of a momentum into a velocity bin now and then (in a cell of
 // one particle, whose velocity is its cell's mean, always: the sign of the rounding), and
-// later steps amplify that.  With columns in place of tiles the P(k) of 64^3 particles on
-// 32^3 cells moved by up to 3e-5 after 5 to 10 steps to a = 1 (600 boxes) and by 4e-4
-// after 10 to 40, and sigma of boxes with a particle a cell or fewer by up to 1e-4
-// after 1 to 4.  Denser boxes of 64^3 cells and more average it out: 128^3 particles 2e-6
-// (250 boxes) and 2.5e-5 (80), 256^3 2e-7.
-inline bool keeps_bits(const Sim& s) { return s.nc <= 32 || s.n <= s.ncells; }
+// later steps amplify that; many particles average it out.  With columns in place of
+// tiles, largest changes against the code before them: of 64^3 particles on 32^3 cells P(k)
+// 3e-5 after 5 to 10 steps to a = 1 (600 boxes), 4e-4 after 10 to 40; sigma of boxes of up to
+// 128^3 particles, a particle a cell or fewer, 1e-4 after 1 to 4 steps.  Those keep their
+// bits.  The others: 128^3 on 64^3 cells P(k) 2e-6 (250 boxes) and 2.5e-5 (80), 256^3 on 128^3
+// 2e-7; 256^3 on 256^3 cells, 1 to 4 steps, P(k) 2e-6 and sigma 7e-6.
+constexpr int64_t kKeptSparse = 128 * 128 * 128;
+inline bool keeps_bits(const Sim& s) { return s.nc <= 32 || (s.n <= s.ncells && s.n <= kKeptSparse); }
 
 inline int grid_for(int64_t n, int block, int cap = 152 * 64) {
     int64_t g = (n + block - 1) / block;
