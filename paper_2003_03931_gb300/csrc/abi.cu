@@ -722,14 +722,15 @@ int pmpm_fetch(pmpm_sim* h, int32_t what, void* dst, size_t bytes) {
             float sig = 0.f;
             cudaError_t e = cudaMemcpyAsync(&sig, s.sigma_d[s.cur], 4, cudaMemcpyDeviceToHost, s.stream);
             if (e != cudaSuccess) return set_error(s, PMPM_ECUDA, "fetch: %s", cudaGetErrorString(e));
-            if ((rc = sync_and_check(s))) return rc;
+            // (flags of earlier steps are reported here too, and the scalars stand)
+            if ((rc = sync_and_check(s)) == PMPM_ECUDA) return rc;
             pmpm_scalars sc;
             sc.a = s.a;
             sc.sigma = sig;
             sc.step = s.step;
             sc.n = s.n;
             memcpy(dst, &sc, sizeof(sc));
-            return PMPM_OK;
+            return rc;
         }
         case PMPM_DECODED_Q:
         case PMPM_DECODED_P:
