@@ -263,19 +263,10 @@ void fft_setup() {
     cudaFuncSetAttribute(k_fft_pass_r<16, 32, 1>, cudaFuncAttributeMaxDynamicSharedMemorySize, kPassSmem);
 }
 
-// The same three float passes for a caller-supplied twiddle table of tw_n
-// entries (n divides tw_n); used where no Sim exists.
+// The radix-2 float passes on a caller's twiddle table of tw_n entries (n divides it),
+// for meshes past 1024 points a side; used where no Sim exists.
 cudaError_t fft3d_float_raw(cudaStream_t st, float2* data, int n, int sign, const float2* tw,
                             int tw_n) {
-    if (n >= 64 && n <= 1024 && n <= tw_n) {   // the same passes as fft3d<float>
-        if (n > 512) fft_setup();                // more than 48 KB of shared memory
-        if (n == 64) launch_pass_r<8, 8>(data, n, sign, tw, tw_n, st);
-        else if (n == 128) launch_pass_r<8, 16>(data, n, sign, tw, tw_n, st);
-        else if (n == 256) launch_pass_r<16, 16>(data, n, sign, tw, tw_n, st);
-        else if (n == 512) launch_pass_r<16, 32>(data, n, sign, tw, tw_n, st);
-        else launch_pass_r<32, 32>(data, n, sign, tw, tw_n, st);
-        return cudaGetLastError();
-    }
     int log2n = 0;
     while ((1 << log2n) < n) ++log2n;
     const int P = pencils_per_block<float>(n);

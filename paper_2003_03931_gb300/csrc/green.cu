@@ -14,8 +14,8 @@
 //  * Matching A(d): coarse-mesh force between fine-cell centres a fine
 //    separation d apart, averaged over the 64 centres of a coarse cell.
 //  * Short-range kernel K_s(d) = K_per(d) - A(d) for 0 < |d| < 6, and its
-//    32^3 DFT stored the same way (for the FP16 tiles), and its 32^2 DFT over x
-//    and y for every dz (for the column pass).
+//    32^3 DFT stored the same way (for the 32^3-box tiles), and its 32^2 DFT over
+//    x and y for every dz (for the column pass).
 #include "pmpm_impl.cuh"
 
 namespace pmpm {

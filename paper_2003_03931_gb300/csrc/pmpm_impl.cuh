@@ -51,7 +51,7 @@ struct Sim {
     float* Fl = nullptr;                        // [3][nc^3]
     float4* green_coarse = nullptr;             // [(nc/2+1)^3] (S_x, S_y, S_z, 0), |kx| fastest
     float* green_col = nullptr;                 // [17][17][17] column pass: taps x |kx| x |ky|
-    float* green_packed = nullptr;              // [15 x 153] 32^3 DFT (FP16 tiles)
+    float* green_packed = nullptr;              // [15 x 153] 32^3 DFT (32^3-box tiles)
     float* Tdec = nullptr;                      // [256]
     float* Eedge = nullptr;                     // [256]
     float2* tw_f = nullptr;                     // [fft_max] exp(-2 pi i k / fft_max)
@@ -165,7 +165,6 @@ int build_green_tables(Sim& s);
 size_t green_scratch_bytes(int nc);
 template <typename R>
 int fft3d(Sim& s, void* data, int n, int sign);
-int fft_pass_count(int n);
 int coarse_force(Sim& s);             // FFT + Green of s.rho_c -> s.Fl
 int coarse_deposit(Sim& s, bool cleared = false);   // -> s.rho_c
 int tile_pass(Sim& s, int mode, float* G);
@@ -210,7 +209,7 @@ namespace pmpm {
 
 // Device pointers of the three force tables (Sec. II): the coarse-kernel
 // spectrum, the fine kernel K_s transformed along x and y (column pass) and its
-// packed 32^3 spectrum (FP16 tiles).
+// packed 32^3 spectrum (32^3-box tiles).
 struct GreenRefs {
     const float4* coarse;
     const float* fine;
