@@ -346,8 +346,8 @@ __global__ void __launch_bounds__(256) k_coarse_extract(int64_t ncells, const fl
 // k = k1 + N1 k2 the forward pass ends with all k2 of one k1 in a thread's
 // registers, which is where the inverse one begins: the z pass transforms,
 // multiplies and transforms back without another exchange.  116 bytes a cell
-// over five launches against 212 over twelve: 64^3 cells 73 -> 38 us, 128^3
-// 126 -> 72, 256^3 (HBM-bound) 710 -> 399.
+// over five launches against 212 over twelve: 64^3 cells 76 -> 41 us, 128^3
+// 126 -> 75, 256^3 (HBM-bound) 709 -> 412.
 // x: integer density rows -> delta -> spectrum
 template <int N1, int N2>
 __global__ void __launch_bounds__(kPassWidth) k_coarse_fwd_x(long long mean, const long long* rho,

@@ -26,9 +26,11 @@
 //
 // What bounds it: issue (49% of the slots, 16.5k warp instructions a layer, 6.3k of
 // them floating point) and the waits between the three barriers of a layer and
-// for the particles' bytes; memory moves 41 B a particle.  Short-range pass of a step on a GB300 against
-// the 32^3-box tiles of one CTA a SM before: 512^3 particles 36.5 -> 19.1 ms,
-// 256^3 4.57 -> 2.54 ms, 128^3 607 -> 404 us, 64^3 125 -> 84 us.
+// for the particles' bytes; memory moves 41 B a particle.  Short-range pass of a step on
+// a GB300 against the 32^3-box tiles of one CTA a SM: 512^3 particles 35.5 -> 18.8 ms,
+// 256^3 4.52 -> 2.52 ms, 128^3 598 -> 398 us; denser boxes, 256^3 on 64^3 cells 2.40 -> 1.87
+// ms and 512^3 on 64^3, where every node is checked, 21.8 -> 15.0.  (keeps_bits: boxes that
+// take tiles all the same.)
 #include <algorithm>
 
 #include "pmpm_impl.cuh"
@@ -117,7 +119,6 @@ __device__ __forceinline__ void tmem_alloc(uint32_t* dst) {
 __device__ __forceinline__ void tmem_free(uint32_t addr) {
     asm volatile("tcgen05.dealloc.cta_group::1.sync.aligned.b32 %0, %1;" ::"r"(addr), "r"(kTmemCols));
 }
-// waits for this thread's loads; their registers are read only after it
 // waits for this thread's loads; their registers are read only after it
 template <int N>
 __device__ __forceinline__ void tmem_wait_ld(float (&r)[N]) {
@@ -880,14 +881,16 @@ void column_setup() {
 // Layers of a segment.  A CTA walks lz layers and 5.5 more to fill its 11
 // planes; a layer takes 16k cycles with two CTAs on the SM and 12k alone
 // (measured), so the last 152 CTAs or fewer run at 0.74 of the time.  The
-// shortest walk: 64^3 particles on 32^3 cells lz = 6 (98 us against 111 at 11
-// and 120 at 3), 128^3 on 64^3 22 (431 us; 509 at 6, 540 at 64), 256^3 on 128^3 64
-// (2.58 ms; 2.83 at 16, 2.93 at 128).
+// shortest walk: 128^3 particles on 64^3 cells lz = 22 (404 us; 469 at 6, 407 at 11, 567 at
+// 64), 256^3 on 128^3 64 (2.52 ms; 2.78 at 16, 2.58 at 43, 2.84 at 128), 512^3 on 256^3 256
+// (18.8 ms; 19.7 at 43, 19.3 at 64).
 //
 // Where other boxes fill the SMs (sharers of them in all), the last CTAs of a pass cost
 // nothing and what counts is the sum of all walks: longer ones, but none that would take
 // 1.3 times as long alone.  Sixteen boxes of 32^3 to 128^3 particles 23.7 -> 22.5 ms; 400
-// requests as they come at 1.5 times the capacity, p99 1.98 -> 1.85 s.
+// requests as they come at 1.5 times the capacity, p99 1.98 -> 1.85 s.  A captured step
+// keeps the segments of the time of its capture (engines with graphs on); results do
+// not depend on them.
 static int column_layers(int nc, int nt, int sharers) {
     const auto ctas = [=](int lz) { return (int64_t)nt * nt * ((nc + lz - 1) / lz); };
     const auto alone = [=](int lz) {

@@ -198,8 +198,8 @@ int tile_pass(Sim& s, int mode, float* G) {
     if (s.lowmem) P.Qn = nullptr;
     const int grid = s.nt * s.nt * s.nt;
     // Columns of tiles (column.cu), but for boxes that keep their bits (keeps_bits) and FP16
-    // storage.  128^3 particles on 64^3 cells take 404 us on a GB300 by columns, 607 by tiles;
-    // 64^3 on 32^3, which keep tiles, 84 against 106.  Up to 16^3 cells columns would not pay:
+    // storage.  128^3 particles on 64^3 cells take 398 us on a GB300 by columns, 598 by tiles;
+    // 64^3 on 32^3, which keep tiles, 84 against 108.  Up to 16^3 cells columns would not pay:
     // tiles are one wave there, 36 us against 42 to 50 (by how the particles cluster).
     if (!s.fp16 && !keeps_bits(s)) column_pass(s.stream, P, s.green_col, s.lowmem, s.pb, s.chained, s.sharers);
     else if (s.lowmem) chain(s.chained, k_tile<1, float2, true>, grid, kTileThreads, kTileSmemBytes, s.stream, P);
