@@ -110,7 +110,7 @@ extern "C" int pmpm_power_spectrum_noalloc(int32_t nc, int64_t n, const uint8_t*
     const bool chained = ncells <= kChainCells;
     scan_raw(st, chained, ncells, d_counts, reinterpret_cast<long long*>(base + kNaOffSums), offsets, n, err, &launches);
     const PkStore store = {nc, 1, n, offsets, d_counts, {d_m0, d_m1, d_m2}, chained};
-    cudaError_t e = pk_enqueue(st, store, nmesh, nbins, reinterpret_cast<float2*>(base + kNaOffMesh), bins, err,
+    cudaError_t e = pk_enqueue(st, store, nmesh, nbins, reinterpret_cast<float2*>(base + kNaOffMesh), nullptr, bins, err,
                                reinterpret_cast<const float2*>(base + kNaOffTw), kNaMaxMesh, &launches);
     double hb[3 * kNaMaxBins + 1];
     if (e == cudaSuccess)

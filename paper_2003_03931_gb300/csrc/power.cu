@@ -325,14 +325,15 @@ __device__ __forceinline__ void add_limbs(uint32_t* limb, int stride, unsigned l
 }
 
 // ------------------------------------------------------------ transforms
-// The deltas are real, so planes z = 2m and 2m + 1 go through x and y as the real and
-// the imaginary part of one plane: half the points.  The z pass takes them apart again.
-// x; clears the sums that the z pass adds to
-template <int N1, int N2>
-__global__ void __launch_bounds__(kPassWidth) k_pk_x(const float* delta, float2* mesh,
-                                                     int nbins, double* bins,
-                                                     const uint32_t* err,
-                                                     const float2* __restrict__ tw, int twsh) {
+// Complex passes over the real deltas, every mode beside its mirror image: their roundings
+// are different ones, and a shell's mean takes both.  Two real planes as one complex
+// plane through x and y, or half the spectrum, cost half the points (256^3 particles on 512^3
+// points 1.36 ms and not 1.93) but give one of the two, and P(k) was up to sqrt(2) further off 64 bits
+// (512^3 points on fresh initial conditions 9.4e-7 against 6.6e-7, median).
+// x, from real deltas or in place; clears the sums that the z pass adds to
+template <int N1, int N2, bool REAL>
+__global__ void __launch_bounds__(kPassWidth) k_pk_x(const float* delta, float2* mesh, int nbins, double* bins,
+                                                     const uint32_t* err, const float2* __restrict__ tw, int twsh) {
     chain_begin();
     using Q = Pass<N1, N2>;
     extern __shared__ __align__(16) unsigned char pass_smem[];
@@ -344,12 +345,11 @@ __global__ void __launch_bounds__(kPassWidth) k_pk_x(const float* delta, float2*
     const int64_t q0 = (int64_t)blockIdx.x * Q::P;
     for (int it = threadIdx.x; it < Q::P * N2; it += kPassWidth) {
         const int p = it >> Q::L2, n2 = it & (N2 - 1);
-        const int64_t m = q0 >> Q::LN, plane = 1ll << (2 * Q::LN);
-        const float* src = delta + m * plane + ((q0 + p) << Q::LN) + n2;   // row q - m n of plane 2 m
+        const int64_t i = ((q0 + p) << Q::LN) + n2;
         float2 a[N1];
 #pragma unroll
         for (int n1 = 0; n1 < N1; ++n1)
-            a[bitrev<Q::L1>(n1)] = make_float2(src[N2 * n1], src[plane + N2 * n1]);
+            a[bitrev<Q::L1>(n1)] = REAL ? make_float2(delta[i + N2 * n1], 0.f) : mesh[i + N2 * n1];
         pass_first<N1, N2>(a, Y, p, n2, tw, twsh);
     }
     __syncthreads();
@@ -403,10 +403,6 @@ __device__ __forceinline__ float block_max(float v, float* sh) {
 // P pencils (one ky, P neighbouring kx) in turn and keep their shells in double
 // precision, one owner thread each.  A shell takes at most 2 sqrt(2 j) + 1 modes of a
 // pencil, so a limb's 2048 hold a group at every size.
-// Of the packed planes' spectra C, twice the even planes' is C(kx, ky) +
-// conj C(-kx, -ky) and twice the odd ones' -i times the difference: a pencil's input.  A
-// mode's square is that of its mirror image, so rows 0 < ky < n/2 count twice and those
-// past n/2 are left out.
 template <int N1, int N2>
 __global__ void __launch_bounds__(kPassWidth) k_pk_z(int nbins, double norm, double kf,
                                                      const float2* mesh,
@@ -416,7 +412,7 @@ __global__ void __launch_bounds__(kPassWidth) k_pk_z(int nbins, double norm, dou
     using Q = Pass<N1, N2>;
     constexpr int64_t plane = (int64_t)Q::n * Q::n;
     constexpr int h = Q::n / 2, kItems = (Q::P * N1 + kPassWidth - 1) / kPassWidth;
-    constexpr int kGroups = (h + 1) * (Q::n / Q::P);
+    constexpr int kGroups = (int)(plane / Q::P);
     extern __shared__ __align__(16) unsigned char pass_smem[];
     double* acc = reinterpret_cast<double*>(pass_smem);
     uint32_t* limb = reinterpret_cast<uint32_t*>(acc + h + 1);
@@ -430,24 +426,15 @@ __global__ void __launch_bounds__(kPassWidth) k_pk_z(int nbins, double norm, dou
     }
     for (int g = blockIdx.x; g < kGroups; g += gridDim.x) {
         const int64_t q0 = (int64_t)g * Q::P;
-        const int ky = (int)(q0 >> Q::LN), kx0 = (int)(q0 & (Q::n - 1));
+        const int ky = (int)(q0 >> Q::LN), kx0 = (int)(q0 & (Q::n - 1)), ny = ky < h ? ky : ky - Q::n;
         for (int it = tid; it < Q::P * N2; it += kPassWidth) {
-            const int p = it & (Q::P - 1), n2 = it >> Q::LP, kx = kx0 + p;
-            const float2* at = mesh + (n2 >> 1) * plane;
-            const float2* c = at + q0 + p;
-            const float2* mirror = at + ((((Q::n - ky) & (Q::n - 1)) << Q::LN) + ((Q::n - kx) & (Q::n - 1)));
-            const float sg = (n2 & 1) ? -1.f : 1.f;
+            const int p = it & (Q::P - 1), n2 = it >> Q::LP;
             float2 a[N1];
 #pragma unroll
-            for (int n1 = 0; n1 < N1; ++n1) {
-                const float2 u = c[(N2 / 2 * n1) * plane], w = mirror[(N2 / 2 * n1) * plane];
-                const float x = __fmaf_rn(sg, w.x, u.x), y = __fmaf_rn(-sg, w.y, u.y);
-                a[bitrev<Q::L1>(n1)] = (n2 & 1) ? make_float2(y, -x) : make_float2(x, y);
-            }
+            for (int n1 = 0; n1 < N1; ++n1) a[bitrev<Q::L1>(n1)] = mesh[q0 + p + (N2 * n1 + n2) * plane];
             pass_first<N1, N2>(a, Y, p, n2, tw, twsh);
         }
         __syncthreads();
-        const int twice = ky == 0 || ky == h ? 0 : 1;
         float2 a[kItems][N2];
         float big = 0.f;
 #pragma unroll
@@ -465,14 +452,13 @@ __global__ void __launch_bounds__(kPassWidth) k_pk_z(int nbins, double norm, dou
             const int it = tid + u * kPassWidth, p = it & (Q::P - 1), k1 = it >> Q::LP;
             if (it < Q::P * N1) {
                 const int kx = kx0 + p, nx = kx < h ? kx : kx - Q::n;
-                const int m0 = nx * nx + ky * ky;
+                const int m0 = nx * nx + ny * ny;
 #pragma unroll
                 for (int k2 = 0; k2 < N2; ++k2) {
                     const int kz = k1 + N1 * k2, nz = kz < h ? kz : kz - Q::n;
                     const int j = shell_of(m0 + nz * nz);
                     if (j >= 1 && j <= nbins)
-                        add_limbs(limb + j, h + 1,
-                                  (square_of<12>(a[u][k2].x, emax) + square_of<12>(a[u][k2].y, emax)) << twice);
+                        add_limbs(limb + j, h + 1, square_of<13>(a[u][k2].x, emax) + square_of<13>(a[u][k2].y, emax));
                 }
             }
         }
@@ -480,14 +466,14 @@ __global__ void __launch_bounds__(kPassWidth) k_pk_z(int nbins, double norm, dou
         for (int j = tid; j <= nbins; j += kPassWidth) {
             uint32_t* l = limb + j;
             if (l[0] | l[h + 1] | l[2 * (h + 1)]) {
-                acc[j] += limbs_value<12>(l[0], l[h + 1], l[2 * (h + 1)], emax);
+                acc[j] += limbs_value<13>(l[0], l[h + 1], l[2 * (h + 1)], emax);
                 l[0] = l[h + 1] = l[2 * (h + 1)] = 0u;
             }
         }
         // (the next group's writes to limb and mx come after its own barrier)
     }
     for (int j = tid; j <= nbins; j += kPassWidth)
-        if (j >= 1 && acc[j] != 0.0) atomicAdd(&bins[j - 1], 0.25 * norm * acc[j]);   // of twice the input
+        if (j >= 1 && acc[j] != 0.0) atomicAdd(&bins[j - 1], norm * acc[j]);
 }
 
 // Up to 16^3 points: transforms, shells and the mesh's own sums in one CTA.  Real
@@ -665,13 +651,14 @@ template <int N1, int N2>
 void launch_transforms(cudaStream_t stream, bool chained, int nbins, double norm, double kf, float2* mesh,
                        const float* delta, double* bins, const uint32_t* err, const float2* tw, int tw_n) {
     using Q = Pass<N1, N2>;
-    const unsigned groups = (unsigned)((int64_t)Q::n * Q::n / (2 * Q::P));
+    const unsigned groups = (unsigned)((int64_t)Q::n * Q::n / Q::P);
     const bool ahead = chained && (int64_t)Q::n * Q::n * Q::n <= kChainCells;
     int twsh = 0;
     while ((Q::n << twsh) < tw_n) ++twsh;
-    chain(ahead, k_pk_x<N1, N2>, groups, kPassWidth, Q::kBytes, stream, delta, mesh, nbins, bins, err, tw, twsh);
+    chain(ahead, delta ? k_pk_x<N1, N2, true> : k_pk_x<N1, N2, false>, groups, kPassWidth, Q::kBytes, stream, delta, mesh,
+          nbins, bins, err, tw, twsh);
     chain(ahead, k_pk_y<N1, N2>, groups, kPassWidth, Q::kBytes, stream, mesh, tw, twsh);
-    const unsigned gz = groups + Q::n / Q::P < 152 * 6 ? groups + Q::n / Q::P : 152 * 6;
+    const unsigned gz = groups < 152 * 6 ? groups : 152 * 6;
     chain(ahead, k_pk_z<N1, N2>, gz, kPassWidth, z_bytes<N1, N2>(), stream, nbins, norm, kf, mesh, bins, tw, twsh);
 }
 
@@ -686,7 +673,8 @@ template <int N1, int N2>
 void setup_transforms() {
     using Q = Pass<N1, N2>;
     const auto smem = cudaFuncAttributeMaxDynamicSharedMemorySize;
-    cudaFuncSetAttribute(k_pk_x<N1, N2>, smem, (int)Q::kBytes);
+    cudaFuncSetAttribute(k_pk_x<N1, N2, true>, smem, (int)Q::kBytes);
+    cudaFuncSetAttribute(k_pk_x<N1, N2, false>, smem, (int)Q::kBytes);
     cudaFuncSetAttribute(k_pk_y<N1, N2>, smem, (int)Q::kBytes);
     cudaFuncSetAttribute(k_pk_z<N1, N2>, smem, (int)z_bytes<N1, N2>());
 }
@@ -708,7 +696,7 @@ void pk_setup() {
 }
 
 cudaError_t pk_enqueue(cudaStream_t stream, const PkStore& st, int nmesh, int nbins, float2* mesh,
-                       double* bins, const uint32_t* err, const float2* tw, int tw_n, int64_t* launches) {
+                       float* delta, double* bins, const uint32_t* err, const float2* tw, int tw_n, int64_t* launches) {
     const int64_t m3 = (int64_t)nmesh * nmesh * nmesh;
     int lh = 0;
     while ((nmesh << lh) < 4 * st.nc) ++lh;
@@ -726,9 +714,8 @@ cudaError_t pk_enqueue(cudaStream_t stream, const PkStore& st, int nmesh, int nb
     }
     const double L = 4.0 * st.nc, norm = L * L * L / ((double)m3 * (double)m3), kf = 2.0 * kPi / L;
     const bool small = nmesh <= 16;
-    // the packed planes take the first half of `mesh`, the deltas the second
-    float* real = reinterpret_cast<float*>(small ? mesh : mesh + m3 / 2);
-    if (nmesh <= 1024) deposit(stream, st, lh, mean, real);
+    float* real = small ? reinterpret_cast<float*>(mesh) : (nmesh <= 1024 ? delta : nullptr);
+    if (real) deposit(stream, st, lh, mean, real);
     else deposit(stream, st, lh, mean, mesh);
     *launches += 1;
     if (small) {
@@ -763,10 +750,12 @@ int power_spectrum_enqueue(Sim& s, int nmesh, int nbins, double* host_bins, bool
     if (nbins < 1 || nbins > nmesh / 2)
         return set_error(s, PMPM_EINVAL, "nbins %d must be in [1, nmesh/2]", nbins);
     if (nmesh < s.nc) return set_error(s, PMPM_EINVAL, "nmesh below nf/4 is not supported");
+    const int64_t m3 = (int64_t)nmesh * nmesh * nmesh;
     float2* mesh = reinterpret_cast<float2*>(s.scratch);
+    float* delta = reinterpret_cast<float*>(align_up(reinterpret_cast<uintptr_t>(mesh + m3)));   // (16 pk_max^3 + 512 bytes)
     const PkStore st = {s.nc, s.pb, s.n, s.offsets[s.cur], s.counts[s.cur],
                         {m_stream(s, s.cur, 0), m_stream(s, s.cur, 1), m_stream(s, s.cur, 2)}, s.chained};
-    cudaError_t e = pk_enqueue(s.stream, st, nmesh, nbins, mesh, s.pk_bins, s.err, s.tw_f, s.fft_max, &s.launches);
+    cudaError_t e = pk_enqueue(s.stream, st, nmesh, nbins, mesh, delta, s.pk_bins, s.err, s.tw_f, s.fft_max, &s.launches);
     if (e == cudaSuccess)
         e = cudaMemcpyAsync(host_bins, s.pk_bins, sizeof(double) * (3 * nbins + word), cudaMemcpyDeviceToHost, s.stream);
     if (e != cudaSuccess) return set_error(s, PMPM_ECUDA, "power spectrum: %s", cudaGetErrorString(e));

@@ -18,10 +18,10 @@ struct PkStore {
 // Enqueues P(k) sums of `st` on an nmesh^3 mesh (a power of two from nc to 4 nc,
 // at least 8): bins[0..nbins) sum of P, then of |k|, then modes, per shell, then one
 // double more: *err as the stream finds it.
-// mesh: 8 nmesh^3 bytes.
+// mesh: 8 nmesh^3 bytes; delta: 4 nmesh^3 bytes more, or null (nmesh up to 1024).
 // tw: exp(-2 pi i k / tw_n), nmesh dividing tw_n.  launches: added to.
 cudaError_t pk_enqueue(cudaStream_t stream, const PkStore& st, int nmesh, int nbins, float2* mesh,
-                       double* bins, const uint32_t* err, const float2* tw, int tw_n, int64_t* launches);
+                       float* delta, double* bins, const uint32_t* err, const float2* tw, int tw_n, int64_t* launches);
 void pk_setup();
 
 // offsets[0..nc^3] of `counts` (sort.cu); sums: kScanSums words
