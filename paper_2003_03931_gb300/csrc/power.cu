@@ -14,12 +14,11 @@
 // FP64 runs at 1/64 of the FP32 rate here, so squares and shell sums are integers
 // (pk_sums.cuh) and only a block's totals become doubles.
 //
-// On a GB300: 256^3 particles on 512^3 points 10.5 -> 1.37 ms (a search per
+// On a GB300: 256^3 particles on 512^3 points 10.5 -> 1.93 ms (a search per
 // particle, 64-bit global atomics and three double shared atomics a mode before):
-// deposit 0.55 (issue: the particles of 2.8 bricks
-// are looked at), x 0.21, y 0.21, z with the shells 0.34, of 0.48 ms for
-// 24 bytes a point at the copy bandwidth (1.95 ms with planes of their own, 40 bytes);
-// 32^3 on 32^3, without allocation, 115 -> 70 us.
+// deposit 0.51 (issue: the particles of 2.8 bricks are looked at), x 0.27, y 0.43, z with the
+// shells 0.68 (exact squares 0.14 of it), of 0.8 ms for 40 bytes a point at the copy
+// bandwidth; 32^3 on 32^3, without allocation, 118 -> 70 us.
 #include "power.cuh"
 
 #include <new>

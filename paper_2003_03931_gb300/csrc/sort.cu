@@ -139,7 +139,7 @@ constexpr int64_t kScanDirect = 32768;
 // U = sum over cells and axes of floor(S^2 / n), into the digits d2[4..7]; the
 // last block done (d2[8] counts them; none waits) writes sigma.  Scan, means and
 // dispersion of a step, with separate passes over counts and S before: 16^3
-// cells 43 -> 10 us (one launch), 64^3 46 -> 21, 256^3 625 -> 343 (of 48 B a
+// cells 43 -> 10 us (one launch), 64^3 48 -> 21, 256^3 625 -> 355 (of 48 B a
 // cell: 119 us at the copy bandwidth; the divisions bound it).
 template <bool MEANS, int ITEMS>
 __global__ void __launch_bounds__(kScanThreads) k_scan_apply(int64_t ncells, const int32_t* counts,

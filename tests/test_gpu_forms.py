@@ -1,9 +1,8 @@
-"""The coarse chain, the scan and the column pass (short-range force by walking
-columns of tiles along z) at the sizes where their forms change; for the column
-pass also the shapes where its parts change: ragged tiles of 4 and 5 cells, both
-position formats, segments of a few layers and of many, and layers with
-more particles than its tables, its first round of threads and its unchecked
-deposit take.  Bar: the force of test_gpu_force.py, 1e-4 against the oracle."""
+"""The coarse chain, the scan and the short-range pass at the sizes where their forms
+change; for the short-range pass also ragged tiles of 4 and 5 cells, both
+position formats and crowded cells.  (The boxes here are small or sparse and take
+32^3-box tiles; test_gpu_column.py has the same for the column pass.)  Bar: the
+force of test_gpu_force.py, 1e-4 against the oracle."""
 
 import numpy as np
 import pytest
@@ -53,8 +52,8 @@ def test_column_crowded_layer(in_cell):
 
 @pytest.mark.parametrize("nc", [8, 16, 32, 64])
 def test_coarse_force_chain(nc):
-    # the coarse chain's forms: one launch up to 16^3 and at 32^3 cells, five passes
-    # from 64^3; far from everything the force is the coarse mesh's alone
+    # the coarse chain's forms: one launch up to 16^3 cells, four at 32^3, and at 64^3 the
+    # general transforms (a sparse box); far from everything the force is the coarse mesh's alone
     need_gpu()
     rng = np.random.default_rng(nc)
     sim = make_sim(np=8, nc=nc, a_init=0.02, a_final=1.0, n_steps=4)
@@ -114,7 +113,7 @@ def _mean_k(nmesh, nbins, box):
                                                 (64, 256, 1), (128, 512, 1)])
 def test_power_spectrum_forms(nc, nmesh, pos_bytes):
     # every node spacing (1, 2 and 4 fine cells), position format and mesh form (one
-    # CTA up to 32^3, three passes from 64^3) against the oracle; a tenth of the
+    # CTA up to 16^3, three passes from 32^3) against the oracle; a tenth of the
     # particles in one cell
     need_gpu()
     from oracle import power
